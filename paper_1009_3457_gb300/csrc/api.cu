@@ -203,14 +203,6 @@ int fgt_workspace(size_t bytes, float** out)
     return FMM_OK;
 }
 
-double m2l_balance(int p)
-{
-    // s = 2e / (2p - 2) balances j! s^j |D|^-(j+1) (|D| >= 2) against
-    // 1 / (n! s^n) over the index ranges j <= 2p-2, n <= p-1.
-    const double jmax = (p > 1) ? 2.0 * p - 2.0 : 1.0;
-    return 2.0 * 2.718281828459045 / jmax;
-}
-
 int get_m2l_tables(int p, const M2LTables** out)
 {
     std::lock_guard<std::mutex> lk(g_mu);
@@ -228,13 +220,9 @@ int get_m2l_tables(int p, const M2LTables** out)
     const size_t nh = (size_t)kOffsetSlots * (2 * p - 1);
     cudaError_t e;
     if ((e = cudaMalloc(&t->h_fwd, nh * sizeof(float2))) != cudaSuccess ||
-        (e = cudaMalloc(&t->h_adj, nh * sizeof(float2))) != cudaSuccess ||
-        (e = cudaMalloc(&t->h_adjc, nh * sizeof(float2))) != cudaSuccess ||
         (e = cudaMalloc(&t->a, p * sizeof(float))) != cudaSuccess ||
         (e = cudaMalloc(&t->b, p * sizeof(float))) != cudaSuccess) {
         cudaFree(t->h_fwd);
-        cudaFree(t->h_adj);
-        cudaFree(t->h_adjc);
         cudaFree(t->a);
         cudaFree(t->b);
         delete t;
@@ -685,8 +673,8 @@ static int m2l_dispatch(const char* who, const fmm_tree* tree, int32_t lmin, int
         d.tc_ntiles = tc_ntiles;
     }
     if (job.nlev == 0) return FMM_OK;
-    // The adjoint is the forward stencil with the table of -a(D) (plain) or
-    // -conj a(D) (FMM_CONJ): a(D)^T = -a(-D) on symmetric lists.
+    // The adjoint is the forward stencil of -a(D) (plain) or -conj a(D) (FMM_CONJ):
+    // a(D)^T = -a(-D) on symmetric lists.
     if (prec != FMM_FP32) {
         const int variant = !adjoint ? 0 : ((flags & FMM_CONJ) ? 2 : 1);
         const void* img = nullptr;
@@ -694,8 +682,9 @@ static int m2l_dispatch(const char* who, const fmm_tree* tree, int32_t lmin, int
         if ((rc = get_tc_image(p, variant, tf32, &img))) return rc;
         return launch_m2l_tc(job, p, img, prec != FMM_TC_BF16, tf32, st);
     }
-    const float2* h = !adjoint ? t->h_fwd : ((flags & FMM_CONJ) ? t->h_adjc : t->h_adj);
-    return launch_m2l_fp32(job, p, h, t->a, t->b, st);
+    job.sgn = adjoint ? -1.f : 1.f;
+    job.cj = adjoint && (flags & FMM_CONJ) ? -1.f : 1.f;
+    return launch_m2l_fp32(job, p, *t, st);
 }
 
 static int levels_common(const char* who, const fmm_tree* tree, int32_t lmin, int32_t lmax, int32_t p, int32_t prec,

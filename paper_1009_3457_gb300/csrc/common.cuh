@@ -143,12 +143,11 @@ void class_stencil(int cls, StencilEntry out[27]);
 // a Hankel matrix between two diagonal scalings.  The balance factor s keeps
 // every factor well inside FP32 range for p <= 32.
 // ---------------------------------------------------------------------------
+constexpr int kM2LOrbits = 7;  // offset orbits (2,0), (2,2), (2,1), (3,0), (3,1), (3,2), (3,3)
 struct M2LTables {
     int p = 0;
     double s = 0.0;
-    float2* h_fwd = nullptr;   // [49][2p-1] complex: forward M2L
-    float2* h_adj = nullptr;   // [49][2p-1]: plain adjoint  (= -h_fwd)
-    float2* h_adjc = nullptr;  // [49][2p-1]: conjugate adjoint (= -conj h_fwd)
+    float2* h_fwd = nullptr;   // [49][2p-1] complex, per offset (the paper's data flow)
     float* a = nullptr;        // [p] post-scale
     float* b = nullptr;        // [p] pre-scale
     // dense scaled operators for the tensor-core path, built on demand:
@@ -158,7 +157,9 @@ struct M2LTables {
     int tc_ready[2][3] = {{0, 0, 0}, {0, 0, 0}};
 };
 int get_m2l_tables(int p, const M2LTables** out);
-double m2l_balance(int p);
+// s = 2e / (2p - 2) balances j! s^j |D|^-(j+1) (|D| >= 2) against 1 / (n! s^n) over the index
+// ranges j <= 2p-2, n <= p-1.
+constexpr double m2l_balance(int p) { return 2.0 * 2.718281828459045 / (p > 1 ? 2.0 * p - 2.0 : 1.0); }
 
 // One launch of the M2L stencil over several uniform levels (kernel parameter).
 struct M2LLevel {
@@ -178,6 +179,8 @@ struct M2LLaunch {
     int nlev;
     int periodic;
     int accumulate;
+    // FP32 adjoints: L = sgn * K(M) with sgn = -1, and with cj = -1 conj(K(conj M))
+    float sgn, cj;
 };
 
 // tree handle accessors (api.cu)
@@ -193,7 +196,7 @@ int tree_device_tc_tiles(const fmm_tree* t, int level, const int32_t** tiles, in
 // launchers (m2l_fp32.cu)
 int launch_build_m2l_tables(const M2LTables& t, cudaStream_t st);
 bool m2l_fp32_supported(int p);
-int launch_m2l_fp32(M2LLaunch& job, int p, const float2* hsel, const float* a, const float* b, cudaStream_t st);
+int launch_m2l_fp32(M2LLaunch& job, int p, const M2LTables& t, cudaStream_t st);
 
 // launchers (m2l_tc.cu)
 bool m2l_tc_supported(int p);

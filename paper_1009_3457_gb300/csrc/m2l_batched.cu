@@ -8,7 +8,7 @@
 // per plan.  Each resident CTA takes its first chunk of items by blockIdx and
 // then claims further chunks from a work counter, so a greedy
 // longest-processing-time schedule balances problems whose sizes differ by
-// four orders of magnitude.  A CTA keeps the operator tables of its current p
+// four orders of magnitude.  A CTA keeps the diagonal scalings of its current p
 // in shared memory and reloads them only when the p of its next item differs
 // (items are grouped by p, so that happens a few times per CTA).
 //
@@ -16,9 +16,8 @@
 // instantiated CUDA graph of the two, and a caller's stream capture records
 // them as they are.  The autotuner times, on the plan itself with every output
 // pointer redirected to library scratch, first the grid sizes (resident CTAs
-// per SM) and claim chunks, then the work-unit variants (how a warp's lanes
-// share a target's rows and list entries, and the halo loads a thread keeps in
-// flight) at the best of those; the choice is cached per GPU and workload
+// per SM) and claim chunks, then the work-unit variants (the halo loads a thread
+// keeps in flight) at the best of those; the choice is cached per GPU and workload
 // signature in memory and in a JSON file that later processes reload.
 #include "m2l_fp32_tile.cuh"
 
@@ -49,7 +48,6 @@ struct BatchDesc {
 // Operator tables per batched order, indexed by batch_p_index(p).
 constexpr int kBatchOrders = 4;
 struct BatchTables {
-    const float2* h[kBatchOrders];
     const float* a[kBatchOrders];
     const float* b[kBatchOrders];
 };
@@ -65,21 +63,18 @@ static inline int batch_p_index(int p)
     }
 }
 
-constexpr size_t kBatchSmem = M2LCfg<16>::smem;  // the largest batched order
-constexpr int kBatchMinCtas = 6;
+constexpr int kBatchThreads = 64;  // one warp per 32 targets: a batch has many tiles per SM
+constexpr size_t kBatchSmem = M2LCfg<16, kBatchThreads>::smem;  // the largest batched order
+constexpr int kBatchMinCtas = M2LCfg<16, kBatchThreads>::MIN_CTAS;
 
-// Work-unit variants the autotuner chooses between: the lane form of the work unit
-// (m2l_fp32_tile.cuh) and the halo loads a thread keeps in flight while staging (the
-// one kernel holds every order's code, so its register budget is the largest order's).
-struct BatchVariant {
-    int form, loads;
-};
-constexpr BatchVariant kBatchVariants[] = {
-    {kFormAuto, 3}, {kFormRowsPacked, 3}, {kFormRowsPacked, 2}, {kFormEntries, 3}, {kFormRows, 3}};
-constexpr int kBatchNumVariants = 5;
+// Work-unit variants the autotuner chooses between: the halo loads a thread keeps in
+// flight while staging (the one kernel holds every order's code, so its register budget
+// is the largest order's).  The work unit has one lane form, reported as form -1.
+constexpr int kBatchLoads[] = {3, 2};
+constexpr int kBatchNumVariants = 2;
 
-template <int FORM, int LOADS>
-__global__ void __launch_bounds__(kThreads, kBatchMinCtas)
+template <int LOADS>
+__global__ void __launch_bounds__(kBatchThreads, kBatchMinCtas)
     m2l_batched_kernel(const BatchDesc* __restrict__ desc, const int2* __restrict__ items, int nitems,
                        int* __restrict__ counter, int chunk, int accumulate, BatchTables tabs)
 {
@@ -95,20 +90,20 @@ __global__ void __launch_bounds__(kThreads, kBatchMinCtas)
             if (d.p != cur_p) {
                 __syncthreads();  // no thread still reads the previous operator
                 switch (d.p) {
-                    case 6: m2l_load_operator<6>(smem_raw, tabs.h[0], tabs.a[0], tabs.b[0]); break;
-                    case 8: m2l_load_operator<8>(smem_raw, tabs.h[1], tabs.a[1], tabs.b[1]); break;
-                    case 12: m2l_load_operator<12>(smem_raw, tabs.h[2], tabs.a[2], tabs.b[2]); break;
-                    default: m2l_load_operator<16>(smem_raw, tabs.h[3], tabs.a[3], tabs.b[3]); break;
+                    case 6: m2l_load_operator<6, kBatchThreads>(smem_raw, tabs.a[0], tabs.b[0]); break;
+                    case 8: m2l_load_operator<8, kBatchThreads>(smem_raw, tabs.a[1], tabs.b[1]); break;
+                    case 12: m2l_load_operator<12, kBatchThreads>(smem_raw, tabs.a[2], tabs.b[2]); break;
+                    default: m2l_load_operator<16, kBatchThreads>(smem_raw, tabs.a[3], tabs.b[3]); break;
                 }
                 cur_p = d.p;
             }
             const TileGeom g = tile_geom_of(d.M, d.L, nullptr, d.level, item.y);
             __syncthreads();  // operator visible; previous tile done with the halo buffer
             switch (d.p) {
-                case 6: m2l_tile<6, false, LOADS, FORM>(smem_raw, g, d.periodic, accumulate); break;
-                case 8: m2l_tile<8, false, LOADS, FORM>(smem_raw, g, d.periodic, accumulate); break;
-                case 12: m2l_tile<12, false, LOADS, FORM>(smem_raw, g, d.periodic, accumulate); break;
-                default: m2l_tile<16, false, LOADS, FORM>(smem_raw, g, d.periodic, accumulate); break;
+                case 6: m2l_tile<6, kBatchThreads, false, LOADS>(smem_raw, g, d.periodic, accumulate); break;
+                case 8: m2l_tile<8, kBatchThreads, false, LOADS>(smem_raw, g, d.periodic, accumulate); break;
+                case 12: m2l_tile<12, kBatchThreads, false, LOADS>(smem_raw, g, d.periodic, accumulate); break;
+                default: m2l_tile<16, kBatchThreads, false, LOADS>(smem_raw, g, d.periodic, accumulate); break;
             }
         }
         if (!counter) break;  // one chunk per CTA (grid covers every item)
@@ -123,13 +118,7 @@ __global__ void __launch_bounds__(kThreads, kBatchMinCtas)
 // the kernel of variant v (kBatchVariants order)
 static const void* batch_kernel(int v)
 {
-    switch (v) {
-        case 1: return (const void*)m2l_batched_kernel<kFormRowsPacked, 3>;
-        case 2: return (const void*)m2l_batched_kernel<kFormRowsPacked, 2>;
-        case 3: return (const void*)m2l_batched_kernel<kFormEntries, 3>;
-        case 4: return (const void*)m2l_batched_kernel<kFormRows, 3>;
-        default: return (const void*)m2l_batched_kernel<kFormAuto, 3>;
-    }
+    return v == 1 ? (const void*)m2l_batched_kernel<2> : (const void*)m2l_batched_kernel<3>;
 }
 
 }  // namespace fmmgb
@@ -228,13 +217,13 @@ int tune_key(const fmm_batch* b, std::string* key)
     std::string name = prop.name;
     for (char& ch : name)
         if (ch == '"' || ch == '|' || ch == '\\') ch = '_';
-    *key = name + "|" + std::to_string(prop.multiProcessorCount) + "|fp32|" + b->signature;
+    *key = name + "|" + std::to_string(prop.multiProcessorCount) + "|fp32|fold;" + b->signature;  // "fold": choices timed on an earlier work unit do not match
     return FMM_OK;
 }
 
 int batch_occupancy(int v, int* occ)
 {
-    FMM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, batch_kernel(v), kThreads, kBatchSmem));
+    FMM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, batch_kernel(v), kBatchThreads, kBatchSmem));
     if (*occ < 1) return fail(FMM_ECUDA, "batched M2L: kernel variant %d cannot be resident (occupancy 0)", v);
     return FMM_OK;
 }
@@ -249,7 +238,7 @@ int launch_batch(const fmm_batch* b, const BatchDesc* desc, int grid, int chunk,
     int acc = b->accumulate;
     BatchTables tabs = b->tabs;
     void* args[] = {(void*)&desc, (void*)&items, (void*)&nitems, (void*)&ctr, (void*)&chunk, (void*)&acc, (void*)&tabs};
-    FMM_CUDA_TRY(cudaLaunchKernel(batch_kernel(variant), dim3((unsigned)grid), dim3(kThreads), args, kBatchSmem, st));
+    FMM_CUDA_TRY(cudaLaunchKernel(batch_kernel(variant), dim3((unsigned)grid), dim3(kBatchThreads), args, kBatchSmem, st));
     return FMM_OK;
 }
 
@@ -277,7 +266,7 @@ int build_graph(fmm_batch* b)
         cudaKernelNodeParams kp{};
         kp.func = const_cast<void*>(batch_kernel(b->variant));
         kp.gridDim = dim3((unsigned)b->grid);
-        kp.blockDim = dim3(kThreads);
+        kp.blockDim = dim3(kBatchThreads);
         kp.sharedMemBytes = (unsigned)kBatchSmem;
         kp.kernelParams = args;
         e = cudaGraphAddKernelNode(&nker, g, &nset, 1, &kp);
@@ -485,7 +474,6 @@ int create_batch(const fmm_tree* const* trees, const int32_t* p, int32_t nprob, 
         int rc = get_m2l_tables(pv, &t);
         if (rc) { delete b; return rc; }
         const int j = batch_p_index(pv);
-        b->tabs.h[j] = t->h_fwd;
         b->tabs.a[j] = t->a;
         b->tabs.b[j] = t->b;
     }
@@ -566,8 +554,8 @@ int fmm_batch_info(const fmm_batch* b, fmm_batch_info_t* out)
     out->tuned = b->tuned;
     out->tuned_ms = b->tuned_ms;
     out->variant = b->variant;
-    out->form = kBatchVariants[b->variant].form;
-    out->loads = kBatchVariants[b->variant].loads;
+    out->form = -1;
+    out->loads = kBatchLoads[b->variant];
     out->from_cache = b->from_cache;
     return FMM_OK;
 }

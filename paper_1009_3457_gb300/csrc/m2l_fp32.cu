@@ -3,7 +3,7 @@
 // plus the FP64 operator-table builder.
 //
 // The work unit (a 4 x 4 tile of parent boxes, the Hankel factorisation of the
-// operator and the class-split shared-memory halo) and the stencil kernel are
+// operator, the offsets folded by symmetry) and the stencil kernel are
 // in m2l_fp32_tile.cuh; this file holds the operator-table builder and the
 // launcher.
 #include "m2l_fp32_tile.cuh"
@@ -13,8 +13,7 @@ namespace fmmgb {
 // ---------------------------------------------------------------------------
 // operator tables, computed in FP64 on the GPU, stored as FP32
 // ---------------------------------------------------------------------------
-__global__ void build_m2l_tables_kernel(int p, double s, float2* __restrict__ hf, float2* __restrict__ ha,
-                                        float2* __restrict__ hac, float* __restrict__ a, float* __restrict__ b)
+__global__ void build_m2l_tables_kernel(int p, double s, float2* __restrict__ hf, float* __restrict__ a, float* __restrict__ b)
 {
     const int nh = 2 * p - 1;
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
@@ -39,8 +38,6 @@ __global__ void build_m2l_tables_kernel(int p, double s, float2* __restrict__ hf
             v = make_float2((float)hr, (float)hi);
         }
         hf[idx] = v;
-        ha[idx] = make_float2(-v.x, -v.y);
-        hac[idx] = make_float2(-v.x, v.y);
     }
     if (idx < p) {
         double fact = 1.0, sp = 1.0;
@@ -56,7 +53,7 @@ __global__ void build_m2l_tables_kernel(int p, double s, float2* __restrict__ hf
 int launch_build_m2l_tables(const M2LTables& t, cudaStream_t st)
 {
     const int n = kOffsetSlots * (2 * t.p - 1);
-    build_m2l_tables_kernel<<<(n + 127) / 128, 128, 0, st>>>(t.p, t.s, t.h_fwd, t.h_adj, t.h_adjc, t.a, t.b);
+    build_m2l_tables_kernel<<<(n + 127) / 128, 128, 0, st>>>(t.p, t.s, t.h_fwd, t.a, t.b);
     FMM_CUDA_TRY(cudaGetLastError());
     return FMM_OK;
 }
@@ -64,7 +61,7 @@ int launch_build_m2l_tables(const M2LTables& t, cudaStream_t st)
 bool m2l_fp32_supported(int p) { return p == 6 || p == 8 || p == 12 || p == 16 || p == 24; }
 
 template <int P>
-static int launch_p(M2LLaunch& job, const float2* h, const float* a, const float* b, cudaStream_t st)
+static int launch_p(M2LLaunch& job, const M2LTables& t, cudaStream_t st)
 {
     using C = M2LCfg<P>;
     int total = 0;
@@ -84,7 +81,7 @@ static int launch_p(M2LLaunch& job, const float2* h, const float* a, const float
     if ((rc = smem_opt_in((const void*)kern, (int)C::smem, &opted[adaptive]))) return rc;
     static int occ_cache[2];  // resident CTAs per SM (same on every device of one model)
     if (!(occ = __atomic_load_n(&occ_cache[adaptive], __ATOMIC_ACQUIRE))) {
-        FMM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kThreads, C::smem));
+        FMM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, C::THREADS, C::smem));
         __atomic_store_n(&occ_cache[adaptive], occ, __ATOMIC_RELEASE);
     }
     int grid = total, *counter = nullptr;
@@ -92,19 +89,19 @@ static int launch_p(M2LLaunch& job, const float2* h, const float* a, const float
         grid = occ * sms;
         if ((rc = tile_counter(&counter, st))) return rc;
     }
-    kern<<<grid, kThreads, C::smem, st>>>(job, h, a, b, total, counter);
+    kern<<<grid, C::THREADS, C::smem, st>>>(job, t.a, t.b, total, counter);
     FMM_CUDA_TRY(cudaGetLastError());
     return FMM_OK;
 }
 
-int launch_m2l_fp32(M2LLaunch& job, int p, const float2* h, const float* a, const float* b, cudaStream_t st)
+int launch_m2l_fp32(M2LLaunch& job, int p, const M2LTables& t, cudaStream_t st)
 {
     switch (p) {
-        case 6: return launch_p<6>(job, h, a, b, st);
-        case 8: return launch_p<8>(job, h, a, b, st);
-        case 12: return launch_p<12>(job, h, a, b, st);
-        case 16: return launch_p<16>(job, h, a, b, st);
-        case 24: return launch_p<24>(job, h, a, b, st);
+        case 6: return launch_p<6>(job, t, st);
+        case 8: return launch_p<8>(job, t, st);
+        case 12: return launch_p<12>(job, t, st);
+        case 16: return launch_p<16>(job, t, st);
+        case 24: return launch_p<24>(job, t, st);
         default: return fail(FMM_EINVAL, "M2L FP32: unsupported p = %d", p);
     }
 }

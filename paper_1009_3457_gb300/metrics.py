@@ -9,6 +9,10 @@ m2l_flops_per_translation(p): real floating-point operations of one complex
 p x p matrix-vector product (p^2 complex multiply-adds, 8 flops each) --
 the algorithmic work of one translation by Eq. (M2Lmat).
 
+m2l_fp32_flops_per_box(p): real floating-point operations the FP32 kernel runs per
+target box (its 27 offsets folded by symmetry: 20 p^2 multiply-adds and about
+158 p additions, whether or not an entry lies inside the domain).
+
 m2l_bytes_per_box(p, elem): algorithmic HBM traffic of one box of one level:
 read its ME once and write its LE once (2 p complex values).
 """
@@ -20,6 +24,10 @@ def paper_ops_per_translation(p: int) -> int:
 
 def m2l_flops_per_translation(p: int) -> int:
     return 8 * p * p
+
+
+def m2l_fp32_flops_per_box(p: int) -> int:
+    return 40 * p * p + 158 * p
 
 
 def m2l_bytes_per_box(p: int, elem_bytes: int = 4) -> int:

@@ -357,3 +357,45 @@ def test_host_stream_pipeline_matches_direct_calls(fmm, orc):
     for out, fo, ref in zip(host_out, flat_out, refs):
         for a, f, b in zip(out, pipe.level_views(fo), ref):
             assert torch.equal(a, b) and torch.equal(f, b)
+
+
+@pytest.mark.parametrize("p", [6, 8, 12, 16, 24])
+def test_m2l_single_sources_reach_their_lists_only(fmm, p):
+    """One non-zero source box at a time (every child class, inside the domain, at a corner and
+    at an edge, tiles with and without a neighbour), forward and conjugate adjoint: each target
+    of its lists holds T(D) m to the FP32 rounding of a p-term sum, every other box exactly 0.
+    The 27 offsets are folded by symmetry in the kernel, so each offset is checked apart."""
+    import math
+    import torch
+
+    level, side = 4, 16
+    tree = fmm.fmm_build_lists(None, level)
+    lst, _ = tree.lists(level)
+    rng = np.random.default_rng(p)
+    nk = np.arange(p)
+    binom = np.array([[math.comb(n + k, k) for k in range(p)] for n in range(p)], dtype=np.float64)
+    for sx, sy in [(7, 6), (8, 9), (5, 8), (10, 11), (0, 0), (15, 3), (2, 15)]:
+        m = (rng.standard_normal(p) + 1j * rng.standard_normal(p)).astype(np.complex64)
+        src = sy * side + sx
+        M = np.zeros((side * side, p), np.complex64)
+        M[src] = m
+        for adjoint in (False, True):
+            Md, out = _dev(M), torch.full((side * side, p), float("nan"), dtype=torch.complex64, device="cuda")
+            if adjoint:
+                fmm.fmm_m2l_adjoint(tree, level, p, Md, out, conj=True)
+            else:
+                fmm.fmm_m2l(tree, level, p, Md, out)
+            fmm.fmm_sync_status()
+            got = _host(out)
+            for t in range(side * side):
+                if src not in lst[t]:
+                    assert (got[t] == 0).all(), (sx, sy, t, adjoint)
+                    continue
+                d = complex(t % side - sx, t // side - sy)  # target - source (symmetric lists: adjoint of -d)
+                D = -d if adjoint else d
+                T = (-1.0) ** nk[:, None] * binom * D ** -(nk[:, None] + nk[None, :] + 1.0)
+                T = T.conj().T if adjoint else T
+                # p products and sums, two roundings of each scaling and of the operator's value, and the
+                # folded combinations' few additions, on both parts: (2 p + 24) units of 2^-24
+                bound = (2 * p + 24) * 2.0 ** -24 * (np.abs(T) @ np.abs(m))
+                assert (np.abs(got[t] - T @ m) <= bound).all(), (sx, sy, t, adjoint)
