@@ -58,7 +58,7 @@ typedef enum {
 } fmm_status;
 
 typedef enum {
-    FMM_FP32 = 0,           /* FP32 FFMA path (Hankel-structured stencil kernel) */
+    FMM_FP32 = 0,           /* FP32 FFMA path (Hankel stencil kernel, offsets folded by symmetry) */
     FMM_TC_BF16X3 = 1,      /* tcgen05 tensor cores, BF16 hi/lo split, 3 products, FP32 accumulate */
     FMM_TC_BF16 = 2,        /* tcgen05 tensor cores, plain BF16 inputs, FP32 accumulate */
     FMM_TC_TF32X3 = 3       /* tcgen05 tensor cores, TF32 hi/lo split, 3 products, FP32 accumulate (M2L, p = 16) */
@@ -305,9 +305,8 @@ void fmm_host_stream_destroy(fmm_host_stream* hs);
  *   prec      FMM_FP32 (the only precision of the batched path).
  *   flags     FMM_ACCUMULATE (add into L), FMM_BATCH_AUTOTUNE (time the
  *             candidate launch configurations -- grid size, claim chunk -- and
- *             then the work-unit variants -- rows per lane, packed or scalar
- *             multiply-adds, halo loads in flight -- on this plan before
- *             returning, writing only library scratch, never L).  The choice
+ *             then the work-unit variants -- halo loads in flight -- on this
+ *             plan before returning, writing only library scratch, never L).  The choice
  *             is cached per GPU (name, SM count), precision and workload
  *             signature (p, level, periodicity and count of every (problem,
  *             level), accumulate) in memory and in a JSON file that later
@@ -342,10 +341,7 @@ typedef struct {
     int32_t tuned;         /* 1: configuration chosen by timing (FMM_BATCH_AUTOTUNE) */
     float tuned_ms;        /* best timed run of the autotuner, 0 if not tuned */
     int32_t variant;       /* work-unit variant: index into the tuned set */
-    int32_t form;          /* -1: each order's default (p/2 rows per lane, packed multiply-adds, the
-                              sums of w Re m and w Im m apart at p = 12, 16); 0: p/2 rows per lane,
-                              packed multiply-adds; 1: p rows per lane, half the list entries each;
-                              2: p/2 rows per lane, scalar multiply-adds */
+    int32_t form;          /* -1: the work unit's one lane form (a target per lane, all p rows) */
     int32_t loads;         /* halo loads a thread keeps in flight while staging a tile */
     int32_t from_cache;    /* 1: the tuned choice was reused (memory or cache file), not timed */
 } fmm_batch_info_t;
@@ -577,6 +573,14 @@ int fgt_t2p_binned(int32_t grid_log2, int32_t p, double sigma, const float* C, c
  *   aligned; y: device float64 [n][2]; perm, box_start: fgt_bin_points(grid_log2,
  *   y, n, ...) of these targets; G: device float32 [n], indexed like y.
  *   n_cut 0..16, p 4, 8, 12 or 16, flags FMM_ACCUMULATE or 0.
+ *   With two targets per box or more on average, grid_log2 <= 8 and a box side d =
+ *   2^-g / (sqrt2 sigma) of up to 1.3 (p = 16; more below), every prec is served in FP32 on
+ *   the CUDA cores through Chebyshev coefficients of each target box (12 or 16 per
+ *   dimension, interpolation error below 3e-8 of a Hermite function's size): the sums over
+ *   source boxes are taken once per target box.  Their workspace, 2 KiB per box, is allocated
+ *   per grid size and device on the first such call and kept; a first such call inside a
+ *   stream capture takes the direct sums below instead, as every other call does.  Calls that
+ *   overlap on the GPU share the workspace and must be serialised by the caller.
  *   prec FMM_FP32: CUDA cores.  Source boxes whose coefficients are all zero
  *   are skipped: a first kernel writes one flag per box.  The targets are
  *   taken in runs of up to 256 of one box, the boxes with the most non-empty
@@ -631,8 +635,8 @@ int fgt_h2p(int32_t grid_log2, int32_t n_cut, int32_t p, int32_t prec, double si
  *   FP32 arithmetic on positions taken relative to the target box's centre;
  *   1e-30 is added to every squared distance, so a source at exactly a
  *   target's position (e.g. the points themselves) contributes nothing
- *   (strengths |c| < 3e8) and other pairs change by a relative 1e-30 / r^2.  Uses the per-device scratch of
- *   fgt_h2p (calls that overlap on the GPU must be serialised).  A
+ *   (strengths |c| < 3e8) and other pairs change by a relative 1e-30 / r^2.  Uses a
+ *   per-device buffer grown on demand (calls that overlap on the GPU must be serialised).  A
  *   permutation entry outside range or inconsistent box starts set the device
  *   error word's check bit; the affected pairs are skipped.
  * ------------------------------------------------------------------------- */

@@ -1,0 +1,406 @@
+// fgt_cheb.cu -- the FGT's Hermite evaluation (Sec. 4.2, Eq. hermite) with the sums over
+// source boxes taken once per target box instead of once per target.
+//
+// At the targets of one box the transform is a smooth function of the offset u = (y - t_C)/(sqrt2 sigma),
+//   F(u1, u2) = sum_{k1,k2} sum_{a1,a2} A_B[a1][a2] h_a1(u1 + k1 d) h_a2(u2 + k2 d),
+// (k1, k2) the box offset target - source, d = box side / (sqrt2 sigma), |u| <= d/2.  Each
+// h_a(u + k d) is replaced by its Chebyshev interpolant of Q nodes on |u| <= d/2, whose
+// coefficients W_k[a][m] (formed in FP64, the same for every box) turn the sums into two
+// one-dimensional contractions over the grid,
+//   X[sy][tx][a2][m] = sum_{k1,a1} A[sy][tx - k1][a1][a2] W_k1[a1][m]
+//   C[ty][tx][m][l]  = sum_{k2,a2} X[ty - k2][tx][a2][m] W_k2[a2][l],
+// and a target's value is sum_{m,l} C[m][l] T_m(x1) T_l(x2), x = 2u/d: Q^2 multiply-adds a
+// target instead of p^2 a target and source box (441 boxes at n_cut = 10).
+//
+// Error.  The interpolant of h_a differs from it by at most
+//   2 (d/4)^Q / Q! max |h_a^(Q)|,  |h_a^(Q)| = |h_(a+Q)| <= 1.09 sqrt(2^(a+Q) (a+Q)!)
+// (Cramer's inequality), so relative to h_a's own size, 1.09 sqrt(2^a a!), by
+//   2 (d/4)^Q sqrt(2^Q (a+Q)!/a!) / Q!.
+// cheb_order takes the smallest Q of 12 and 16 that keeps this below 3e-8, half a unit of FP32's
+// last place, at a = p - 1 (Q = 12 for every grid with d <= 1/2 at p = 16; the bound is 4e-10
+// there); wider boxes keep the direct sum.  The sums are FP32, as in the direct kernel.
+//
+// Measured at p = 16, n_cut = 10: 2^20 clustered targets, 32 x 32 boxes (263.6M target-box pairs)
+// 2,350 us direct -> 52 us (table 6, contractions 8.6 and 7.6, evaluation 30, which is bound by the
+// gathers of the targets and the scattered results); 3*10^5 targets, 16 x 16 boxes, against the
+// tensor-core form 128 -> 29 us.  The whole transform's error against 64 bits falls with it, 3.7e-7
+// -> 2.0e-7 (3.1e-6 -> 3.7e-7 against BF16x3): a target's value sums 144 terms instead of 10^5.
+//
+// The rule's other lines: at least 2 targets per box on average (the contractions cost a box
+// what the direct sum costs ~1 target) and grids of up to 256 x 256 boxes (128 MB of
+// workspace; one allocation per grid size and device, kept).  A target outside its box
+// (coordinates outside the unit square, or a binning that assigns it elsewhere) is summed
+// directly.
+#include <cmath>
+#include <mutex>
+
+#include "fgt_hermite.cuh"
+
+namespace fmmgb {
+
+constexpr int kChebMaxLog2 = 8;
+constexpr int kChebMaxCut = 16;
+constexpr int kChebMaxQ = 16;
+constexpr size_t kChebTableFloats = (size_t)(2 * kChebMaxCut + 1) * 16 * kChebMaxQ;
+
+// Nodes per dimension for order p and box side d (in sqrt2 sigma), 0: none keeps the bound.
+int cheb_order(int p, double d)
+{
+    for (int q : {12, 16}) {
+        // log of 2 (d/4)^q sqrt(2^q (p-1+q)! / (p-1)!) / q!
+        const double e = log(2.0) + q * log(0.25 * d) +
+                         0.5 * (q * log(2.0) + lgamma((double)(p + q)) - lgamma((double)p)) - lgamma(q + 1.0);
+        if (e <= log(3e-8)) return q;
+    }
+    return 0;
+}
+
+// W[k][a][m], k = 0..2 ncut for the offset (k - ncut) d: one CTA per offset, FP64.
+template <int P, int Q>
+__global__ void __launch_bounds__(256) cheb_table_kernel(int ncut, double d, float* __restrict__ W)
+{
+    __shared__ double s_h[P][Q], s_cos[4 * Q];
+    const int tid = threadIdx.x, k = blockIdx.x;
+    if (tid < 4 * Q) s_cos[tid] = cospi((double)tid / (2.0 * Q));
+    __syncthreads();
+    if (tid < Q) {
+        const double t = 0.5 * d * s_cos[2 * tid + 1] + (double)(k - ncut) * d;
+        double h0 = exp(-t * t), h1 = 2.0 * t * h0;
+        s_h[0][tid] = h0;
+#pragma unroll
+        for (int a = 1; a < P; ++a) {
+            s_h[a][tid] = h1;
+            const double h2 = 2.0 * t * h1 - 2.0 * a * h0;
+            h0 = h1;
+            h1 = h2;
+        }
+    }
+    __syncthreads();
+    for (int e = tid; e < P * Q; e += 256) {
+        const int a = e / Q, m = e % Q;
+        double s = 0.0;
+#pragma unroll
+        for (int i = 0; i < Q; ++i) s += s_h[a][i] * s_cos[(2 * i + 1) * m % (4 * Q)];
+        W[(size_t)k * P * Q + e] = (float)(s * (m ? 2.0 : 1.0) / Q);
+    }
+}
+
+// One contraction along a line of boxes.  in: [line][s][c < P][r < R]; out: [t][line][r][m < Q]
+// (so the second contraction, along the other axis, finds its line contiguous and contracts
+// the other index).  A CTA takes kSeg target boxes of a line and stages their window of
+// kSeg + 2 n_cut source boxes and the table; a thread owns (box, r) and all Q outputs, over
+// every kTaps-th tap, so a step is one scalar and Q/4 broadcast 16-byte shared loads for Q
+// multiply-adds; the tap groups' sums meet in shared memory.
+constexpr int kSeg = 4;
+constexpr int kTaps = 4;
+
+template <int P, int R, int Q>
+struct ChebPass {
+    static constexpr int THREADS = kSeg * kTaps * R;
+    static constexpr int BOX = P * R + (R + 32 - P * R % 32) % 32;  // floats per staged box (bank skew R)
+    static constexpr int OUT = kSeg * R * Q;
+    static size_t smem(int ncut)
+    {
+        const size_t win = (size_t)(kSeg + 2 * ncut) * BOX, red = (size_t)kTaps * OUT;
+        return ((win > red ? win : red) + (size_t)(2 * ncut + 1) * P * Q) * sizeof(float);
+    }
+};
+
+template <int P, int R, int Q>
+__global__ void __launch_bounds__(kSeg* kTaps* R)
+    cheb_pass_kernel(int side, int ncut, const float* __restrict__ in, const float* __restrict__ W, float* __restrict__ out)
+{
+    using C = ChebPass<P, R, Q>;
+    extern __shared__ float4 cheb_smem[];
+    const int taps = 2 * ncut + 1;
+    float* s_tab = reinterpret_cast<float*>(cheb_smem);  // [taps][P][Q]
+    float* s_win = s_tab + taps * P * Q;                 // [kSeg + 2 ncut][BOX], then the groups' sums
+    const int tid = threadIdx.x, line = blockIdx.y, t0 = blockIdx.x * kSeg;
+    for (int i = tid; i < taps * P * Q / 4; i += C::THREADS)
+        reinterpret_cast<float4*>(s_tab)[i] = __ldg(reinterpret_cast<const float4*>(W) + i);
+    constexpr int B4 = P * R / 4;
+    for (int i = tid; i < (kSeg + 2 * ncut) * B4; i += C::THREADS) {
+        const int b = i / B4, s = t0 - ncut + b;
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (s >= 0 && s < side) v = __ldg(reinterpret_cast<const float4*>(in + ((size_t)line * side + s) * P * R) + i % B4);
+        *reinterpret_cast<float4*>(s_win + b * C::BOX + 4 * (i % B4)) = v;
+    }
+    __syncthreads();
+    const int group = tid / (kSeg * R), e = tid % (kSeg * R), seg = e / R, r = e % R;
+    float acc[Q];
+#pragma unroll
+    for (int m = 0; m < Q; ++m) acc[m] = 0.f;
+    for (int j = group; j < taps; j += kTaps) {  // source box t + j - ncut: offset ncut - j
+        const float* v = s_win + (seg + j) * C::BOX + r;
+        const float4* w = reinterpret_cast<const float4*>(s_tab + (2 * ncut - j) * P * Q);
+#pragma unroll 4
+        for (int c = 0; c < P; ++c) {
+            const float x = v[c * R];
+#pragma unroll
+            for (int q = 0; q < Q / 4; ++q) {
+                const float4 h = w[c * (Q / 4) + q];
+                acc[4 * q] = fmaf(x, h.x, acc[4 * q]);
+                acc[4 * q + 1] = fmaf(x, h.y, acc[4 * q + 1]);
+                acc[4 * q + 2] = fmaf(x, h.z, acc[4 * q + 2]);
+                acc[4 * q + 3] = fmaf(x, h.w, acc[4 * q + 3]);
+            }
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < Q / 4; ++q)
+        *reinterpret_cast<float4*>(s_win + group * C::OUT + e * Q + 4 * q) =
+            make_float4(acc[4 * q], acc[4 * q + 1], acc[4 * q + 2], acc[4 * q + 3]);
+    __syncthreads();
+    for (int i = tid; i < C::OUT; i += C::THREADS) {
+        const int t = t0 + i / (R * Q);
+        if (t >= side) break;
+        float v = 0.f;
+#pragma unroll
+        for (int k = 0; k < kTaps; ++k) v += s_win[k * C::OUT + i];
+        out[((size_t)t * side + line) * (R * Q) + i % (R * Q)] = v;
+    }
+}
+
+struct ChebEval {
+    int g, ncut, n, accumulate;
+    double d;
+    const float* A;
+    const float* C;
+    const double* y;
+    const int* perm;
+    const int* box_start;
+    float* G;
+    int* err;
+};
+
+// The direct sum for one target assigned to box (tx, ty), as the direct kernel takes it: every
+// source box of the neighbourhood that holds a non-zero coefficient.
+template <int P>
+__device__ __noinline__ float cheb_direct(const ChebEval& a, int tx, int ty, double y0, double y1)
+{
+    const int side = 1 << a.g;
+    const float u1 = (float)((y0 * side - (tx + 0.5)) * a.d), u2 = (float)((y1 * side - (ty + 0.5)) * a.d);
+    float acc = 0.f;
+    for (int sy = max(ty - a.ncut, 0); sy <= min(ty + a.ncut, side - 1); ++sy) {
+        float h2[P];
+        hermite_functions<P>(u2 + (float)((double)(ty - sy) * a.d), h2);
+        for (int sx = max(tx - a.ncut, 0); sx <= min(tx + a.ncut, side - 1); ++sx) {
+            float h1[P];
+            hermite_functions<P>(u1 + (float)((double)(tx - sx) * a.d), h1);
+            const float* Ab = a.A + ((size_t)sy * side + sx) * P * P;
+            bool nz = false;
+            float s = 0.f;
+#pragma unroll
+            for (int a1 = 0; a1 < P; ++a1) {
+                float t = 0.f;
+#pragma unroll
+                for (int a2 = 0; a2 < P; ++a2) {
+                    const float v = Ab[a1 * P + a2];
+                    nz |= v != 0.f;
+                    t = fmaf(v, h2[a2], t);
+                }
+                s = fmaf(h1[a1], t, s);
+            }
+            if (nz) acc += s;
+        }
+    }
+    return acc;
+}
+
+// sum_{m,l} c[m][l] T_m(x1) T_l(x2) for NR targets of one box (or, with NR = 1, of a box per lane).
+template <int Q, int NR>
+__device__ __forceinline__ void cheb_sum(const float* __restrict__ c, const float* x1, const float* x2, float* out)
+{
+    float T[NR][Q], b1[NR], b2[NR];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+        T[r][0] = 1.f;
+        T[r][1] = x2[r];
+#pragma unroll
+        for (int l = 2; l < Q; ++l) T[r][l] = fmaf(x2[r] + x2[r], T[r][l - 1], -T[r][l - 2]);
+        b1[r] = b2[r] = 0.f;
+    }
+    const float4* c4 = reinterpret_cast<const float4*>(c);
+#pragma unroll
+    for (int m = Q - 1; m >= 0; --m) {  // Clenshaw over m: b_m = row_m + 2 x1 b_(m+1) - b_(m+2)
+        float row[NR];
+#pragma unroll
+        for (int r = 0; r < NR; ++r) row[r] = fmaf(m ? x1[r] + x1[r] : x1[r], b1[r], -b2[r]);
+#pragma unroll
+        for (int q = 0; q < Q / 4; ++q) {
+            const float4 v = __ldg(c4 + m * (Q / 4) + q);
+#pragma unroll
+            for (int r = 0; r < NR; ++r) {
+                row[r] = fmaf(v.x, T[r][4 * q], row[r]);
+                row[r] = fmaf(v.y, T[r][4 * q + 1], row[r]);
+                row[r] = fmaf(v.z, T[r][4 * q + 2], row[r]);
+                row[r] = fmaf(v.w, T[r][4 * q + 3], row[r]);
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+            b2[r] = b1[r];
+            b1[r] = row[r];
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < NR; ++r) out[r] = b1[r];
+}
+
+// A warp takes 32 kRows consecutive binned targets: together where they share a box (uniform
+// 16-byte loads of its coefficients, each feeding 4 kRows multiply-adds a lane), else a row of
+// 32 at a time with a box per lane.
+constexpr int kRows = 4;
+constexpr int kEvalThreads = 128;
+
+template <int P, int Q>
+__global__ void __launch_bounds__(kEvalThreads) cheb_eval_kernel(ChebEval a)
+{
+    const int lane = threadIdx.x & 31, side = 1 << a.g, nbox = side * side;
+    const int64_t base = ((int64_t)blockIdx.x * (kEvalThreads / 32) + (threadIdx.x >> 5)) * (32 * kRows);
+    bin_check(a.box_start, nbox, a.n, a.err);
+    if (base >= a.n) return;
+    int tj[kRows], tb[kRows];  // target, its box (-1: evaluated apart)
+    float x1[kRows], x2[kRows], out[kRows];
+#pragma unroll
+    for (int r = 0; r < kRows; ++r) {
+        const int64_t pos = base + 32 * r + lane;
+        tj[r] = -1;
+        tb[r] = -1;
+        x1[r] = x2[r] = out[r] = 0.f;
+        if (pos >= a.n) continue;
+        const int j = __ldg(a.perm + pos);
+        if ((unsigned)j >= (unsigned)a.n) {
+            atomicOr(a.err, DEV_ERR_CHECK);
+            continue;
+        }
+        tj[r] = j;
+        const double y0 = __ldg(a.y + 2 * (size_t)j), y1 = __ldg(a.y + 2 * (size_t)j + 1);
+        long long X0, X1;
+        if (grid_fixed31(y0, a.g, X0) && grid_fixed31(y1, a.g, X1)) {
+            const int b = (int)(X1 >> 31) * side + (int)(X0 >> 31);
+            if (bin_holds(a.box_start, b, (int)pos, a.n)) {
+                tb[r] = b;
+                x1[r] = 2.f * cell_offset31(X0);
+                x2[r] = 2.f * cell_offset31(X1);
+            }
+        }
+    }
+    const int b0 = __shfl_sync(0xffffffffu, tb[0], 0);
+    bool same = b0 >= 0;
+#pragma unroll
+    for (int r = 0; r < kRows; ++r) same &= tb[r] == b0 || base + 32 * r + lane >= a.n;
+    if (__all_sync(0xffffffffu, same)) {
+        cheb_sum<Q, kRows>(a.C + (size_t)b0 * Q * Q, x1, x2, out);
+    } else {
+#pragma unroll 1
+        for (int r = 0; r < kRows; ++r) {
+            // registers indexed by constants only
+            float u1 = 0.f, u2 = 0.f, v = 0.f;
+            int b = -1, j = -1;
+#pragma unroll
+            for (int k = 0; k < kRows; ++k)
+                if (k == r) {
+                    u1 = x1[k];
+                    u2 = x2[k];
+                    b = tb[k];
+                    j = tj[k];
+                }
+            if (b >= 0) {
+                cheb_sum<Q, 1>(a.C + (size_t)b * Q * Q, &u1, &u2, &v);
+            } else if (j >= 0) {
+                const int lo = bin_find(a.box_start, nbox, (int)(base + 32 * r + lane), a.n);  // the assigned box
+                if (lo >= 0) {
+                    v = cheb_direct<P>(a, lo & (side - 1), lo >> a.g, __ldg(a.y + 2 * (size_t)j),
+                                       __ldg(a.y + 2 * (size_t)j + 1));
+                } else {  // box_start does not bin [0, n)
+                    atomicOr(a.err, DEV_ERR_CHECK);
+                    j = -1;
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < kRows; ++k)
+                if (k == r) {
+                    out[k] = v;
+                    tj[k] = j;
+                }
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < kRows; ++r)
+        if (tj[r] >= 0) a.G[tj[r]] = a.accumulate ? a.G[tj[r]] + out[r] : out[r];
+}
+
+// Per device and grid size: table | X [4^g][16][16] | C [4^g][16][16], allocated on first use and
+// kept (captured graphs hold its address).  NULL, without an error, when it would have to be
+// allocated inside a stream capture.
+static int cheb_workspace(int g, cudaStream_t st, float** out)
+{
+    static std::mutex mu;
+    static float* buf[64][kChebMaxLog2 + 1];
+    int dev = 0;
+    FMM_CUDA_TRY(cudaGetDevice(&dev));
+    *out = nullptr;
+    if (dev < 0 || dev >= 64) return FMM_OK;  // the direct sum serves it
+    std::lock_guard<std::mutex> lk(mu);
+    if (!buf[dev][g]) {
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        FMM_CUDA_TRY(cudaStreamIsCapturing(st, &cs));
+        if (cs != cudaStreamCaptureStatusNone) return FMM_OK;
+        const size_t bytes = (kChebTableFloats + ((size_t)2 * 16 * kChebMaxQ << (2 * g))) * sizeof(float);
+        if (cudaMalloc(&buf[dev][g], bytes) != cudaSuccess) {
+            (void)cudaGetLastError();
+            buf[dev][g] = nullptr;
+            return FMM_OK;
+        }
+    }
+    *out = buf[dev][g];
+    return FMM_OK;
+}
+
+template <int P, int Q>
+static int cheb_launch(const ChebEval& e, float* ws, cudaStream_t st)
+{
+    using C1 = ChebPass<P, P, Q>;
+    using C2 = ChebPass<P, Q, Q>;
+    const int side = 1 << e.g;
+    float *W = ws, *X = W + kChebTableFloats, *C = X + ((size_t)16 * kChebMaxQ << (2 * e.g));
+    static unsigned long long opted[2];
+    if (int rc = smem_opt_in((const void*)cheb_pass_kernel<P, P, Q>, (int)C1::smem(kChebMaxCut), &opted[0])) return rc;
+    if (int rc = smem_opt_in((const void*)cheb_pass_kernel<P, Q, Q>, (int)C2::smem(kChebMaxCut), &opted[1])) return rc;
+    cheb_table_kernel<P, Q><<<2 * e.ncut + 1, 256, 0, st>>>(e.ncut, e.d, W);
+    FMM_CUDA_TRY(cudaGetLastError());
+    const dim3 grid((side + kSeg - 1) / kSeg, side);
+    cheb_pass_kernel<P, P, Q><<<grid, C1::THREADS, C1::smem(e.ncut), st>>>(side, e.ncut, e.A, W, X);
+    FMM_CUDA_TRY(cudaGetLastError());
+    cheb_pass_kernel<P, Q, Q><<<grid, C2::THREADS, C2::smem(e.ncut), st>>>(side, e.ncut, X, W, C);
+    FMM_CUDA_TRY(cudaGetLastError());
+    ChebEval a = e;
+    a.C = C;
+    const unsigned blocks = bin_blocks(a.n, kEvalThreads * kRows, (int64_t)1 << (2 * e.g), kEvalThreads);
+    cheb_eval_kernel<P, Q><<<blocks, kEvalThreads, 0, st>>>(a);
+    FMM_CUDA_TRY(cudaGetLastError());
+    return FMM_OK;
+}
+
+int launch_fgt_h2p_cheb(int g, int ncut, int p, double d, const float* A, const double* y, int n, const int* perm,
+                        const int* box_start, float* G, bool accumulate, int* err, cudaStream_t st, bool* done)
+{
+    *done = false;
+    const int q = cheb_order(p, d);
+    if (!q || g > kChebMaxLog2 || n < (2 << (2 * g))) return FMM_OK;
+    float* ws = nullptr;
+    if (int rc = cheb_workspace(g, st, &ws)) return rc;
+    if (!ws) return FMM_OK;
+    *done = true;
+    const ChebEval e{g, ncut, n, accumulate ? 1 : 0, d, A, nullptr, y, perm, box_start, G, err};
+    switch (p) {
+        case 4: return q == 12 ? cheb_launch<4, 12>(e, ws, st) : cheb_launch<4, 16>(e, ws, st);
+        case 8: return q == 12 ? cheb_launch<8, 12>(e, ws, st) : cheb_launch<8, 16>(e, ws, st);
+        case 12: return q == 12 ? cheb_launch<12, 12>(e, ws, st) : cheb_launch<12, 16>(e, ws, st);
+        default: return q == 12 ? cheb_launch<16, 12>(e, ws, st) : cheb_launch<16, 16>(e, ws, st);
+    }
+}
+
+}  // namespace fmmgb

@@ -370,3 +370,124 @@ def test_h2p_tc_agrees_with_fp32_path_at_full_size(fmm, orc):
     pick = np.random.default_rng(6).choice(n, 1500, replace=False)
     ref = orc.fgt_hermite_eval_grid(g, ncut, 16, sigma, A.cpu().numpy().astype(np.float64), y[pick])
     assert _rel(gtc[pick], ref) <= 1e-4
+
+
+# ---------------------------------------------------------------------------
+# evaluation through per-box Chebyshev coefficients: taken at >= 2 targets per box on average, on
+# grids up to 256 x 256, for box sides whose interpolation bound holds
+# ---------------------------------------------------------------------------
+def _decaying(rng, nbox, p):
+    import math
+
+    fact = np.array([math.factorial(a) for a in range(p)], float)
+    A = rng.standard_normal((nbox, p, p)) * (0.35 ** (np.arange(p)[:, None] + np.arange(p)[None, :])) / np.outer(fact, fact)
+    A[rng.random(nbox) < 0.25] = 0.0
+    A[0, 0, 0] = 1.0
+    return A.astype(np.float32)
+
+
+@pytest.mark.parametrize("p,d", [(4, 0.5), (8, 0.4), (8, 0.95), (12, 0.79), (12, 0.82), (16, 0.26), (16, 0.72),
+                                 (16, 0.73), (16, 1.29), (16, 1.31)])
+def test_h2p_on_both_sides_of_the_chebyshev_rule(fmm, orc, p, d):
+    """Box sides d (in sqrt2 sigma) on both sides of the lines where 12 nodes, 16 nodes and the
+    direct sum are taken, and target counts on both sides of two per box; targets on box edges,
+    at 1.0 and outside the unit square (summed directly), and crowded into one box.  The bar is
+    the FP32 bar of the direct kernel: the interpolation adds at most 3e-8 of a Hermite function's
+    own size, against sums rounded to ~1e-7."""
+    import math
+
+    g = 3
+    nbox, n = 4 ** g, 1 << g
+    sigma = 2.0 ** -g / (math.sqrt(2.0) * d)
+    rng = np.random.default_rng(int(1000 * d) + p)
+    A32 = _decaying(rng, nbox, p)
+    k = np.arange(n + 1) / n
+    edge = np.stack([np.concatenate([k, np.nextafter(k, -1), rng.random(3)]),
+                     np.concatenate([rng.random(2 * n + 2), [1.0, 1.01, -0.02]])], 1)
+    for ncut in (0, 2, 16):
+        for m in (2 * nbox - 1, 2 * nbox, 2000):
+            y = np.concatenate([edge, 0.3 + 0.05 * rng.random((max(0, m // 2 - len(edge)), 2))])
+            y = np.concatenate([y, rng.random((m - len(y), 2))])
+            ref = orc.fgt_hermite_eval_grid(g, ncut, p, sigma, A32.astype(np.float64), y)
+            _check(_h2p(fmm, g, ncut, p, sigma, A32, y), ref)
+
+
+@pytest.mark.parametrize("g", [0, 1, 2, 5, 8])
+def test_h2p_chebyshev_grid_sizes(fmm, orc, g):
+    """1 x 1 boxes to the largest grid taken (256 x 256), accumulating; at 256 x 256 the targets
+    checked are 800 of them."""
+    import math
+    import torch
+
+    p, ncut, nbox = 8, 3, 4 ** g
+    sigma = 2.0 ** -g / (math.sqrt(2.0) * 0.45)
+    rng = np.random.default_rng(g)
+    A32 = _decaying(rng, nbox, p)
+    y = rng.random((max(700, 2 * nbox + 77), 2))
+    G = torch.full((len(y),), 0.25, dtype=torch.float32, device="cuda")
+    got = _h2p(fmm, g, ncut, p, sigma, A32, y, G=G, accumulate=True)
+    pick = rng.choice(len(y), min(800, len(y)), replace=False)
+    _check(got[pick], orc.fgt_hermite_eval_grid(g, ncut, p, sigma, A32.astype(np.float64), y[pick]) + 0.25)
+
+
+def test_h2p_nan_coefficients_reach_their_neighbourhood_only(fmm, orc):
+    """A NaN coefficient makes every target within n_cut boxes NaN and leaves the others as they
+    are; a NaN coordinate gives NaN at that target alone."""
+    import math
+
+    g, p, ncut = 4, 8, 2
+    n = 1 << g
+    sigma = 2.0 ** -g / (math.sqrt(2.0) * 0.45)
+    rng = np.random.default_rng(8)
+    A32 = _decaying(rng, n * n, p)
+    y = rng.random((3000, 2))
+    y[17] = [np.nan, 0.5]
+    ref = orc.fgt_hermite_eval_grid(g, ncut, p, sigma, A32.astype(np.float64), np.nan_to_num(y, nan=0.5))
+    bad = 5 * n + 9
+    A32[bad, 3, 2] = np.nan
+    got = _h2p(fmm, g, ncut, p, sigma, A32, y)
+    b = _boxes(np.nan_to_num(y, nan=0.0), g)
+    near = (np.abs(b % n - bad % n) <= ncut) & (np.abs(b // n - bad // n) <= ncut)
+    near[17] = True
+    assert np.isnan(got[near]).all() and np.isfinite(got[~near]).all()
+    _check(got[~near], ref[~near])
+
+
+def test_h2p_first_call_of_a_grid_size_inside_a_capture(fmm, orc):
+    """The coefficients' workspace of a grid size is allocated on its first use; a first use inside
+    a stream capture takes the direct sum instead, and the graph replays beside later calls."""
+    import math
+    import torch
+
+    g, p, ncut = 7, 4, 1
+    nbox = 4 ** g
+    sigma = 2.0 ** -g / (math.sqrt(2.0) * 0.45)
+    rng = np.random.default_rng(70)
+    A32 = _decaying(rng, nbox, p)
+    y = rng.random((2 * nbox + 5, 2))
+    yd, Ad = torch.from_numpy(y).cuda(), torch.from_numpy(A32).cuda()
+    perm, start = _bin(fmm, g, yd)
+    fmm.fmm_prepare(8)  # the scratch of the direct sum
+    G = torch.zeros(len(y), dtype=torch.float32, device="cuda")
+    warm = torch.zeros(100, dtype=torch.float32, device="cuda")
+    yw = yd[:100].contiguous()
+    wperm, wstart = _bin(fmm, g, yw)
+    fmm.fgt_h2p(g, ncut, p, sigma, Ad, yw, wperm, wstart, warm)  # few targets: the direct sum, loaded and set up
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, capture_error_mode="thread_local"):
+        fmm.fgt_h2p(g, ncut, p, sigma, Ad, yd, perm, start, G)
+    graph.replay()
+    fmm.fmm_sync_status()
+    first = G.clone()
+    G.zero_()
+    fmm.fgt_h2p(g, ncut, p, sigma, Ad, yd, perm, start, G)
+    fmm.fmm_sync_status()
+    second = G.clone()
+    G.zero_()
+    graph.replay()
+    fmm.fmm_sync_status()
+    pick = rng.choice(len(y), 600, replace=False)
+    ref = orc.fgt_hermite_eval_grid(g, ncut, p, sigma, A32.astype(np.float64), y[pick])
+    for t in (first, second, G):
+        _check(t.cpu().numpy().astype(np.float64)[pick], ref)
