@@ -232,6 +232,10 @@ int launch_p2m_binned(int level, int p, const double* xy, const double* c, int n
 int launch_p2m(int level, int p, const double* xy, const double* c, int64_t n, float2* M, bool accumulate,
                cudaStream_t st);
 int launch_m2m(int child_level, int p, const float2* Mc, float2* Mp, bool accumulate, cudaStream_t st);
+// M2M (up) / L2L (down) and their conjugate transposes for the orders of the M2L path (shift.cu)
+bool shift_supported(int p);
+int launch_shift(bool up, int child_level, int p, const float2* In, float2* Out, float scale, bool conj, bool acc,
+                 cudaStream_t st);
 // FGT H2T on the tensor cores (fgt_h2t_tc.cu): p = 16, grid_log2 >= 3, n_cut <= 16
 bool fgt_h2t_tc_supported(int g, int ncut, int p);
 int launch_fgt_h2t_tc(int g, int ncut, double sigma, bool split, const float* A, float* Y, float* C, bool acc,

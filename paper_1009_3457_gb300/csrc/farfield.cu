@@ -11,6 +11,7 @@
 
 namespace fmmgb {
 
+// The orders of the M2L path take the kernels of shift.cu; these two serve every other p.
 // One thread per (child box, j): Lc[child][j] (+)= sum_n T_c[j][n] Lp[parent][n]; the
 // binomials from the compile-time table.
 __global__ void l2l_kernel(int child_level, int p, const float2* __restrict__ Lp, float2* __restrict__ Lc,
@@ -221,6 +222,7 @@ __global__ void p2m_adjoint_kernel(int level, int p, const double* __restrict__ 
 
 int launch_l2l(int child_level, int p, const float2* Lp, float2* Lc, bool acc, bool adjoint, cudaStream_t st)
 {
+    if (shift_supported(p)) return launch_shift(adjoint, child_level, p, Lp, Lc, 0.5f, adjoint, acc, st);
     const int64_t side = (int64_t)1 << child_level;
     const int64_t total = (adjoint ? side * side / 4 : side * side) * p;
     const unsigned blocks = (unsigned)((total + 255) / 256);

@@ -136,6 +136,7 @@ int launch_p2m_binned(int level, int p, const double* xy, const double* c, int n
     return FMM_OK;
 }
 
+// The orders of the M2L path take the kernels of shift.cu; these serve every other p.
 // Scaled M2M: parent box side R = 2r, child offset z = (x_c - x_P)/R = (+-1/4, +-1/4):
 //   M~P_j = sum_{k<=j} C(j,k) z^(j-k) 2^-k M~c_k, summed over the 4 children.
 // The entries (binomials, powers of (+-1 +- i)/4, powers of 2) are exact in FP32;
@@ -261,6 +262,7 @@ int launch_p2m(int level, int p, const double* xy, const double* c, int64_t n, f
 
 int launch_m2m_adjoint(int child_level, int p, const float2* Wp, float2* Wc, bool acc, cudaStream_t st)
 {
+    if (shift_supported(p)) return launch_shift(false, child_level, p, Wp, Wc, 1.f, true, acc, st);
     const int64_t side = (int64_t)1 << child_level;
     const int64_t total = side * side * p;
     m2m_adjoint_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(child_level, p, Wp, Wc, acc ? 1 : 0);
@@ -270,6 +272,7 @@ int launch_m2m_adjoint(int child_level, int p, const float2* Wp, float2* Wc, boo
 
 int launch_m2m(int child_level, int p, const float2* Mc, float2* Mp, bool acc, cudaStream_t st)
 {
+    if (shift_supported(p)) return launch_shift(true, child_level, p, Mc, Mp, 1.f, false, acc, st);
     const int64_t np = (int64_t)1 << (child_level - 1);
     const int64_t total = np * np * p;
     m2m_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(child_level, p, Mc, Mp, acc ? 1 : 0);

@@ -262,3 +262,45 @@ def test_m2m_adjoint(fmm, orc):
             for px in range(n // 2):
                 ref[(2 * py + iy) * n + 2 * px + ix] = T.conj().T @ W[py * (n // 2) + px]
     assert _rel(_host(Wc), ref) <= 1e-6
+
+
+@pytest.mark.parametrize("p", [6, 7, 8, 12, 16, 24])
+@pytest.mark.parametrize("cl", [1, 2, 5])
+def test_child_parent_translations_of_every_order(fmm, p, cl):
+    """M2M, L2L and their conjugate transposes against their entries in FP64, written and
+    accumulated: the orders with the four children folded (the last block ragged at p = 6, 12, 24)
+    and one (7) that takes the general kernels.  FP32 sums of at most 4 p products: 1e-6."""
+    import math
+
+    rng = np.random.default_rng(100 * cl + p)
+    half, nc = 1 << (cl - 1), 1 << cl
+    n = np.arange(p)
+    C = np.array([[math.comb(a, b) if b <= a else 0 for b in range(p)] for a in range(p)], float)
+    par = rng.standard_normal((half, half, p)) + 1j * rng.standard_normal((half, half, p))
+    chl = rng.standard_normal((nc, nc, p)) + 1j * rng.standard_normal((nc, nc, p))
+    par, chl = par.astype(np.complex64), chl.astype(np.complex64)
+    up, upa = np.zeros((2, half, half, p), complex)
+    dn, dna = np.zeros((2, nc, nc, p), complex)
+    for cy in (0, 1):
+        for cx in (0, 1):
+            z = complex(cx - 0.5, cy - 0.5) / 2
+            Z = np.where(n[:, None] >= n[None, :], z ** np.maximum(n[:, None] - n[None, :], 0), 0)
+            M2M = C * Z * 0.5 ** n[None, :]            # parent j from child k
+            L2L = (C * Z * 0.5 ** (n[None, :] + 1)).T  # child j from parent n
+            sub = np.s_[cy::2, cx::2]
+            up += chl[sub] @ M2M.T
+            upa += chl[sub] @ L2L.conj()
+            dn[sub] = par @ L2L.T
+            dna[sub] = par @ M2M.conj()
+    for f, src, ref in ((fmm.fmm_m2m, chl, up), (fmm.fmm_l2l_adjoint, chl, upa), (fmm.fmm_l2l, par, dn),
+                        (fmm.fmm_m2m_adjoint, par, dna)):
+        src, ref = src.reshape(-1, p), ref.reshape(-1, p)
+        out = _dev(np.full(ref.shape, np.nan))
+        f(cl, p, _dev(src), out)
+        fmm.fmm_sync_status()
+        assert _rel(_host(out), ref) <= 1e-6
+        x = (rng.standard_normal(ref.shape) + 1j * rng.standard_normal(ref.shape)).astype(np.complex64)
+        out = _dev(x)
+        f(cl, p, _dev(src), out, accumulate=True)
+        fmm.fmm_sync_status()
+        assert _rel(_host(out), ref + x) <= 1e-6
