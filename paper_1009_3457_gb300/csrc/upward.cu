@@ -9,7 +9,10 @@ namespace fmmgb {
 
 // M~_b[k] += c_i w^k,  w = (y_i - x_b) / r_l  (|w| <= 1/sqrt 2): w read off the bits of
 // the FP64 coordinates (points outside the unit square: the clamped box, in FP64), the
-// powers in FP32, added by FP32 atomics.
+// powers in FP32, added by FP32 atomics, two coefficients (16 bytes) an atomic where the rows
+// allow it (VEC: M 16-byte aligned, p even).  Bound by the atomics: 2^20 clustered
+// points at level 9, p = 16, 211 us with 32 4-byte atomics a point, 57 us with 8 of 16 bytes.
+template <bool VEC>
 __global__ void p2m_kernel(int level, int p, const double* __restrict__ xy, const double* __restrict__ c, int64_t n,
                            float2* __restrict__ M)
 {
@@ -37,11 +40,20 @@ __global__ void p2m_kernel(int level, int p, const double* __restrict__ xy, cons
     float pr = (float)c[i], pi = 0.f;
     float2* mb = M + ((size_t)iy * side + ix) * p;
     for (int k = 0; k < p; ++k) {
-        atomicAdd(&mb[k].x, pr);
-        atomicAdd(&mb[k].y, pi);
+        const float ar = pr, ai = pi;
         const float t = fmaf(pr, wr, -pi * wi);
         pi = fmaf(pr, wi, pi * wr);
         pr = t;
+        if constexpr (VEC) {
+            atomicAdd(reinterpret_cast<float4*>(mb + k), make_float4(ar, ai, pr, pi));
+            const float u = fmaf(pr, wr, -pi * wi);
+            pi = fmaf(pr, wi, pi * wr);
+            pr = u;
+            ++k;
+        } else {
+            atomicAdd(&mb[k].x, ar);
+            atomicAdd(&mb[k].y, ai);
+        }
     }
 }
 
@@ -255,7 +267,10 @@ int launch_p2m(int level, int p, const double* xy, const double* c, int64_t n, f
     if (!acc) FMM_CUDA_TRY(cudaMemsetAsync(M, 0, bytes, st));
     if (n == 0) return FMM_OK;
     const int64_t blocks = (n + 255) / 256;
-    p2m_kernel<<<(unsigned)blocks, 256, 0, st>>>(level, p, xy, c, n, M);
+    if (p % 2 == 0 && ((uintptr_t)M & 15) == 0)
+        p2m_kernel<true><<<(unsigned)blocks, 256, 0, st>>>(level, p, xy, c, n, M);
+    else
+        p2m_kernel<false><<<(unsigned)blocks, 256, 0, st>>>(level, p, xy, c, n, M);
     FMM_CUDA_TRY(cudaGetLastError());
     return FMM_OK;
 }

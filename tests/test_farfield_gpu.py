@@ -304,3 +304,25 @@ def test_child_parent_translations_of_every_order(fmm, p, cl):
         f(cl, p, _dev(src), out, accumulate=True)
         fmm.fmm_sync_status()
         assert _rel(_host(out), ref + x) <= 1e-6
+
+
+def test_p2m_orders_and_alignments(fmm, orc):
+    """Per-point P2M with 16-byte atomics (even p, aligned rows) and 4-byte ones (odd p, rows only
+    8-byte aligned) against each other's FP64 sums."""
+    import torch
+
+    rng = np.random.default_rng(77)
+    level, side = 3, 8
+    xy = np.concatenate([rng.random((3000, 2)), 0.4 + 0.01 * rng.random((500, 2)), [[1.0, 0.2], [-0.01, 0.5]]])
+    c = rng.uniform(-1, 1, len(xy))
+    cell = np.clip(np.floor(xy * side), 0, side - 1)
+    d = (xy * side - cell - 0.5) @ np.array([1, 1j])
+    box = (cell[:, 1] * side + cell[:, 0]).astype(int)
+    for p, shift in ((16, 0), (16, 1), (7, 0), (2, 0), (1, 0)):
+        ref = np.zeros((side * side, p), complex)
+        np.add.at(ref, box, c[:, None] * d[:, None] ** np.arange(p))
+        buf = torch.full((side * side * p + 1,), float("nan"), dtype=torch.complex64, device="cuda")
+        M = buf[shift:shift + side * side * p].view(side * side, p)
+        fmm.fmm_p2m(level, p, torch.from_numpy(xy).cuda(), torch.from_numpy(c).cuda(), M)
+        fmm.fmm_sync_status()
+        assert _rel(_host(M), ref) <= 1e-6, (p, shift)
