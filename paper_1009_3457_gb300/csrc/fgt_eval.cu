@@ -4,7 +4,7 @@
 //   G(y) (+)= sum_{b1,b2 < p} C[box][b1][b2] t1^b1 t2^b2,  t = (y - t_C) / (sqrt(2) sigma).
 // With P2H and H2T this completes the transform on the device.  Horner in
 // FP32 on t formed in FP64 (|t| <= 0.36 on the workload grids).
-#include "common.cuh"
+#include "fgt_hermite.cuh"
 
 namespace fmmgb {
 
@@ -51,15 +51,52 @@ static int t2p_p(int g, double sigma, const float* C, int64_t n, const double* y
     return FMM_OK;
 }
 
-// T2P at targets binned by box (fgt_bin_points): one block per box holds the
-// box's p x p Taylor coefficients in shared memory (every lane reads the same
-// entry: a broadcast) and evaluates them at each of the box's targets, whose
-// offsets from the box centre are read off the bits of their FP64 coordinates.
-// The per-target kernel above reads a random box's 1 KB of coefficients per
-// target from L1/L2.
+// T2P at targets binned by box (fgt_bin_points).  A warp takes 128 consecutive binned targets,
+// four per lane: where they share a box, each uniform 16-byte load of its coefficients (served
+// by the L1) feeds 16 multiply-adds a lane; else a row of 32 targets at a time, each lane from
+// its own box.  A warp's work does not depend on how the targets are spread over the boxes (a
+// block per box left the SMs waiting for the crowded boxes), and a scalar shared load per
+// multiply-add is gone.  Target offsets are read off the bits of the FP64 coordinates.
+// 2^20 uniform targets on 32 x 32 boxes, p = 16: 40 -> 26 us, bound by the gathers and the
+// scattered results.
 constexpr int kT2pThreads = 128;
+constexpr int kT2pRows = 4;
 
-template <int P>
+template <bool VEC>
+__device__ __forceinline__ float4 t2p_load4(const float* c)
+{
+    if constexpr (VEC) return __ldg(reinterpret_cast<const float4*>(c));
+    return make_float4(__ldg(c), __ldg(c + 1), __ldg(c + 2), __ldg(c + 3));
+}
+
+// sum_{b1,b2} c[b1][b2] t1^b1 t2^b2 by Horner's rule, NR targets of one box (NR = 1: a box per lane)
+template <int P, int NR, bool VEC>
+__device__ __forceinline__ void t2p_sum(const float* __restrict__ c, const float* t1, const float* t2, float* out)
+{
+#pragma unroll
+    for (int r = 0; r < NR; ++r) out[r] = 0.f;
+#pragma unroll 4
+    for (int b1 = P - 1; b1 >= 0; --b1) {
+        float inner[NR];
+#pragma unroll
+        for (int r = 0; r < NR; ++r) inner[r] = 0.f;
+#pragma unroll
+        for (int q = P / 4 - 1; q >= 0; --q) {
+            const float4 v = t2p_load4<VEC>(c + b1 * P + 4 * q);
+#pragma unroll
+            for (int r = 0; r < NR; ++r) {
+                inner[r] = fmaf(inner[r], t2[r], v.w);
+                inner[r] = fmaf(inner[r], t2[r], v.z);
+                inner[r] = fmaf(inner[r], t2[r], v.y);
+                inner[r] = fmaf(inner[r], t2[r], v.x);
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < NR; ++r) out[r] = fmaf(out[r], t1[r], inner[r]);
+    }
+}
+
+template <int P, bool VEC>
 __global__ void __launch_bounds__(kT2pThreads) fgt_t2p_binned_kernel(int g, double inv_scale, float dcell,
                                                                      const float* __restrict__ C, int n,
                                                                      const double* __restrict__ y,
@@ -67,44 +104,60 @@ __global__ void __launch_bounds__(kT2pThreads) fgt_t2p_binned_kernel(int g, doub
                                                                      const int* __restrict__ box_start,
                                                                      float* __restrict__ G, int accumulate, int* err)
 {
-    __shared__ float s_c[P * P];
-    const int side = 1 << g;
-    const int b = blockIdx.x, tid = threadIdx.x;
-    const int bx = b & (side - 1), by = b >> g;
-    const int first = box_start[b], end = box_start[b + 1];
-    if (first < 0 || end > n || first > end) {
-        if (tid == 0) atomicOr(err, DEV_ERR_CHECK);
-        return;
-    }
-    if (first == end) return;
-    for (int k = tid; k < P * P; k += kT2pThreads) s_c[k] = C[(size_t)b * P * P + k];
-    __syncthreads();
-    for (int q = first + tid; q < end; q += kT2pThreads) {
-        const int j = perm[q];
+    const int lane = threadIdx.x & 31, side = 1 << g, nbox = side * side;
+    const int64_t base = ((int64_t)blockIdx.x * (kT2pThreads / 32) + (threadIdx.x >> 5)) * (32 * kT2pRows);
+    bin_check(box_start, nbox, n, err);
+    if (base >= n) return;
+    int tj[kT2pRows], tb[kT2pRows];
+    float t1[kT2pRows], t2[kT2pRows], out[kT2pRows];
+#pragma unroll
+    for (int r = 0; r < kT2pRows; ++r) {
+        const int64_t pos = base + 32 * r + lane;
+        tj[r] = tb[r] = -1;
+        t1[r] = t2[r] = out[r] = 0.f;
+        if (pos >= n) continue;
+        const int j = __ldg(perm + pos);
         if ((unsigned)j >= (unsigned)n) {
             atomicOr(err, DEV_ERR_CHECK);
             continue;
         }
-        const double y0 = y[2 * (size_t)j], y1 = y[2 * (size_t)j + 1];
+        const double y0 = __ldg(y + 2 * (size_t)j), y1 = __ldg(y + 2 * (size_t)j + 1);
         long long X0, X1;
-        float t1, t2;
-        if (grid_fixed31(y0, g, X0) && grid_fixed31(y1, g, X1) && (int)(X0 >> 31) == bx && (int)(X1 >> 31) == by) {
-            t1 = cell_offset31(X0) * dcell;
-            t2 = cell_offset31(X1) * dcell;
-        } else {  // outside the unit square (the nearest box): offset in FP64
-            t1 = (float)((y0 * side - (bx + 0.5)) / side * inv_scale);
-            t2 = (float)((y1 * side - (by + 0.5)) / side * inv_scale);
+        if (grid_fixed31(y0, g, X0) && grid_fixed31(y1, g, X1)) {
+            const int b = (int)(X1 >> 31) * side + (int)(X0 >> 31);
+            if (bin_holds(box_start, b, (int)pos, n)) {
+                tj[r] = j;
+                tb[r] = b;
+                t1[r] = cell_offset31(X0) * dcell;
+                t2[r] = cell_offset31(X1) * dcell;
+            }
         }
-        float outer = 0.f;
-#pragma unroll 4
-        for (int b1 = P - 1; b1 >= 0; --b1) {
-            float inner = 0.f;
-#pragma unroll
-            for (int b2 = P - 1; b2 >= 0; --b2) inner = fmaf(inner, t2, s_c[b1 * P + b2]);
-            outer = fmaf(outer, t1, inner);
+        if (tb[r] < 0) {  // not in the box of its coordinates: the box the binning assigns, offset in FP64
+            const int b = bin_find(box_start, nbox, (int)pos, n);
+            if (b >= 0) {
+                tj[r] = j;
+                tb[r] = b;
+                t1[r] = (float)((y0 * side - ((b & (side - 1)) + 0.5)) / side * inv_scale);
+                t2[r] = (float)((y1 * side - ((b >> g) + 0.5)) / side * inv_scale);
+            } else {  // box_start does not bin [0, n)
+                atomicOr(err, DEV_ERR_CHECK);
+            }
         }
-        G[j] = accumulate ? G[j] + outer : outer;
     }
+    const int b0 = __shfl_sync(0xffffffffu, tb[0], 0);
+    bool same = b0 >= 0;
+#pragma unroll
+    for (int r = 0; r < kT2pRows; ++r) same &= tb[r] == b0 || base + 32 * r + lane >= n;
+    if (__all_sync(0xffffffffu, same)) {
+        t2p_sum<P, kT2pRows, VEC>(C + (size_t)b0 * P * P, t1, t2, out);
+    } else {
+#pragma unroll
+        for (int r = 0; r < kT2pRows; ++r)
+            if (tb[r] >= 0) t2p_sum<P, 1, VEC>(C + (size_t)tb[r] * P * P, t1 + r, t2 + r, out + r);
+    }
+#pragma unroll
+    for (int r = 0; r < kT2pRows; ++r)
+        if (tj[r] >= 0) G[tj[r]] = accumulate ? G[tj[r]] + out[r] : out[r];
 }
 
 template <int P>
@@ -112,8 +165,14 @@ static int t2p_binned_p(int g, double sigma, const float* C, int n, const double
                         const int* box_start, float* G, bool acc, int* err, cudaStream_t st)
 {
     const double inv_scale = 1.0 / (sqrt(2.0) * sigma);
-    fgt_t2p_binned_kernel<P><<<1u << (2 * g), kT2pThreads, 0, st>>>(
-        g, inv_scale, (float)(ldexp(1.0, -g) * inv_scale), C, n, y, perm, box_start, G, acc ? 1 : 0, err);
+    const float dcell = (float)(ldexp(1.0, -g) * inv_scale);
+    const unsigned grid = bin_blocks(n, kT2pThreads * kT2pRows, (int64_t)1 << (2 * g), kT2pThreads);
+    if (((uintptr_t)C & 15) == 0)
+        fgt_t2p_binned_kernel<P, true><<<grid, kT2pThreads, 0, st>>>(g, inv_scale, dcell, C, n, y, perm, box_start, G,
+                                                                     acc ? 1 : 0, err);
+    else
+        fgt_t2p_binned_kernel<P, false><<<grid, kT2pThreads, 0, st>>>(g, inv_scale, dcell, C, n, y, perm, box_start, G,
+                                                                      acc ? 1 : 0, err);
     FMM_CUDA_TRY(cudaGetLastError());
     return FMM_OK;
 }

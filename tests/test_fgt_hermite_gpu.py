@@ -491,3 +491,57 @@ def test_h2p_first_call_of_a_grid_size_inside_a_capture(fmm, orc):
     ref = orc.fgt_hermite_eval_grid(g, ncut, p, sigma, A32.astype(np.float64), y[pick])
     for t in (first, second, G):
         _check(t.cpu().numpy().astype(np.float64)[pick], ref)
+
+
+@pytest.mark.parametrize("p", [4, 8, 12, 16])
+def test_p2h_and_t2p_binned_runs_and_alignments(fmm, orc, p):
+    """P2H over 256-point blocks of one box, of several and of many, the last one ragged, into
+    coefficients 16-byte aligned and not; T2P at the same points from coefficients aligned and not
+    (several targets of one box together, and a box per lane)."""
+    import torch
+
+    g, sigma = 3, 0.2
+    rng = np.random.default_rng(p)
+    x = np.concatenate([0.51 + 0.01 * rng.random((700, 2)), 0.13 + 0.3 * rng.random((300, 2)), rng.random((411, 2)),
+                        [[1.0, 0.4], [1.02, 0.7], [-0.01, 0.3]]])
+    q = rng.uniform(-1, 1, len(x))
+    ref = orc.fgt_p2h_grid(g, p, sigma, x, q)
+    xd, qd = torch.from_numpy(x).cuda(), torch.from_numpy(q).cuda()
+    perm, start = _bin(fmm, g, xd)
+    m = 4 ** g * p * p
+    ev = orc.fgt_taylor_eval_grid(g, p, sigma, ref.astype(np.float32).astype(np.float64), x)
+    for shift in (0, 1):
+        A = torch.full((m + 1,), float("nan"), dtype=torch.float32, device="cuda")[shift:shift + m].view(4 ** g, p, p)
+        fmm.fgt_p2h_binned(g, p, sigma, xd, qd, perm, A)
+        fmm.fmm_sync_status()
+        got = A.cpu().numpy().astype(np.float64)
+        assert np.linalg.norm(got - ref) / np.linalg.norm(ref) <= 1e-5
+        A.copy_(torch.from_numpy(ref.astype(np.float32)))
+        G = torch.zeros(len(x), dtype=torch.float32, device="cuda")
+        fmm.fgt_t2p_binned(g, p, sigma, A, xd, perm, start, G)
+        fmm.fmm_sync_status()
+        _check(G.cpu().numpy().astype(np.float64), ev)
+
+
+def test_t2p_and_h2p_report_a_bad_box_start(fmm):
+    """A box start out of range, or a box that ends before it starts, sets the error word; the other
+    boxes' targets are evaluated."""
+    import torch
+
+    g, p = 3, 4
+    y = torch.from_numpy(np.random.default_rng(2).random((600, 2))).cuda()
+    perm, start = _bin(fmm, g, y)
+    C = torch.zeros((4 ** g, p, p), dtype=torch.float32, device="cuda")
+    C[:, 0, 0] = 1.0
+    for b, v in ((5, -3), (40, 601), (20, 0)):
+        bad = start.clone()
+        bad[b] = v
+        for call in (lambda G: fmm.fgt_t2p_binned(g, p, 0.2, C, y, perm, bad, G),
+                     lambda G: fmm.fgt_h2p(g, 2, p, 0.2, C, y, perm, bad, G)):
+            G = torch.zeros(600, dtype=torch.float32, device="cuda")
+            call(G)
+            with pytest.raises(fmm.FmmError) as e:
+                fmm.fmm_sync_status()
+            assert e.value.code == fmm.FMM_EDEVICE
+            fmm.fmm_sync_status()
+            assert int((G > 0).sum()) > 500
