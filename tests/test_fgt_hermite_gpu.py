@@ -545,3 +545,19 @@ def test_t2p_and_h2p_report_a_bad_box_start(fmm):
             assert e.value.code == fmm.FMM_EDEVICE
             fmm.fmm_sync_status()
             assert int((G > 0).sum()) > 500
+
+
+@pytest.mark.parametrize("g", [6, 7, 8, 9])
+def test_bin_points_scans_over_many_blocks(fmm, g):
+    """Grids whose prefix is taken by one block (64 x 64) and by many, a few boxes crowded."""
+    import torch
+
+    rng = np.random.default_rng(g)
+    y = np.concatenate([rng.random((20000, 2)), 0.7 + 1e-4 * rng.random((5000, 2)), np.full((777, 2), 0.999999)])
+    perm, start = _bin(fmm, g, torch.from_numpy(y).cuda())
+    box = _boxes(y, g)
+    np.testing.assert_array_equal(np.diff(start.cpu().numpy()), np.bincount(box, minlength=4 ** g))
+    assert int(start[0]) == 0
+    pm = perm.cpu().numpy()
+    np.testing.assert_array_equal(box[pm], np.sort(box))
+    assert np.array_equal(np.sort(pm), np.arange(len(y)))
