@@ -23,7 +23,9 @@ class M2LLevels(torch.autograd.Function):
     @staticmethod
     def forward(ctx, tree, p, *Ms):
         Ms = [m.contiguous() for m in Ms]
-        Ls = [torch.zeros_like(m) for m in Ms]
+        Ls = [torch.empty_like(m) for m in Ms]
+        if tree.adaptive:  # entries of absent boxes are not written: one launch zeroes every level
+            torch._foreach_zero_(Ls)
         fmmgb.fmm_m2l_levels(tree, 2, p, Ms, Ls)
         ctx.tree = tree
         ctx.p = p
@@ -32,7 +34,9 @@ class M2LLevels(torch.autograd.Function):
     @staticmethod
     def backward(ctx, *gLs):
         Ws = [g.contiguous() for g in gLs]
-        Gs = [torch.zeros_like(w) for w in Ws]
+        Gs = [torch.empty_like(w) for w in Ws]
+        if ctx.tree.adaptive:
+            torch._foreach_zero_(Gs)
         fmmgb.fmm_m2l_adjoint_levels(ctx.tree, 2, ctx.p, Ws, Gs, conj=True)
         return (None, None, *Gs)
 

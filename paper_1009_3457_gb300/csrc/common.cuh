@@ -236,6 +236,8 @@ int launch_m2m(int child_level, int p, const float2* Mc, float2* Mp, bool accumu
 bool shift_supported(int p);
 int launch_shift(bool up, int child_level, int p, const float2* In, float2* Out, float scale, bool conj, bool acc,
                  cudaStream_t st);
+// launchers (farfield.cu)
+int launch_l2l(int child_level, int p, const float2* Lp, float2* Lc, bool acc, bool adjoint, cudaStream_t st);
 // FGT H2T on the tensor cores (fgt_h2t_tc.cu): p = 16, grid_log2 >= 3, n_cut <= 16
 bool fgt_h2t_tc_supported(int g, int ncut, int p);
 int launch_fgt_h2t_tc(int g, int ncut, double sigma, bool split, const float* A, float* Y, float* C, bool acc,

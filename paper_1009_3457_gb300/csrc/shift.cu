@@ -179,3 +179,36 @@ int launch_shift(bool up, int child_level, int p, const float2* In, float2* Out,
 }
 
 }  // namespace fmmgb
+
+using namespace fmmgb;
+
+// A whole pass of fmm_m2m (op 0), fmm_l2l_adjoint (1, accumulating), fmm_l2l (2, accumulating) or
+// fmm_m2m_adjoint (3, accumulating) over levels lmin..lmax, levels[i] the array of level lmin + i:
+// the same launches as the per-level calls, enqueued by one.  Used by the Python layer, whose calls
+// cost more than the coarse levels' kernels; not part of the public header.
+extern "C" int fmmgb_shift_levels(int32_t op, int32_t p, int32_t lmin, int32_t lmax, void* const* levels, void* stream)
+{
+    clear_error();
+    if (op < 0 || op > 3) return fail(FMM_EINVAL, "fmmgb_shift_levels: op %d", op);
+    if (lmin < 0 || lmax > FMM_MAX_LEVEL || lmin > lmax)
+        return fail(FMM_EINVAL, "fmmgb_shift_levels: levels %d..%d outside 0..%d", lmin, lmax, FMM_MAX_LEVEL);
+    if (p < 1 || p > 64) return fail(FMM_EINVAL, "fmmgb_shift_levels: p = %d outside 1..64", p);
+    if (!levels) return fail(FMM_EINVAL, "fmmgb_shift_levels: NULL level array");
+    for (int i = 0; i <= lmax - lmin; ++i)
+        if (!levels[i] || ((uintptr_t)levels[i] & 7))
+            return fail(FMM_EINVAL, "fmmgb_shift_levels: level %d NULL or misaligned", lmin + i);
+    const cudaStream_t st = (cudaStream_t)stream;
+    for (int k = 1; k <= lmax - lmin; ++k) {
+        const int l = op < 2 ? lmax + 1 - k : lmin + k;  // child level: finest first upward, last downward
+        float2 *child = (float2*)levels[l - lmin], *parent = (float2*)levels[l - 1 - lmin];
+        int rc = FMM_OK;
+        switch (op) {
+            case 0: rc = launch_m2m(l, p, child, parent, false, st); break;
+            case 1: rc = launch_l2l(l, p, child, parent, true, true, st); break;
+            case 2: rc = launch_l2l(l, p, parent, child, true, false, st); break;
+            default: rc = launch_m2m_adjoint(l, p, parent, child, true, st); break;
+        }
+        if (rc) return rc;
+    }
+    return FMM_OK;
+}

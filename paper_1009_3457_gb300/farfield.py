@@ -36,6 +36,18 @@ def leaf_boxes(tree, xy: torch.Tensor):
     return lev, box
 
 
+def _level_block(levels, p: int, device, zero: bool):
+    """One complex64 allocation for the [4^l, p] arrays of `levels`, and each level's address (a tensor
+    and an allocation per level cost the host more than the kernels they served)."""
+    sizes = [4 ** l * p for l in levels]
+    flat = (torch.zeros if zero else torch.empty)(sum(sizes), dtype=torch.complex64, device=device)
+    at, out = flat.data_ptr(), []
+    for n in sizes:
+        out.append(at)
+        at += 8 * n
+    return flat, out
+
+
 class FarFieldObjective(torch.autograd.Function):
     """J(xy) for fixed strengths, evaluation points and weights (see the module docstring)."""
 
@@ -43,17 +55,17 @@ class FarFieldObjective(torch.autograd.Function):
     def forward(ctx, xy, tree, p, c, zxy, zlev, zbox, w):
         L = tree.max_level
         dev = xy.device
+        st = fmmgb._stream(None)  # looked up once
         levels = list(range(2, L + 1))
-        Ms = [torch.empty((4 ** l, p), dtype=torch.complex64, device=dev) for l in levels]
-        fmmgb.fmm_p2m(L, p, xy, c, Ms[-1])  # finest level, then M2M upward (exact for truncated series)
-        for i in range(len(levels) - 1, 0, -1):
-            fmmgb.fmm_m2m(levels[i], p, Ms[i], Ms[i - 1])
-        Ls = [torch.zeros_like(M) for M in Ms]
-        fmmgb.fmm_m2l_levels(tree, 2, p, Ms, Ls)
-        for i in range(1, len(levels)):
-            fmmgb.fmm_l2l(levels[i], p, Ls[i - 1], Ls[i], accumulate=True)
+        mem_m, Ms = _level_block(levels, p, dev, zero=False)
+        fmmgb.fmm_p2m(L, p, xy, c, Ms[-1], stream=st)  # finest level, then M2M upward (exact for truncated series)
+        fmmgb._shift_levels(fmmgb.SHIFT_M2M, p, 2, Ms, st)
+        mem_l, Ls = _level_block(levels, p, dev, zero=tree.adaptive)  # M2L leaves absent boxes as they are
+        fmmgb.fmm_m2l_levels(tree, 2, p, Ms, Ls, stream=st)
+        fmmgb._shift_levels(fmmgb.SHIFT_L2L, p, 2, Ls, st)
         phi = torch.empty(zxy.shape[0], dtype=torch.complex64, device=dev)
-        fmmgb.fmm_l2p(p, zxy, zlev, zbox, dict(zip(levels, Ls)), L, phi)
+        fmmgb.fmm_l2p(p, zxy, zlev, zbox, dict(zip(levels, Ls)), L, phi, stream=st)
+        del mem_m, mem_l  # in use on the stream until here
         ctx.save_for_backward(xy, c, zxy, zlev, zbox, w)
         ctx.tree, ctx.p = tree, p
         return torch.sum(w * phi.real.to(torch.float64))
@@ -66,16 +78,16 @@ class FarFieldObjective(torch.autograd.Function):
         levels = list(range(2, L + 1))
         dev = xy.device
         cot = (gJ * w).to(torch.complex64)  # dJ/dphi (real weights)
-        Gs = [torch.zeros((4 ** l, p), dtype=torch.complex64, device=dev) for l in levels]
-        fmmgb.fmm_l2p_adjoint(p, zxy, zlev, zbox, cot, dict(zip(levels, Gs)), L)
-        for i in range(len(levels) - 1, 0, -1):
-            fmmgb.fmm_l2l_adjoint(levels[i], p, Gs[i], Gs[i - 1], accumulate=True)
-        Ws = [torch.zeros_like(G) for G in Gs]
-        fmmgb.fmm_m2l_adjoint_levels(tree, 2, p, Gs, Ws, conj=True)
-        for i in range(1, len(levels)):  # M_l = M2M(M_{l+1}): coarse to fine
-            fmmgb.fmm_m2m_adjoint(levels[i], p, Ws[i - 1], Ws[i], accumulate=True)
-        grad = torch.zeros_like(xy)
-        fmmgb.fmm_p2m_adjoint(L, p, xy, c, Ws[-1], grad)
+        st = fmmgb._stream(None)  # looked up once
+        mem_g, Gs = _level_block(levels, p, dev, zero=True)
+        fmmgb.fmm_l2p_adjoint(p, zxy, zlev, zbox, cot, dict(zip(levels, Gs)), L, stream=st)
+        fmmgb._shift_levels(fmmgb.SHIFT_L2L_ADJOINT, p, 2, Gs, st)
+        mem_w, Ws = _level_block(levels, p, dev, zero=tree.adaptive)
+        fmmgb.fmm_m2l_adjoint_levels(tree, 2, p, Gs, Ws, conj=True, stream=st)
+        fmmgb._shift_levels(fmmgb.SHIFT_M2M_ADJOINT, p, 2, Ws, st)  # M_l = M2M(M_{l+1}): coarse to fine
+        grad = torch.empty_like(xy)  # every point is written
+        fmmgb.fmm_p2m_adjoint(L, p, xy, c, Ws[-1], grad, stream=st)
+        del mem_g, mem_w
         return grad, None, None, None, None, None, None, None
 
 
@@ -117,34 +129,32 @@ class FmmPotential:
         dev = xy.device
         self.xy, self.c, self.z = xy.contiguous(), c.contiguous(), z.contiguous()
         self.levels = list(range(2, L + 1))
-        self.Ms = [torch.empty((4 ** l, p), dtype=torch.complex64, device=dev) for l in self.levels]
-        self.Ls = [torch.empty_like(M) for M in self.Ms]
-        nb = 4 ** L
-
-        def bins(pts):
-            perm = torch.empty(pts.shape[0], dtype=torch.int32, device=dev)
-            start = torch.empty(nb + 1, dtype=torch.int32, device=dev)
-            work = torch.empty(nb, dtype=torch.int32, device=dev)
-            fmmgb.fmm_bin_points(L, pts, perm, start, work)
-            return perm, start
-
-        self.sperm, self.sstart = bins(self.xy)
-        self.tperm, self.tstart = bins(self.z)
-        self.phi = torch.empty(self.z.shape[0], dtype=torch.complex64, device=dev)
+        # one allocation for the MEs and LEs, one for the binnings: a small problem's buffers cost the
+        # host more than its kernels
+        sizes = [4 ** l * p for l in self.levels]
+        flat = torch.empty(2 * sum(sizes), dtype=torch.complex64, device=dev).split(sizes + sizes)
+        arrays = [t.view(-1, p) for t in flat]
+        self.Ms, self.Ls = arrays[:len(sizes)], arrays[len(sizes):]
+        nb, n, nz = 4 ** L, self.xy.shape[0], self.z.shape[0]
+        self.sperm, self.sstart, self.tperm, self.tstart, work = torch.empty(
+            n + nz + 3 * nb + 2, dtype=torch.int32, device=dev).split([n, nb + 1, nz, nb + 1, nb])
+        st = fmmgb._stream(None)
+        fmmgb.fmm_bin_points(L, self.xy, self.sperm, self.sstart, work, stream=st)
+        fmmgb.fmm_bin_points(L, self.z, self.tperm, self.tstart, work, stream=st)
+        self.phi = torch.empty(nz, dtype=torch.complex64, device=dev)
         self.side = torch.cuda.Stream(device=dev)
 
     def __call__(self) -> torch.Tensor:
         p, L = self.p, self.L
         cur = torch.cuda.current_stream(self.phi.device)
+        st = fmmgb._stream(None)
         self.side.wait_stream(cur)  # the inputs and phi are the current stream's until here
         fmmgb.fmm_p2p(L, self.xy, self.c, self.sperm, self.sstart, self.z, self.tperm, self.tstart, self.phi,
                       stream=self.side, share_sm=True)
-        fmmgb.fmm_p2m_binned(L, p, self.xy, self.c, self.sperm, self.sstart, self.Ms[-1])
-        for i in range(len(self.levels) - 1, 0, -1):
-            fmmgb.fmm_m2m(self.levels[i], p, self.Ms[i], self.Ms[i - 1])
-        fmmgb.fmm_m2l_levels(self.tree, 2, p, self.Ms, self.Ls, prec=self.prec)
-        for i in range(1, len(self.levels)):
-            fmmgb.fmm_l2l(self.levels[i], p, self.Ls[i - 1], self.Ls[i], accumulate=True)
+        fmmgb.fmm_p2m_binned(L, p, self.xy, self.c, self.sperm, self.sstart, self.Ms[-1], stream=st)
+        fmmgb._shift_levels(fmmgb.SHIFT_M2M, p, 2, self.Ms, st)
+        fmmgb.fmm_m2l_levels(self.tree, 2, p, self.Ms, self.Ls, prec=self.prec, stream=st)
+        fmmgb._shift_levels(fmmgb.SHIFT_L2L, p, 2, self.Ls, st)
         cur.wait_stream(self.side)
-        fmmgb.fmm_l2p_binned(L, p, self.z, self.tperm, self.tstart, self.Ls[-1], self.phi, accumulate=True)
+        fmmgb.fmm_l2p_binned(L, p, self.z, self.tperm, self.tstart, self.Ls[-1], self.phi, accumulate=True, stream=st)
         return self.phi

@@ -98,7 +98,8 @@ _i64 = ctypes.c_int64
 _d = ctypes.c_double
 _f = ctypes.c_float
 
-# name -> (restype, argtypes); the list of exported entry points of include/fmmgb.h
+# name -> (restype, argtypes); the list of exported entry points of include/fmmgb.h, and
+# fmmgb_shift_levels, which serves _shift_levels below
 SIGNATURES = {
     "fmm_build_lists": (ctypes.c_int, [_vp, _i64, _i32, _i32, _i32, ctypes.POINTER(_vp)]),
     "fmm_tree_level_info": (ctypes.c_int, [_vp, _i32, ctypes.POINTER(fmm_level_info)]),
@@ -145,6 +146,7 @@ SIGNATURES = {
     "fmm_p2p": (ctypes.c_int, [_i32, _vp, _vp, _i64, _vp, _vp, _vp, _i64, _vp, _vp, _vp, _i32, _vp]),
     "fgt_p2h_binned": (ctypes.c_int, [_i32, _i32, _d, _vp, _vp, _i64, _vp, _vp, _i32, _vp]),
     "fgt_h2p": (ctypes.c_int, [_i32, _i32, _i32, _i32, _d, _vp, _vp, _i64, _vp, _vp, _vp, _i32, _vp]),
+    "fmmgb_shift_levels": (ctypes.c_int, [_i32, _i32, _i32, _i32, ctypes.POINTER(_vp), _vp]),
     "fmm_wait_probe": (ctypes.c_int, [_i32, _i32, _vp]),
     "fmm_sync_status": (ctypes.c_int, [_vp]),
     "fmm_last_error": (ctypes.c_char_p, []),
@@ -189,11 +191,16 @@ def _ptr(t) -> int:
     return t.data_ptr()
 
 
+_torch = None
+
+
 def _stream(stream):
     if stream is None:
-        import torch
-
-        return torch.cuda.current_stream().cuda_stream
+        # the current stream's handle, without building the Python object around it
+        global _torch
+        if _torch is None:
+            import torch as _torch
+        return _torch._C._cuda_getCurrentRawStream(_torch.cuda.current_device())
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
@@ -436,6 +443,15 @@ def fmm_l2l(child_level: int, p: int, Lp, Lc, accumulate: bool = False, stream=N
 def fmm_l2l_adjoint(child_level: int, p: int, Wc, Wp, accumulate: bool = False, stream=None):
     _check(load().fmm_l2l_adjoint(child_level, p, _ptr(Wc), _ptr(Wp), FMM_ACCUMULATE if accumulate else 0,
                                   _stream(stream)))
+
+
+SHIFT_M2M, SHIFT_L2L_ADJOINT, SHIFT_L2L, SHIFT_M2M_ADJOINT = range(4)
+
+
+def _shift_levels(op: int, p: int, lmin: int, arrays, stream):
+    """fmm_m2m, or fmm_l2l_adjoint, fmm_l2l, fmm_m2m_adjoint accumulating, from each of the levels
+    lmin.. (one array each, finest last) to the next, in one call."""
+    _check(load().fmmgb_shift_levels(op, p, lmin, lmin + len(arrays) - 1, _ptr_array(arrays), _stream(stream)))
 
 
 def _level_table(arrays, max_level):
