@@ -9,14 +9,18 @@
 // centre in box sides (read off the bits of the FP64 position, kept in FP32)
 // and strength, so a box's sources are one contiguous range and staging adds
 // only the exact offset between box centres (-1, 0 or 1) -- no FP64
-// arithmetic per staged source or per claim.  Persistent CTAs of 128 threads claim runs of up to 96 targets of
-// one box from a claim table (a finest-level box holds a few dozen points, so
-// nearly every box is one claim), gather the sources of the 3 x 3
-// neighbourhood into shared memory in batches -- position relative to the
-// target box's centre and strength -- and each warp sums the run's targets
-// (one to three rows of 32, as many as the run fills, one target per lane and
-// row) against a quarter of every batch; the four partial sums of a target
-// meet in shared memory.  In FP32:
+// arithmetic per staged source or per claim.  Runs of targets of one box are
+// claimed from a table; two kernels take them:
+//   - fmm_p2p_kernel, dense boxes or few of them: a CTA of 128 threads a claim of
+//     up to 96 targets.  It gathers the sources of the 3 x 3 neighbourhood
+//     into shared memory in batches, and each warp sums the run's targets (one to
+//     three rows of 32, as many as the run fills, one target per lane and row)
+//     against a quarter of every batch; the four partial sums of a target meet in
+//     shared memory;
+//   - fmm_p2p_warp_kernel, many sparse boxes: a warp a claim of up to 64 targets, eight
+//     lanes for the targets and four for the sources, so that a run of 16 targets
+//     fills the warp (a row of 32 lanes was half empty), and no barrier.
+// In FP32:
 //   1/(dx + i dy) = (dx - i dy) / r2 with one approximate reciprocal per pair,
 // dx, dy in box sides, and the sums scaled by 2^level (exact) at the end.
 // Positions relative to the target box keep |dx|, |dy| <= 1.5 box sides, so
@@ -35,6 +39,19 @@ constexpr int kP2pR = 3;                        // targets per lane (rows of 32 
 constexpr int kP2pRun = 32 * kP2pR;             // targets per claim
 constexpr int kP2pBatch = 1024;                 // sources per shared-memory batch
 constexpr int kP2pSharedCtas = 8;               // resident CTAs per SM with FMM_P2P_SHARE_SM
+// The warp kernel takes calls of fewer than kP2pDense targets a box on average, on kP2wBoxes boxes or
+// more (fewer claims than warps otherwise).  us, CTA / warp: 16 a box at level 5 26 / 35, level 6 31 / 35,
+// level 7 68 / 62, level 8 216 / 170, level 9 914 / 676; 32 a box at level 6 41 / 55, level 7 105 / 110,
+// level 8 374 / 344; 64 a box at level 8 931 / 1,038.
+constexpr int kP2pDense = 32, kP2wBoxes = 1 << 14;
+// the warp kernel
+constexpr int kP2wLanes = 8;                    // target lanes; the other factor 4 splits the sources
+constexpr int kP2wSplit = 32 / kP2wLanes;
+constexpr int kP2wPairs = 4;                    // packed target pairs per lane, at most
+constexpr int kP2wRun = 2 * kP2wLanes * kP2wPairs;  // targets per claim
+constexpr int kP2wChunk = 96;                   // sources per staging buffer of a warp
+constexpr int kP2wCtas = 7;                     // resident CTAs per SM (72 registers)
+constexpr int kP2wSharedCtas = 6;               // ... with FMM_P2P_SHARE_SM
 // added to every r^2 (in box sides squared): a source at the target's position
 // (dx = dy = 0) then contributes exactly 0 -- c / 1e-30 is finite for |c| < 3e8 -- and
 // any other pair changes by a relative 1e-30 / r^2 (below FP32 rounding for distances
@@ -51,8 +68,8 @@ struct P2pArgs {
     const double* z;
     const int* tperm;
     const int* tstart;
-    const int* claims;
-    const int4* tab;  // claim table (p2p_claim_table_kernel), ntab entries
+    const int* nclaim;  // claims in the table
+    const int4* tab;    // claim table (p2p_claim_table_kernel), room for ntab entries
     int ntab;
     float2* phi;
     int* cursor;  // [0] next claim index, [1] CTAs finished
@@ -112,6 +129,12 @@ __device__ __forceinline__ unsigned long long p2_sub(unsigned long long a, unsig
 {
     unsigned long long d;
     asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ unsigned long long p2_add(unsigned long long a, unsigned long long b)
+{
+    unsigned long long d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
     return d;
 }
 __device__ __forceinline__ unsigned long long p2_mul(unsigned long long a, unsigned long long b)
@@ -178,27 +201,44 @@ __device__ __forceinline__ void p2p_batch(const float4* __restrict__ s_src, int 
     }
 }
 
-// Claim table: entry k = (first, end, box) of the k-th run of at most kP2pRun
-// targets of one box (the runs of box b are claims[b] .. claims[b+1]-1), so a
-// CTA finds its claim with one load instead of a binary search over the boxes.
-// Runs past `cap` entries, or a box_start that does not bin [0, nz), set the
-// error word (the kernel then skips those runs).
-__global__ void p2p_claim_table_kernel(int nbox, const int* __restrict__ claims, const int* __restrict__ tstart,
-                                       int nz, int cap, int4* __restrict__ tab, int* err)
+// Claim table: one entry (first, end, box) per run of targets of one box, a box's targets cut
+// into equal runs of at most `most`.  The runs of a warp's 32 boxes take consecutive places
+// from one addition to *nclaim (zero before); the order of the table only sets the order in
+// which claims are taken.  Places past `cap`, or a box_start that does not bin [0, nz), set the
+// error word (and those runs are skipped).  (A scan of the boxes' counts by one block, to give every
+// run a place of its own, took 73 us at 256 x 256 boxes and 290 us at 512 x 512.)
+__global__ void p2p_claim_table_kernel(int nbox, const int* __restrict__ tstart, int nz, int most, int cap,
+                                       int* nclaim, int4* __restrict__ tab, int* err)
 {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= nbox) return;
-    const int c0 = claims[b], c1 = claims[b + 1];
-    const int f0 = tstart[b], e0 = min(tstart[b + 1], nz);
-    for (int k = c0; k < c1; ++k) {
-        if (k < 0 || k >= cap) {
+    const int b = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
+    int f = 0, e = 0, n = 0;
+    if (b < nbox) {
+        f = tstart[b];
+        e = tstart[b + 1];
+        if (f < 0 || e > nz || f > e) {
+            atomicOr(err, DEV_ERR_CHECK);
+            e = min(e, nz);
+            if (f < 0 || f > e) f = e = 0;
+        }
+        n = (e - f + most - 1) / most;
+    }
+    int x = n;  // inclusive scan over the warp
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += t;
+    }
+    int at = 0;
+    if (lane == 31 && x > 0) at = atomicAdd(nclaim, x);
+    at = __shfl_sync(0xffffffffu, at, 31) + x - n;
+    if (n <= 0) return;
+    const int run = (e - f + n - 1) / n;
+    for (int k = 0; k < n; ++k) {
+        if ((unsigned)(at + k) >= (unsigned)cap) {
             atomicOr(err, DEV_ERR_CHECK);
             return;
         }
-        const int f = f0 + (k - c0) * kP2pRun, e = min(f + kP2pRun, e0);
-        const bool ok = 0 <= f && f < e;
-        if (!ok) atomicOr(err, DEV_ERR_CHECK);
-        tab[k] = ok ? make_int4(f, e, b, 0) : make_int4(0, 0, b, 0);
+        tab[at + k] = make_int4(f + k * run, min(f + (k + 1) * run, e), b, 0);
     }
 }
 
@@ -212,7 +252,7 @@ __global__ void __launch_bounds__(kP2pThreads) fmm_p2p_kernel(P2pArgs a)
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int side = 1 << a.level;
-    const int total = min(__ldg(a.claims + (side * side)), a.ntab);
+    const int total = min(__ldg(a.nclaim), a.ntab);
     // thread 0 fetches the index of the CTA's next claim one claim ahead
     int knext = tid == 0 ? atomicAdd(a.cursor, 1) : 0;
 
@@ -344,6 +384,167 @@ __global__ void __launch_bounds__(kP2pThreads) fmm_p2p_kernel(P2pArgs a)
     }
 }
 
+__device__ __forceinline__ void p2p_copy16(void* smem, const void* gmem)
+{
+    const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(gmem) : "memory");
+}
+
+// A warp's claim: m <= 16 NP targets of box (tx, ty) from place `first` on, against the 3 x 3
+// neighbourhood, lane q < 9 holding box q's first sorted source b0 and count n.  A lane keeps 2 NP
+// targets as packed pairs (dx, dy, r^2, the weight and both sums in f32x2 operations, the two
+// reciprocals scalar) and takes every fourth source.  A box's sources are one run of the sorted
+// array; the warp copies them into one of its two buffers asynchronously while it sums the other.
+// im sums +w dy.
+template <int NP>
+__device__ __forceinline__ void p2p_claim(const P2pArgs& a, int first, int m, int tx, int ty, int b0, int n,
+                                          float4* buf)
+{
+    const int lane = threadIdx.x & 31, tl = lane & (kP2wLanes - 1), sl = lane / kP2wLanes;
+    const int side = 1 << a.level;
+    unsigned long long zx[NP], zy[NP], re[NP], im[NP];
+    auto target = [&](int k) {  // index of the lane's target k (-1: none)
+        const int t = kP2wLanes * k + tl;
+        const int j = t < m ? __ldg(a.tperm + first + t) : -1;
+        return (unsigned)j < (unsigned)a.nz ? j : -1;
+    };
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+        float2 z[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int j = target(2 * p + h);
+            z[h] = make_float2(0.f, 0.f);
+            if (j < 0) {
+                if (kP2wLanes * (2 * p + h) + tl < m) atomicOr(a.err, DEV_ERR_CHECK);
+                continue;
+            }
+            const double x = __ldg(a.z + 2 * (size_t)j), y = __ldg(a.z + 2 * (size_t)j + 1);
+            long long X, Y;
+            if (grid_fixed31(x, a.level, X) && grid_fixed31(y, a.level, Y) && (int)(X >> 31) == tx &&
+                (int)(Y >> 31) == ty) {
+                z[h] = make_float2(cell_offset31(X), cell_offset31(Y));  // in the claimed box: no FP64 arithmetic
+            } else {  // outside it (coordinates outside the unit square): FP64, x 2^level exact
+                z[h] = make_float2((float)(x * side - (tx + 0.5)), (float)(y * side - (ty + 0.5)));
+            }
+        }
+        zx[p] = p2_pk(z[0].x, z[1].x);
+        zy[p] = p2_pk(z[0].y, z[1].y);
+        re[p] = im[p] = 0ull;
+    }
+    const unsigned long long tiny = p2_pk(kP2pTiny, kP2pTiny);
+    // the neighbourhood's sources, box by box in pieces of up to kP2wChunk: piece [at, at + cnt) of box q
+    int q = -1, at = 0, s1 = 0, cnt = 0;
+    float ox = 0.f, oy = 0.f;
+    auto next = [&](float4* buf) {  // the next piece, its copies issued (one group, empty past the end)
+        at += cnt;
+        while (at >= s1 && q < 8) {
+            ++q;
+            at = __shfl_sync(0xffffffffu, b0, q);
+            s1 = at + __shfl_sync(0xffffffffu, n, q);
+        }
+        cnt = min(kP2wChunk, s1 - at);
+        ox = (float)(q % 3 - 1);  // the box's centre from the target box's
+        oy = (float)(q / 3 - 1);
+        for (int i = lane; i < cnt; i += 32) p2p_copy16(buf + i, a.src + at + i);
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+    };
+    next(buf);
+    for (int k = 0; cnt > 0; k ^= 1) {
+        const float4* cur = buf + k * kP2wChunk;
+        const int m0 = cnt;
+        const float cx = -ox, cy = -oy;
+        next(buf + (k ^ 1) * kP2wChunk);
+        asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+        __syncwarp();
+#pragma unroll 2
+        for (int i = sl; i < m0; i += kP2wSplit) {
+            const float4 u = cur[i];
+            const float x = cx - u.x, y = cy - u.y;
+            const unsigned long long vx = p2_pk(x, x), vy = p2_pk(y, y), c = p2_pk(u.z, u.z);
+#pragma unroll
+            for (int p = 0; p < NP; ++p) {
+                const unsigned long long dx = p2_add(zx[p], vx), dy = p2_add(zy[p], vy);
+                const float2 r2 = p2_upk(p2_fma(dx, dx, p2_fma(dy, dy, tiny)));
+                const unsigned long long w = p2_mul(c, p2_pk(rcp_approx(r2.x), rcp_approx(r2.y)));
+                re[p] = p2_fma(w, dx, re[p]);
+                im[p] = p2_fma(w, dy, im[p]);
+            }
+        }
+        __syncwarp();  // the buffer has been read
+    }
+    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+        const float2 r = p2_upk(re[p]), i = p2_upk(im[p]);
+        float v[4] = {r.x, i.x, r.y, i.y};
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+#pragma unroll
+            for (int o = kP2wLanes; o < 32; o <<= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            if (sl != (2 * p + h) % kP2wSplit) continue;  // the source lanes share the stores
+            const int j = target(2 * p + h);
+            if (j < 0) continue;
+            // 1/(z - y) = 2^level / ((z - y) in box sides): exact scaling
+            float2 o = make_float2(v[2 * h] * (float)side, -v[2 * h + 1] * (float)side);
+            if (a.accumulate) {
+                const float2 old = a.phi[j];
+                o.x += old.x;
+                o.y += old.y;
+            }
+            a.phi[j] = o;
+        }
+    }
+}
+
+__global__ void __launch_bounds__(kP2pThreads, kP2wCtas) fmm_p2p_warp_kernel(P2pArgs a)
+{
+    __shared__ float4 s_src[kP2pThreads / 32][2 * kP2wChunk];  // two staging buffers a warp
+    const int lane = threadIdx.x & 31;
+    float4* buf = s_src[threadIdx.x >> 5];
+    const int side = 1 << a.level;
+    const int total = min(__ldg(a.nclaim), a.ntab);
+    // lane 0 fetches the index of the warp's next claim one claim ahead
+    int knext = lane == 0 ? atomicAdd(a.cursor, 1) : 0;
+    for (;;) {
+        const int k = __shfl_sync(0xffffffffu, knext, 0);
+        if (k >= total) break;
+        if (lane == 0) knext = atomicAdd(a.cursor, 1);
+        const int4 cl = __ldg(a.tab + k);
+        const int first = cl.x, m = cl.y - cl.x, box = cl.z;
+        const int tx = box & (side - 1), ty = box >> a.level;
+        int b0 = 0, n = 0;
+        if (lane < 9) {  // the 3 x 3 neighbourhood, one box per lane
+            const int sx = tx + lane % 3 - 1, sy = ty + lane / 3 - 1;
+            if (sx >= 0 && sy >= 0 && sx < side && sy < side) {
+                const int b = sy * side + sx;
+                b0 = __ldg(a.sstart + b);
+                n = __ldg(a.sstart + b + 1) - b0;
+                if (n < 0 || b0 < 0 || b0 + n > a.n) {
+                    atomicOr(a.err, DEV_ERR_CHECK);
+                    b0 = n = 0;
+                }
+            }
+        }
+        switch ((m + 2 * kP2wLanes - 1) / (2 * kP2wLanes)) {
+            case 1: p2p_claim<1>(a, first, m, tx, ty, b0, n, buf); break;
+            case 2: p2p_claim<2>(a, first, m, tx, ty, b0, n, buf); break;
+            case 3: p2p_claim<3>(a, first, m, tx, ty, b0, n, buf); break;
+            default: p2p_claim<4>(a, first, m, tx, ty, b0, n, buf); break;
+        }
+    }
+    // the last warp to finish returns the cursor slot to zero for its next use
+    if (lane == 0) {
+        __threadfence();
+        if (atomicAdd(a.cursor + 1, 1) == (int)gridDim.x * (kP2pThreads / 32) - 1) {
+            atomicExch(a.cursor, 0);
+            atomicExch(a.cursor + 1, 0);
+        }
+    }
+}
+
 // Per-device buffer of sorted sources (grown on demand).
 static std::mutex g_src_mu;
 static float4* g_src[64];
@@ -405,19 +606,19 @@ extern "C" int fmm_p2p(int32_t level, const double* xy, const double* c, int64_t
     args.phi = reinterpret_cast<float2*>(phi);
     if (int rc = tile_counter(&args.cursor, st)) return rc;
     if (int rc = device_error_word(&args.err)) return rc;
-    unsigned char* scratch = nullptr;
-    if (int rc = fgt_flag_buffer(&scratch)) return rc;
-    int* claims = reinterpret_cast<int*>(scratch + kFgtFlagBytes);
-    args.claims = claims;
     const int nbox = 1 << (2 * level);
-    if (int rc = launch_h2p_claims(nbox, tgt_start, kP2pRun, claims, args.err, st)) return rc;
-    // one buffer: the sources in box order, then the claim table
-    const int64_t most = nz / kP2pRun + nbox;  // claims can be no more
+    const bool dense = nz >= (int64_t)kP2pDense * nbox || nbox < kP2wBoxes;
+    const int run = dense ? kP2pRun : kP2wRun;
+    // one buffer: the sources in box order, the claim table, the number of claims
+    const int64_t most = nz / run + nbox;  // claims can be no more
     float4* src = nullptr;
-    if (int rc = p2p_source_buffer((size_t)(n + most) * sizeof(float4), &src)) return rc;
+    if (int rc = p2p_source_buffer((size_t)(n + most + 1) * sizeof(float4), &src)) return rc;
     int4* tab = reinterpret_cast<int4*>(src + n);
-    p2p_claim_table_kernel<<<(unsigned)((nbox + 255) / 256), 256, 0, st>>>(nbox, claims, tgt_start, (int)nz, (int)most,
-                                                                          tab, args.err);
+    int* nclaim = reinterpret_cast<int*>(tab + most);
+    args.nclaim = nclaim;
+    FMM_CUDA_TRY(cudaMemsetAsync(nclaim, 0, sizeof(int), st));
+    p2p_claim_table_kernel<<<(unsigned)((nbox + 255) / 256), 256, 0, st>>>(nbox, tgt_start, (int)nz, run, (int)most,
+                                                                          nclaim, tab, args.err);
     FMM_CUDA_TRY(cudaGetLastError());
     if (n > 0) {
         p2p_sort_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(level, xy, c, src_perm, (int)n, src, args.err);
@@ -426,23 +627,28 @@ extern "C" int fmm_p2p(int32_t level, const double* xy, const double* c, int64_t
     args.src = src;
     args.tab = tab;
     args.ntab = (int)most;
-    static int occ;
+    static int occ_cache[2];
     static std::mutex mu;
+    auto kern = dense ? fmm_p2p_kernel : fmm_p2p_warp_kernel;
+    int occ = 0;
     {
         std::lock_guard<std::mutex> lk(mu);
-        if (!occ) {
-            FMM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fmm_p2p_kernel, kP2pThreads, 0));
-            if (occ < 1) occ = 1;
+        int& o = occ_cache[dense];
+        if (!o) {
+            FMM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, kern, kP2pThreads, 0));
+            if (o < 1) o = 1;
         }
+        occ = o;
     }
     int sms = 0;
     if (int rc = device_sm_count(&sms)) return rc;
     // sharing the SMs with kernels of other streams: 8 CTAs (132 KB of shared memory, 1,024
     // threads) per SM measured 1.5 % slower alone than the occupancy limit, and left room for
     // the far field of the same FMM beside it (fewer starved the near field itself)
-    const int per_sm = (flags & FMM_P2P_SHARE_SM) ? std::min(occ, kP2pSharedCtas) : occ;
-    const int grid = (int)std::min<int64_t>((int64_t)per_sm * sms, most);
-    fmm_p2p_kernel<<<grid, kP2pThreads, 0, st>>>(args);
+    const int per_sm = (flags & FMM_P2P_SHARE_SM) ? std::min(occ, dense ? kP2pSharedCtas : kP2wSharedCtas) : occ;
+    const int64_t ctas = dense ? most : (most + kP2pThreads / 32 - 1) / (kP2pThreads / 32);
+    const int grid = (int)std::min<int64_t>((int64_t)per_sm * sms, ctas);
+    kern<<<grid, kP2pThreads, 0, st>>>(args);
     FMM_CUDA_TRY(cudaGetLastError());
     return FMM_OK;
 }

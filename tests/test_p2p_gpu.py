@@ -192,3 +192,28 @@ def test_p2m_binned_matches_oracle_and_repeats_exactly(fmm, orc, p):
         again = M.clone()
         fmm.fmm_p2m_binned(level, p, xyd, cd, perm, start, M)
         assert torch.equal(again, M)
+
+
+@pytest.mark.parametrize("level,per_box", [(6, 8), (7, 0.5), (7, 8), (7, 31.9), (7, 32), (8, 8)])
+def test_p2p_sparse_and_dense_claims(fmm, orc, level, per_box):
+    """Both sides of the line between a CTA and a warp per claim (boxes, targets per box), with one
+    box of thousands of targets and sources (several runs of targets, several pieces of sources),
+    empty boxes, and accumulation; 900 targets against the oracle."""
+    import torch
+
+    nb = 4 ** level
+    rng = np.random.default_rng(int(level * 100 + per_box))
+    nz = int(per_box * nb)
+    crowd = min(1500, nz // 4)
+    z = np.concatenate([rng.random((nz - crowd, 2)), 0.37 + 0.9 * 0.5 ** level * rng.random((crowd, 2))])
+    xy = np.concatenate([rng.random((30000, 2)), 0.37 + 0.9 * 0.5 ** level * rng.random((1000, 2))])
+    c = rng.uniform(-1, 1, len(xy))
+    pick = np.concatenate([rng.choice(nz, 600, replace=False), nz - crowd + rng.choice(crowd, 300, replace=False)])
+    phi0 = rng.standard_normal(nz) + 1j * rng.standard_normal(nz)
+    zz = z[:, 0] + 1j * z[:, 1]
+    ref = orc.p2p_uniform(level, xy, c, zz[pick])
+    # ~1000 sources in one box: the closest pair lies ~1e-3 box sides away (the bar of the coarse levels)
+    got = _p2p(fmm, level, xy, c, zz, phi0=phi0)[pick] - phi0.astype(np.complex64)[pick]
+    scale = np.abs(phi0[pick]) + np.abs(ref)
+    assert np.linalg.norm(got - ref) <= 1e-4 * np.linalg.norm(ref)
+    assert (np.abs(got - ref) <= 2e-4 * np.abs(ref).max() + 1e-6 * scale).all()
