@@ -20,13 +20,17 @@
 // launch at the coarse ones.  A 9-level tree at p = 16, seven launches a pass: M2M and L2L's transpose
 // together 253 -> 52 us, L2L and M2M's transpose 207 -> 58 us (a thread per output with its own
 // powers of z and a table read per term before).
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace fmmgb {
 
-template <int P>
+constexpr int kShiftThreads = 128;   // per block, at most
+constexpr int kChainThreads = 1024;  // of a chain's CTAs
+template <int P, int NT>
 struct ShiftCfg {
-    static constexpr int BOXES = 128 / P;           // parents per block
+    static constexpr int BOXES = NT / P;            // parents per block
     static constexpr int THREADS = BOXES * P;
     static constexpr int ROW = P + 1;               // float2 row stride in shared memory
 };
@@ -46,18 +50,23 @@ __device__ __forceinline__ void shift_coefficients(float (*s)[P + 1], float scal
 __device__ __forceinline__ int child_x(int t) { return t == 0 || t == 3; }
 __device__ __forceinline__ int child_y(int t) { return t < 2; }
 
-// Out[parent][j] (+)= sum_t sum_k c_jk (z_t or conj z_t)^(j-k) In[child t][k]
-template <int P>
-__global__ void __launch_bounds__(ShiftCfg<P>::THREADS)
-    shift_up_kernel(int child_level, const float2* __restrict__ In, float2* __restrict__ Out, float scale, int conj,
-                    int accumulate)
+// Shared memory of a block: the coefficients and the rows that its threads exchange.
+template <int P, int NT>
+struct ShiftSmem {
+    float c[P][P + 1];
+    float2 d[ShiftCfg<P, NT>::BOXES][4][ShiftCfg<P, NT>::ROW];
+};
+
+// One block of parents: Out[parent][j] (+)= sum_t sum_k c_jk (z_t or conj z_t)^(j-k) In[child t][k].
+// Loads go to the L2: in a chain of levels another block has just written them.
+template <int P, int NT>
+__device__ __forceinline__ void shift_up_block(ShiftSmem<P, NT>& sm, int child_level, const float2* In, float2* Out, int conj,
+                                               int accumulate, int64_t block)
 {
-    using C = ShiftCfg<P>;
-    __shared__ float s_c[P][P + 1];
-    __shared__ float2 s_d[C::BOXES][4][C::ROW];
+    using C = ShiftCfg<P, NT>;
     const int np = 1 << (child_level - 1), nc = 2 * np;
     const int pl = threadIdx.x / P, j = threadIdx.x % P;
-    const int64_t pb = (int64_t)blockIdx.x * C::BOXES + pl;
+    const int64_t pb = block * C::BOXES + pl;
     const bool ok = pb < (int64_t)np * np;
     float2 m[4];
 #pragma unroll
@@ -65,21 +74,20 @@ __global__ void __launch_bounds__(ShiftCfg<P>::THREADS)
         m[t] = make_float2(0.f, 0.f);
         if (ok) {
             const int px = (int)(pb & (np - 1)), py = (int)(pb >> (child_level - 1));
-            m[t] = __ldg(In + ((size_t)(2 * py + (child_y(t) ^ conj)) * nc + 2 * px + child_x(t)) * P + j);
+            m[t] = __ldcg(In + ((size_t)(2 * py + (child_y(t) ^ conj)) * nc + 2 * px + child_x(t)) * P + j);
         }
     }
     float2 old = make_float2(0.f, 0.f);
-    if (ok && accumulate) old = Out[(size_t)pb * P + j];
-    shift_coefficients<P>(s_c, scale, C::THREADS);
+    if (ok && accumulate) old = __ldcg(Out + (size_t)pb * P + j);
     {
         const float2 e = make_float2(m[0].x + m[2].x, m[0].y + m[2].y), f = make_float2(m[1].x + m[3].x, m[1].y + m[3].y);
         const float2 o = make_float2(m[0].x - m[2].x, m[0].y - m[2].y), g = make_float2(m[1].x - m[3].x, m[1].y - m[3].y);
         const float x1 = o.x - g.y, y1 = o.y + g.x, x3 = o.x + g.y, y3 = o.y - g.x;  // sums of i^t m, (-i)^t m
         const float x2 = e.x - f.x, y2 = e.y - f.y;
-        s_d[pl][0][j] = make_float2(e.x + f.x, e.y + f.y);
-        s_d[pl][1][j] = make_float2(x1 - y1, x1 + y1);
-        s_d[pl][2][j] = make_float2(-2.f * y2, 2.f * x2);
-        s_d[pl][3][j] = make_float2(-2.f * (x3 + y3), 2.f * (x3 - y3));
+        sm.d[pl][0][j] = make_float2(e.x + f.x, e.y + f.y);
+        sm.d[pl][1][j] = make_float2(x1 - y1, x1 + y1);
+        sm.d[pl][2][j] = make_float2(-2.f * y2, 2.f * x2);
+        sm.d[pl][3][j] = make_float2(-2.f * (x3 + y3), 2.f * (x3 - y3));
     }
     __syncthreads();
     if (!ok) return;
@@ -87,8 +95,8 @@ __global__ void __launch_bounds__(ShiftCfg<P>::THREADS)
 #pragma unroll
     for (int k = 0; k < P; ++k)
         if (k <= j) {
-            const float2 d = s_d[pl][(j - k) & 3][k];
-            const float c = s_c[k][j];
+            const float2 d = sm.d[pl][(j - k) & 3][k];
+            const float c = sm.c[k][j];
             s.x = fmaf(c, d.x, s.x);
             s.y = fmaf(c, d.y, s.y);
         }
@@ -99,18 +107,15 @@ __global__ void __launch_bounds__(ShiftCfg<P>::THREADS)
     Out[(size_t)pb * P + j] = s;
 }
 
-// Out[child t][j] (+)= sum_(n >= j) c_nj (z_t or conj z_t)^(n-j) In[parent][n]
-template <int P>
-__global__ void __launch_bounds__(ShiftCfg<P>::THREADS)
-    shift_down_kernel(int child_level, const float2* __restrict__ In, float2* __restrict__ Out, float scale, int conj,
-                      int accumulate)
+// One block of parents: Out[child t][j] (+)= sum_(n >= j) c_nj (z_t or conj z_t)^(n-j) In[parent][n].
+template <int P, int NT>
+__device__ __forceinline__ void shift_down_block(ShiftSmem<P, NT>& sm, int child_level, const float2* In, float2* Out,
+                                                 int conj, int accumulate, int64_t block)
 {
-    using C = ShiftCfg<P>;
-    __shared__ float s_c[P][P + 1];
-    __shared__ float2 s_l[C::BOXES][C::ROW];
+    using C = ShiftCfg<P, NT>;
     const int np = 1 << (child_level - 1), nc = 2 * np;
     const int pl = threadIdx.x / P, j = threadIdx.x % P;
-    const int64_t pb = (int64_t)blockIdx.x * C::BOXES + pl;
+    const int64_t pb = block * C::BOXES + pl;
     const bool ok = pb < (int64_t)np * np;
     float2* out[4];
     float2 old[4];
@@ -119,10 +124,9 @@ __global__ void __launch_bounds__(ShiftCfg<P>::THREADS)
     for (int t = 0; t < 4; ++t) {
         out[t] = Out + ((size_t)(2 * py + (child_y(t) ^ conj)) * nc + 2 * px + child_x(t)) * P + j;
         old[t] = make_float2(0.f, 0.f);
-        if (ok && accumulate) old[t] = *out[t];
+        if (ok && accumulate) old[t] = __ldcg(out[t]);
     }
-    s_l[pl][j] = ok ? __ldg(In + (size_t)pb * P + j) : make_float2(0.f, 0.f);
-    shift_coefficients<P>(s_c, scale, C::THREADS);
+    sm.d[pl][0][j] = ok ? __ldcg(In + (size_t)pb * P + j) : make_float2(0.f, 0.f);
     __syncthreads();
     if (!ok) return;
     float2 b[4];
@@ -131,8 +135,8 @@ __global__ void __launch_bounds__(ShiftCfg<P>::THREADS)
 #pragma unroll
     for (int q = 0; q < P; ++q)
         if (j + q < P) {
-            const float2 l = s_l[pl][j + q];
-            const float c = s_c[j][j + q];
+            const float2 l = sm.d[pl][0][j + q];
+            const float c = sm.c[j][j + q];
             b[q & 3].x = fmaf(c, l.x, b[q & 3].x);
             b[q & 3].y = fmaf(c, l.y, b[q & 3].y);
         }
@@ -147,17 +151,73 @@ __global__ void __launch_bounds__(ShiftCfg<P>::THREADS)
     for (int t = 0; t < 4; ++t) *out[t] = make_float2(r[t].x + old[t].x, r[t].y + old[t].y);
 }
 
+template <int P, bool UP>
+__global__ void __launch_bounds__(kShiftThreads)
+    shift_kernel(int child_level, const float2* In, float2* Out, float scale, int conj, int accumulate)
+{
+    __shared__ ShiftSmem<P, kShiftThreads> sm;
+    shift_coefficients<P>(sm.c, scale, ShiftCfg<P, kShiftThreads>::THREADS);
+    // visible to the block at the barrier inside
+    if constexpr (UP)
+        shift_up_block<P>(sm, child_level, In, Out, conj, accumulate, blockIdx.x);
+    else
+        shift_down_block<P>(sm, child_level, In, Out, conj, accumulate, blockIdx.x);
+}
+
+// A run of levels in one launch: one cluster of CTAs takes the blocks of each level in turn, with a
+// cluster barrier (release / acquire) between the levels.  For the coarse levels, where a launch
+// costs more than the level: child levels up to kChainMax (4,096 boxes: two rounds of the cluster
+// at p = 16, and one for each coarser level).
+constexpr int kChainMax = 6;
+constexpr int kChainCtas = 8;  // portable cluster size
+struct ShiftChain {
+    float2* level[kChainMax + 1];
+    int first, last;  // child levels, in the order they are taken
+};
+
+template <int P, bool UP>
+__global__ void __cluster_dims__(kChainCtas, 1, 1) __launch_bounds__(kChainThreads)
+    shift_chain_kernel(const __grid_constant__ ShiftChain ch, float scale, int conj, int accumulate)
+{
+    using C = ShiftCfg<P, kChainThreads>;
+    __shared__ ShiftSmem<P, kChainThreads> sm;
+    shift_coefficients<P>(sm.c, scale, C::THREADS);
+    for (int l = ch.first;; l += UP ? -1 : 1) {
+        const int64_t parents = (int64_t)1 << (2 * (l - 1));
+        for (int64_t b = blockIdx.x; b * C::BOXES < parents; b += kChainCtas) {
+            if constexpr (UP)
+                shift_up_block<P>(sm, l, ch.level[l], ch.level[l - 1], conj, accumulate, b);
+            else
+                shift_down_block<P>(sm, l, ch.level[l - 1], ch.level[l], conj, accumulate, b);
+            __syncthreads();  // the exchanged rows have been read
+        }
+        if (l == ch.last) break;
+        asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+    }
+}
+
 template <int P>
 static int shift_launch(bool up, int child_level, const float2* In, float2* Out, float scale, bool conj, bool acc,
                         cudaStream_t st)
 {
-    using C = ShiftCfg<P>;
+    using C = ShiftCfg<P, kShiftThreads>;
     const int64_t parents = (int64_t)1 << (2 * (child_level - 1));
     const unsigned grid = (unsigned)((parents + C::BOXES - 1) / C::BOXES);
     if (up)
-        shift_up_kernel<P><<<grid, C::THREADS, 0, st>>>(child_level, In, Out, scale, conj, acc);
+        shift_kernel<P, true><<<grid, C::THREADS, 0, st>>>(child_level, In, Out, scale, conj, acc);
     else
-        shift_down_kernel<P><<<grid, C::THREADS, 0, st>>>(child_level, In, Out, scale, conj, acc);
+        shift_kernel<P, false><<<grid, C::THREADS, 0, st>>>(child_level, In, Out, scale, conj, acc);
+    FMM_CUDA_TRY(cudaGetLastError());
+    return FMM_OK;
+}
+
+template <int P>
+static int chain_launch(bool up, const ShiftChain& ch, float scale, bool conj, bool acc, cudaStream_t st)
+{
+    if (up)
+        shift_chain_kernel<P, true><<<kChainCtas, ShiftCfg<P, kChainThreads>::THREADS, 0, st>>>(ch, scale, conj, acc);
+    else
+        shift_chain_kernel<P, false><<<kChainCtas, ShiftCfg<P, kChainThreads>::THREADS, 0, st>>>(ch, scale, conj, acc);
     FMM_CUDA_TRY(cudaGetLastError());
     return FMM_OK;
 }
@@ -182,10 +242,21 @@ int launch_shift(bool up, int child_level, int p, const float2* In, float2* Out,
 
 using namespace fmmgb;
 
+static int launch_chain(bool up, int p, const ShiftChain& ch, float scale, bool conj, bool acc, cudaStream_t st)
+{
+    switch (p) {
+        case 6: return chain_launch<6>(up, ch, scale, conj, acc, st);
+        case 8: return chain_launch<8>(up, ch, scale, conj, acc, st);
+        case 12: return chain_launch<12>(up, ch, scale, conj, acc, st);
+        case 16: return chain_launch<16>(up, ch, scale, conj, acc, st);
+        default: return chain_launch<24>(up, ch, scale, conj, acc, st);
+    }
+}
+
 // A whole pass of fmm_m2m (op 0), fmm_l2l_adjoint (1, accumulating), fmm_l2l (2, accumulating) or
 // fmm_m2m_adjoint (3, accumulating) over levels lmin..lmax, levels[i] the array of level lmin + i:
-// the same launches as the per-level calls, enqueued by one.  Used by the Python layer, whose calls
-// cost more than the coarse levels' kernels; not part of the public header.
+// the same sums as the per-level calls, the levels up to kChainMax in one launch.  Used by the
+// Python layer, whose calls cost more than the coarse levels' kernels; not part of the public header.
 extern "C" int fmmgb_shift_levels(int32_t op, int32_t p, int32_t lmin, int32_t lmax, void* const* levels, void* stream)
 {
     clear_error();
@@ -198,17 +269,33 @@ extern "C" int fmmgb_shift_levels(int32_t op, int32_t p, int32_t lmin, int32_t l
         if (!levels[i] || ((uintptr_t)levels[i] & 7))
             return fail(FMM_EINVAL, "fmmgb_shift_levels: level %d NULL or misaligned", lmin + i);
     const cudaStream_t st = (cudaStream_t)stream;
-    for (int k = 1; k <= lmax - lmin; ++k) {
-        const int l = op < 2 ? lmax + 1 - k : lmin + k;  // child level: finest first upward, last downward
+    const bool up = op < 2;
+    // child levels lmin + 1 .. chain in one launch where there are at least two of them
+    const int chain = shift_supported(p) && std::min(lmax, kChainMax) - lmin >= 2 ? std::min(lmax, kChainMax) : lmin;
+    auto run_chain = [&]() -> int {
+        if (chain == lmin) return FMM_OK;
+        ShiftChain ch{};
+        for (int l = lmin; l <= chain; ++l) ch.level[l] = (float2*)levels[l - lmin];
+        ch.first = up ? chain : lmin + 1;
+        ch.last = up ? lmin + 1 : chain;
+        return launch_chain(up, p, ch, op == 1 || op == 2 ? 0.5f : 1.f, op & 1, op != 0, st);
+    };
+    auto one = [&](int l) -> int {
         float2 *child = (float2*)levels[l - lmin], *parent = (float2*)levels[l - 1 - lmin];
-        int rc = FMM_OK;
         switch (op) {
-            case 0: rc = launch_m2m(l, p, child, parent, false, st); break;
-            case 1: rc = launch_l2l(l, p, child, parent, true, true, st); break;
-            case 2: rc = launch_l2l(l, p, parent, child, true, false, st); break;
-            default: rc = launch_m2m_adjoint(l, p, parent, child, true, st); break;
+            case 0: return launch_m2m(l, p, child, parent, false, st);
+            case 1: return launch_l2l(l, p, child, parent, true, true, st);
+            case 2: return launch_l2l(l, p, parent, child, true, false, st);
+            default: return launch_m2m_adjoint(l, p, parent, child, true, st);
         }
-        if (rc) return rc;
+    };
+    if (up) {
+        for (int l = lmax; l > chain; --l)
+            if (int rc = one(l)) return rc;
+        return run_chain();
     }
+    if (int rc = run_chain()) return rc;
+    for (int l = chain + 1; l <= lmax; ++l)
+        if (int rc = one(l)) return rc;
     return FMM_OK;
 }

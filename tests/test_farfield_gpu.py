@@ -326,3 +326,37 @@ def test_p2m_orders_and_alignments(fmm, orc):
         fmm.fmm_p2m(level, p, torch.from_numpy(xy).cuda(), torch.from_numpy(c).cuda(), M)
         fmm.fmm_sync_status()
         assert _rel(_host(M), ref) <= 1e-6, (p, shift)
+
+
+@pytest.mark.parametrize("p", [6, 7, 8, 12, 16, 24])
+@pytest.mark.parametrize("lmin,lmax", [(2, 3), (2, 4), (0, 2), (3, 7), (2, 8), (6, 8)])
+def test_level_passes_equal_the_per_level_calls(fmm, p, lmin, lmax):
+    """A pass over several levels (the coarse ones in one launch of a cluster, the finer ones and the
+    general orders level by level) writes what the per-level calls write, bit for bit."""
+    import torch
+
+    g = torch.Generator(device="cuda").manual_seed(100 * lmax + p)
+    lv = list(range(lmin, lmax + 1))
+
+    def data():
+        return [torch.view_as_complex(torch.randn((4 ** l, p, 2), device="cuda", generator=g)) for l in lv]
+
+    def down(f, X):
+        for i in range(1, len(lv)):
+            f(lv[i], p, X[i - 1], X[i], accumulate=True)
+
+    def up(f, X, **kw):
+        for i in range(len(lv) - 1, 0, -1):
+            f(lv[i], p, X[i], X[i - 1], **kw)
+
+    for op, ref in ((fmm.SHIFT_M2M, lambda X: up(fmm.fmm_m2m, X)),
+                    (fmm.SHIFT_L2L_ADJOINT, lambda X: up(fmm.fmm_l2l_adjoint, X, accumulate=True)),
+                    (fmm.SHIFT_L2L, lambda X: down(fmm.fmm_l2l, X)),
+                    (fmm.SHIFT_M2M_ADJOINT, lambda X: down(fmm.fmm_m2m_adjoint, X))):
+        X = data()
+        Y = [x.clone() for x in X]
+        ref(X)
+        fmm._shift_levels(op, p, lmin, Y, None)
+        fmm.fmm_sync_status()
+        for l, a, b in zip(lv, X, Y):
+            assert torch.equal(torch.view_as_real(a), torch.view_as_real(b)), (op, l)
