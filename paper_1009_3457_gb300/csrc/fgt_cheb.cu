@@ -61,6 +61,7 @@ __global__ void __launch_bounds__(256) cheb_table_kernel(int ncut, double d, flo
 {
     __shared__ double s_h[P][Q], s_cos[4 * Q];
     const int tid = threadIdx.x, k = blockIdx.x;
+    after_go();
     if (tid < 4 * Q) s_cos[tid] = cospi((double)tid / (2.0 * Q));
     __syncthreads();
     if (tid < Q) {
@@ -76,6 +77,7 @@ __global__ void __launch_bounds__(256) cheb_table_kernel(int ncut, double d, flo
         }
     }
     __syncthreads();
+    after_wait();  // an earlier call may still read the table
     for (int e = tid; e < P * Q; e += 256) {
         const int a = e / Q, m = e % Q;
         double s = 0.0;
@@ -116,6 +118,8 @@ __global__ void __launch_bounds__(kSeg* kTaps* R)
     float* s_tab = reinterpret_cast<float*>(cheb_smem);  // [taps][P][Q]
     float* s_win = s_tab + taps * P * Q;                 // [kSeg + 2 ncut][BOX], then the groups' sums
     const int tid = threadIdx.x, line = blockIdx.y, t0 = blockIdx.x * kSeg;
+    after_go();
+    after_wait();
     for (int i = tid; i < taps * P * Q / 4; i += C::THREADS)
         reinterpret_cast<float4*>(s_tab)[i] = __ldg(reinterpret_cast<const float4*>(W) + i);
     constexpr int B4 = P * R / 4;
@@ -258,6 +262,8 @@ template <int P, int Q>
 __global__ void __launch_bounds__(kEvalThreads) cheb_eval_kernel(ChebEval a)
 {
     const int lane = threadIdx.x & 31, side = 1 << a.g, nbox = side * side;
+    after_go();
+    after_wait();
     const int64_t base = ((int64_t)blockIdx.x * (kEvalThreads / 32) + (threadIdx.x >> 5)) * (32 * kRows);
     bin_check(a.box_start, nbox, a.n, a.err);
     if (base >= a.n) return;
@@ -369,18 +375,14 @@ static int cheb_launch(const ChebEval& e, float* ws, cudaStream_t st)
     static unsigned long long opted[2];
     if (int rc = smem_opt_in((const void*)cheb_pass_kernel<P, P, Q>, (int)C1::smem(kChebMaxCut), &opted[0])) return rc;
     if (int rc = smem_opt_in((const void*)cheb_pass_kernel<P, Q, Q>, (int)C2::smem(kChebMaxCut), &opted[1])) return rc;
-    cheb_table_kernel<P, Q><<<2 * e.ncut + 1, 256, 0, st>>>(e.ncut, e.d, W);
-    FMM_CUDA_TRY(cudaGetLastError());
+    FMM_CUDA_TRY(launch_after(cheb_table_kernel<P, Q>, 2 * e.ncut + 1, 256, 0, st, e.ncut, e.d, W));
     const dim3 grid((side + kSeg - 1) / kSeg, side);
-    cheb_pass_kernel<P, P, Q><<<grid, C1::THREADS, C1::smem(e.ncut), st>>>(side, e.ncut, e.A, W, X);
-    FMM_CUDA_TRY(cudaGetLastError());
-    cheb_pass_kernel<P, Q, Q><<<grid, C2::THREADS, C2::smem(e.ncut), st>>>(side, e.ncut, X, W, C);
-    FMM_CUDA_TRY(cudaGetLastError());
+    FMM_CUDA_TRY(launch_after(cheb_pass_kernel<P, P, Q>, grid, C1::THREADS, C1::smem(e.ncut), st, side, e.ncut, e.A, W, X));
+    FMM_CUDA_TRY(launch_after(cheb_pass_kernel<P, Q, Q>, grid, C2::THREADS, C2::smem(e.ncut), st, side, e.ncut, X, W, C));
     ChebEval a = e;
     a.C = C;
     const unsigned blocks = bin_blocks(a.n, kEvalThreads * kRows, (int64_t)1 << (2 * e.g), kEvalThreads);
-    cheb_eval_kernel<P, Q><<<blocks, kEvalThreads, 0, st>>>(a);
-    FMM_CUDA_TRY(cudaGetLastError());
+    FMM_CUDA_TRY(launch_after(cheb_eval_kernel<P, Q>, blocks, kEvalThreads, 0, st, a));
     return FMM_OK;
 }
 

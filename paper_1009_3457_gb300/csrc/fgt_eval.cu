@@ -105,6 +105,7 @@ __global__ void __launch_bounds__(kT2pThreads) fgt_t2p_binned_kernel(int g, doub
                                                                      float* __restrict__ G, int accumulate, int* err)
 {
     const int lane = threadIdx.x & 31, side = 1 << g, nbox = side * side;
+    after_wait();
     const int64_t base = ((int64_t)blockIdx.x * (kT2pThreads / 32) + (threadIdx.x >> 5)) * (32 * kT2pRows);
     bin_check(box_start, nbox, n, err);
     if (base >= n) return;
@@ -167,13 +168,9 @@ static int t2p_binned_p(int g, double sigma, const float* C, int n, const double
     const double inv_scale = 1.0 / (sqrt(2.0) * sigma);
     const float dcell = (float)(ldexp(1.0, -g) * inv_scale);
     const unsigned grid = bin_blocks(n, kT2pThreads * kT2pRows, (int64_t)1 << (2 * g), kT2pThreads);
-    if (((uintptr_t)C & 15) == 0)
-        fgt_t2p_binned_kernel<P, true><<<grid, kT2pThreads, 0, st>>>(g, inv_scale, dcell, C, n, y, perm, box_start, G,
-                                                                     acc ? 1 : 0, err);
-    else
-        fgt_t2p_binned_kernel<P, false><<<grid, kT2pThreads, 0, st>>>(g, inv_scale, dcell, C, n, y, perm, box_start, G,
-                                                                      acc ? 1 : 0, err);
-    FMM_CUDA_TRY(cudaGetLastError());
+    auto kern = ((uintptr_t)C & 15) == 0 ? fgt_t2p_binned_kernel<P, true> : fgt_t2p_binned_kernel<P, false>;
+    FMM_CUDA_TRY(launch_after(kern, grid, kT2pThreads, 0, st, g, inv_scale, dcell, C, n, y, perm, box_start, G, acc ? 1 : 0,
+                              err));
     return FMM_OK;
 }
 

@@ -65,6 +65,7 @@ __device__ __forceinline__ int warp_box_claim(int* __restrict__ counter, int key
 // grid-stride over warps: all 32 lanes of a warp take part in every round
 __global__ void bin_count_kernel(int g, const double* __restrict__ y, int64_t n, int* __restrict__ counts)
 {
+    after_go();
     const int lane = threadIdx.x & 31;
     const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -121,6 +122,8 @@ __device__ void block_exclusive_scan(int nbox, Load v, Put put, int* out)
 // box_start[0..nbox] = exclusive scan of counts; counts becomes the scatter cursor (the same prefix)
 __global__ void __launch_bounds__(kScanThreads) bin_scan_kernel(int nbox, int* counts, int* __restrict__ box_start)
 {
+    after_go();
+    after_wait();
     block_exclusive_scan(
         nbox, [&](int i) { return counts[i]; }, [&](int i, int e) { counts[i] = e; }, box_start);
 }
@@ -137,6 +140,8 @@ __global__ void __launch_bounds__(kScanThreads) bin_scan_tiles_kernel(int nbox, 
                                                                       int* __restrict__ box_start)
 {
     __shared__ int s_warp[kScanThreads / 32], s_before;
+    after_go();
+    after_wait();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, first = blockIdx.x * kScanTile;
     int before = 0;
 #pragma unroll 4
@@ -188,6 +193,8 @@ __global__ void __launch_bounds__(kScanThreads) bin_scan_tiles_kernel(int nbox, 
 __global__ void bin_scatter_kernel(int g, const double* __restrict__ y, int64_t n, int* __restrict__ cursor,
                                    int* __restrict__ perm)
 {
+    after_go();
+    after_wait();
     const int lane = threadIdx.x & 31;
     const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -230,6 +237,7 @@ __device__ __forceinline__ void for_boxes(const double* __restrict__ y, int g, i
 __global__ void __launch_bounds__(kBinThreads) bin_count_smem_kernel(int g, const double* __restrict__ y, int64_t n,
                                                                      int64_t chunk, int* __restrict__ counts)
 {
+    after_go();
     extern __shared__ int s_cnt[];
     const int nbox = 1 << (2 * g);
     for (int b = threadIdx.x; b < nbox; b += kBinThreads) s_cnt[b] = 0;
@@ -248,9 +256,11 @@ __global__ void __launch_bounds__(kBinThreads) bin_scatter_smem_kernel(int g, co
                                                                        int64_t chunk, int* __restrict__ cursor,
                                                                        int* __restrict__ perm)
 {
+    after_go();
     extern __shared__ int s_cnt[];
     const int nbox = 1 << (2 * g);
     for (int b = threadIdx.x; b < nbox; b += kBinThreads) s_cnt[b] = 0;
+    after_wait();
     __syncthreads();
     const int64_t i0 = (int64_t)blockIdx.x * chunk, i1 = i0 + chunk < n ? i0 + chunk : n;
     for_boxes(y, g, i0 + threadIdx.x, i1, [&](int64_t, int b) { atomicAdd(&s_cnt[b], 1); });
@@ -926,19 +936,17 @@ extern "C" int fgt_bin_points(int32_t grid_log2, const double* y, int64_t n, int
         FMM_CUDA_TRY(cudaGetLastError());
     }
     if (nbox <= kScanTile) {
-        bin_scan_kernel<<<1, kScanThreads, 0, st>>>(nbox, work, box_start);
-        FMM_CUDA_TRY(cudaGetLastError());
+        FMM_CUDA_TRY(launch_after(bin_scan_kernel, 1, kScanThreads, 0, st, nbox, work, box_start));
     } else {
-        bin_scan_tiles_kernel<<<nbox / kScanTile, kScanThreads, 0, st>>>(nbox, work, box_start);
-        FMM_CUDA_TRY(cudaGetLastError());
+        FMM_CUDA_TRY(launch_after(bin_scan_tiles_kernel, nbox / kScanTile, kScanThreads, 0, st, nbox, work, box_start));
         FMM_CUDA_TRY(cudaMemcpyAsync(work, box_start, sizeof(int) * (size_t)nbox, cudaMemcpyDeviceToDevice, st));
     }
     if (n > 0) {
         if (smem)
-            bin_scatter_smem_kernel<<<grid, kBinThreads, smem_bytes, st>>>(grid_log2, y, n, chunk, work, perm);
+            FMM_CUDA_TRY(launch_after(bin_scatter_smem_kernel, grid, kBinThreads, smem_bytes, st, grid_log2, y, n, chunk,
+                                      work, perm));
         else
-            bin_scatter_kernel<<<grid, kBinThreads, 0, st>>>(grid_log2, y, n, work, perm);
-        FMM_CUDA_TRY(cudaGetLastError());
+            FMM_CUDA_TRY(launch_after(bin_scatter_kernel, grid, kBinThreads, 0, st, grid_log2, y, n, work, perm));
     }
     return FMM_OK;
 }

@@ -89,8 +89,7 @@ static int launch_p(M2LLaunch& job, const M2LTables& t, cudaStream_t st)
         grid = occ * sms;
         if ((rc = tile_counter(&counter, st))) return rc;
     }
-    kern<<<grid, C::THREADS, C::smem, st>>>(job, t.a, t.b, total, counter);
-    FMM_CUDA_TRY(cudaGetLastError());
+    FMM_CUDA_TRY(launch_after(kern, grid, C::THREADS, C::smem, st, job, t.a, t.b, total, counter));
     return FMM_OK;
 }
 

@@ -551,7 +551,8 @@ __global__ void __launch_bounds__(M2LCfg<P>::THREADS, M2LCfg<P>::MIN_CTAS)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int s_next;
-    m2l_load_operator<P, M2LCfg<P>::THREADS>(smem_raw, ascale, bscale);
+    m2l_load_operator<P, M2LCfg<P>::THREADS>(smem_raw, ascale, bscale);  // tables of long ago
+    after_wait();
     int tile = blockIdx.x;
     while (tile < total) {
         int li = 0;

@@ -157,6 +157,7 @@ __global__ void __launch_bounds__(kShiftThreads)
 {
     __shared__ ShiftSmem<P, kShiftThreads> sm;
     shift_coefficients<P>(sm.c, scale, ShiftCfg<P, kShiftThreads>::THREADS);
+    after_wait();
     // visible to the block at the barrier inside
     if constexpr (UP)
         shift_up_block<P>(sm, child_level, In, Out, conj, accumulate, blockIdx.x);
@@ -182,6 +183,7 @@ __global__ void __cluster_dims__(kChainCtas, 1, 1) __launch_bounds__(kChainThrea
     using C = ShiftCfg<P, kChainThreads>;
     __shared__ ShiftSmem<P, kChainThreads> sm;
     shift_coefficients<P>(sm.c, scale, C::THREADS);
+    after_wait();
     for (int l = ch.first;; l += UP ? -1 : 1) {
         const int64_t parents = (int64_t)1 << (2 * (l - 1));
         for (int64_t b = blockIdx.x; b * C::BOXES < parents; b += kChainCtas) {
@@ -203,22 +205,16 @@ static int shift_launch(bool up, int child_level, const float2* In, float2* Out,
     using C = ShiftCfg<P, kShiftThreads>;
     const int64_t parents = (int64_t)1 << (2 * (child_level - 1));
     const unsigned grid = (unsigned)((parents + C::BOXES - 1) / C::BOXES);
-    if (up)
-        shift_kernel<P, true><<<grid, C::THREADS, 0, st>>>(child_level, In, Out, scale, conj, acc);
-    else
-        shift_kernel<P, false><<<grid, C::THREADS, 0, st>>>(child_level, In, Out, scale, conj, acc);
-    FMM_CUDA_TRY(cudaGetLastError());
+    auto kern = up ? shift_kernel<P, true> : shift_kernel<P, false>;
+    FMM_CUDA_TRY(launch_after(kern, grid, C::THREADS, 0, st, child_level, In, Out, scale, conj, acc));
     return FMM_OK;
 }
 
 template <int P>
 static int chain_launch(bool up, const ShiftChain& ch, float scale, bool conj, bool acc, cudaStream_t st)
 {
-    if (up)
-        shift_chain_kernel<P, true><<<kChainCtas, ShiftCfg<P, kChainThreads>::THREADS, 0, st>>>(ch, scale, conj, acc);
-    else
-        shift_chain_kernel<P, false><<<kChainCtas, ShiftCfg<P, kChainThreads>::THREADS, 0, st>>>(ch, scale, conj, acc);
-    FMM_CUDA_TRY(cudaGetLastError());
+    auto kern = up ? shift_chain_kernel<P, true> : shift_chain_kernel<P, false>;
+    FMM_CUDA_TRY(launch_after(kern, kChainCtas, ShiftCfg<P, kChainThreads>::THREADS, 0, st, ch, scale, conj, acc));
     return FMM_OK;
 }
 

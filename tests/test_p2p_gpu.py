@@ -217,3 +217,52 @@ def test_p2p_sparse_and_dense_claims(fmm, orc, level, per_box):
     scale = np.abs(phi0[pick]) + np.abs(ref)
     assert np.linalg.norm(got - ref) <= 1e-4 * np.linalg.norm(ref)
     assert (np.abs(got - ref) <= 2e-4 * np.abs(ref).max() + 1e-6 * scale).all()
+
+
+def test_chains_of_launches_replay_from_a_graph(fmm, orc):
+    """Binning on a grid whose prefix is copied between two kernels, M2L of levels 0.. (memsets before
+    the kernel) and the whole potential with its two streams, recorded in one CUDA graph and replayed,
+    with other strengths too: equal to direct calls."""
+    import torch
+
+    from paper_1009_3457_gb300 import farfield
+
+    level, p, n = 8, 8, 300_000
+    rng = np.random.default_rng(12)
+    sets = [(torch.from_numpy(rng.random((n, 2))).cuda(), torch.from_numpy(rng.uniform(-1, 1, n)).cuda())
+            for _ in range(2)]
+    tree = fmm.fmm_build_lists(None, level)
+    xy, c = sets[0][0].clone(), sets[0][1].clone()
+    Ms = [torch.view_as_complex(torch.randn((4 ** l, p, 2), device="cuda")) for l in range(level + 1)]
+    Ls = [torch.full_like(m, float("nan")) for m in Ms]
+    perm, start = _bins(fmm, level, xy)
+    work = torch.empty(4 ** level, dtype=torch.int32, device="cuda")
+    pot = farfield.FmmPotential(tree, p, xy, c, xy)
+    fmm.fmm_m2l_levels(tree, 0, p, Ms, Ls)
+    pot()
+    torch.cuda.synchronize()
+    want = [l.clone() for l in Ls]
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, capture_error_mode="thread_local"):
+        fmm.fmm_bin_points(level, xy, perm, start, work)
+        fmm.fmm_m2l_levels(tree, 0, p, Ms, Ls)
+        pot()
+    for pts, q in sets:
+        if pts is not sets[0][0]:
+            c.copy_(q)  # the positions keep their bins
+        for l in Ls:
+            l.fill_(float("nan"))
+        perm.zero_()
+        start.zero_()
+        graph.replay()
+        fmm.fmm_sync_status()
+        got = pot.phi.clone()
+        pot()
+        fmm.fmm_sync_status()
+        assert torch.equal(torch.view_as_real(got), torch.view_as_real(pot.phi))
+        for a, b in zip(Ls, want):
+            assert torch.equal(torch.view_as_real(a), torch.view_as_real(b))
+        ix = torch.clamp((xy * 2 ** level).floor().long(), 0, 2 ** level - 1)
+        box = ix[:, 1] * 2 ** level + ix[:, 0]
+        assert torch.equal(torch.diff(start).long(), torch.bincount(box, minlength=4 ** level))
+        assert torch.equal(box[perm.long()], torch.sort(box).values)
