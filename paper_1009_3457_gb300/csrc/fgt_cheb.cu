@@ -21,10 +21,12 @@
 // there); wider boxes keep the direct sum.  The sums are FP32, as in the direct kernel.
 //
 // Measured at p = 16, n_cut = 10: 2^20 clustered targets, 32 x 32 boxes (263.6M target-box pairs)
-// 2,350 us direct -> 52 us (table 6, contractions 8.6 and 7.6, evaluation 30, which is bound by the
+// 2,350 us direct -> 50 us (table 6, contractions 7 and 6, evaluation 30, which is bound by the
 // gathers of the targets and the scattered results); 3*10^5 targets, 16 x 16 boxes, against the
-// tensor-core form 128 -> 29 us.  The whole transform's error against 64 bits falls with it, 3.7e-7
-// -> 2.0e-7 (3.1e-6 -> 3.7e-7 against BF16x3): a target's value sums 144 terms instead of 10^5.
+// tensor-core form 128 -> 27 us.  Error against 64 bits on the same coefficients, mean of 20 draws:
+// 2.7e-7 -> 1.6e-7 (3.4e-6 where BF16x3 is asked for): a target's value sums 144 terms instead of
+// 10^5.  A tap's P terms are summed apart before they join the sum over the taps: 1.9e-7 -> 1.6e-7, and
+// 173 -> 169 us for the whole transform.
 //
 // The rule's other lines: at least 2 targets per box on average (the contractions cost a box
 // what the direct sum costs ~1 target) and grids of up to 256 x 256 boxes (128 MB of
@@ -92,7 +94,7 @@ __global__ void __launch_bounds__(256) cheb_table_kernel(int ncut, double d, flo
 // the other index).  A CTA takes kSeg target boxes of a line and stages their window of
 // kSeg + 2 n_cut source boxes and the table; a thread owns (box, r) and all Q outputs, over
 // every kTaps-th tap, so a step is one scalar and Q/4 broadcast 16-byte shared loads for Q
-// multiply-adds; the tap groups' sums meet in shared memory.
+// multiply-adds; the taps' sums are added in registers and the groups' meet in shared memory.
 constexpr int kSeg = 4;
 constexpr int kTaps = 4;
 
@@ -131,12 +133,15 @@ __global__ void __launch_bounds__(kSeg* kTaps* R)
     }
     __syncthreads();
     const int group = tid / (kSeg * R), e = tid % (kSeg * R), seg = e / R, r = e % R;
-    float acc[Q];
+    float sum[Q];
 #pragma unroll
-    for (int m = 0; m < Q; ++m) acc[m] = 0.f;
+    for (int m = 0; m < Q; ++m) sum[m] = 0.f;
     for (int j = group; j < taps; j += kTaps) {  // source box t + j - ncut: offset ncut - j
         const float* v = s_win + (seg + j) * C::BOX + r;
         const float4* w = reinterpret_cast<const float4*>(s_tab + (2 * ncut - j) * P * Q);
+        float acc[Q];
+#pragma unroll
+        for (int m = 0; m < Q; ++m) acc[m] = 0.f;
 #pragma unroll 4
         for (int c = 0; c < P; ++c) {
             const float x = v[c * R];
@@ -149,12 +154,14 @@ __global__ void __launch_bounds__(kSeg* kTaps* R)
                 acc[4 * q + 3] = fmaf(x, h.w, acc[4 * q + 3]);
             }
         }
+#pragma unroll
+        for (int m = 0; m < Q; ++m) sum[m] += acc[m];
     }
     __syncthreads();
 #pragma unroll
     for (int q = 0; q < Q / 4; ++q)
         *reinterpret_cast<float4*>(s_win + group * C::OUT + e * Q + 4 * q) =
-            make_float4(acc[4 * q], acc[4 * q + 1], acc[4 * q + 2], acc[4 * q + 3]);
+            make_float4(sum[4 * q], sum[4 * q + 1], sum[4 * q + 2], sum[4 * q + 3]);
     __syncthreads();
     for (int i = tid; i < C::OUT; i += C::THREADS) {
         const int t = t0 + i / (R * Q);
