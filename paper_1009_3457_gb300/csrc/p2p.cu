@@ -38,7 +38,13 @@ constexpr int kP2pWarps = kP2pThreads / 32;     // each takes a quarter of the s
 constexpr int kP2pR = 3;                        // targets per lane (rows of 32 targets per claim)
 constexpr int kP2pRun = 32 * kP2pR;             // targets per claim
 constexpr int kP2pBatch = 1024;                 // sources per shared-memory batch
-constexpr int kP2pSharedCtas = 8;               // resident CTAs per SM with FMM_P2P_SHARE_SM
+// With FMM_P2P_SHARE_SM a CTA (a warp of it in the warp kernel) ends after this many claims, and kernels of
+// a stream of higher priority take its place; a persistent CTA would hold its registers to the end.  The
+// potential of 2^22 points with the far field beside it: 1,240 us with persistent CTAs (8 per SM), 1,167 /
+// 1,157 / 1,163 / 1,169 with 1 / 2 / 3 / 4 claims; the near field alone 923 us persistent, 925 with 2.  A warp a claim
+// loses more alone (2^22 points at level 9 689 -> 731), so that without the flag CTAs persist.
+constexpr int kP2pShareClaims = 2;
+constexpr int kP2pShareGrid = 1 << 16;          // more claims a CTA rather than more CTAs (most find none)
 // The warp kernel takes calls of fewer than kP2pDense targets a box on average, on kP2wBoxes boxes or
 // more (fewer claims than warps otherwise).  us, CTA / warp: 16 a box at level 5 26 / 35, level 6 31 / 35,
 // level 7 68 / 62, level 8 216 / 170, level 9 914 / 676; 32 a box at level 6 41 / 55, level 7 105 / 110,
@@ -51,7 +57,6 @@ constexpr int kP2wPairs = 4;                    // packed target pairs per lane,
 constexpr int kP2wRun = 2 * kP2wLanes * kP2wPairs;  // targets per claim
 constexpr int kP2wChunk = 96;                   // sources per staging buffer of a warp
 constexpr int kP2wCtas = 7;                     // resident CTAs per SM (72 registers)
-constexpr int kP2wSharedCtas = 6;               // ... with FMM_P2P_SHARE_SM
 // added to every r^2 (in box sides squared): a source at the target's position
 // (dx = dy = 0) then contributes exactly 0 -- c / 1e-30 is finite for |c| < 3e8 -- and
 // any other pair changes by a relative 1e-30 / r^2 (below FP32 rounding for distances
@@ -73,6 +78,7 @@ struct P2pArgs {
     int ntab;
     float2* phi;
     int* cursor;  // [0] next claim index, [1] CTAs finished
+    int each;     // 0, or claims per CTA (warp): consecutive places of the table, no cursor
     int* err;
 };
 
@@ -254,13 +260,14 @@ __global__ void __launch_bounds__(kP2pThreads) fmm_p2p_kernel(P2pArgs a)
     const int side = 1 << a.level;
     const int total = min(__ldg(a.nclaim), a.ntab);
     // thread 0 fetches the index of the CTA's next claim one claim ahead
-    int knext = tid == 0 ? atomicAdd(a.cursor, 1) : 0;
+    int knext = a.each ? (int)blockIdx.x * a.each : tid == 0 ? atomicAdd(a.cursor, 1) : 0;
+    const int kend = a.each ? min(knext + a.each, total) : total;
 
     for (;;) {
         if (tid == 0) {
             const int k = knext;
-            s_claim = k < total ? __ldg(a.tab + k) : make_int4(-1, -1, 0, 0);
-            if (k < total) knext = atomicAdd(a.cursor, 1);
+            s_claim = k < kend ? __ldg(a.tab + k) : make_int4(-1, -1, 0, 0);
+            if (k < kend) knext = a.each ? k + 1 : atomicAdd(a.cursor, 1);
         }
         __syncthreads();
         const int4 cl = s_claim;
@@ -375,7 +382,7 @@ __global__ void __launch_bounds__(kP2pThreads) fmm_p2p_kernel(P2pArgs a)
         }
     }
     // the last CTA to finish returns the cursor slot to zero for its next use
-    if (tid == 0) {
+    if (tid == 0 && !a.each) {
         __threadfence();
         if (atomicAdd(a.cursor + 1, 1) == (int)gridDim.x - 1) {
             atomicExch(a.cursor, 0);
@@ -507,11 +514,13 @@ __global__ void __launch_bounds__(kP2pThreads, kP2wCtas) fmm_p2p_warp_kernel(P2p
     const int side = 1 << a.level;
     const int total = min(__ldg(a.nclaim), a.ntab);
     // lane 0 fetches the index of the warp's next claim one claim ahead
-    int knext = lane == 0 ? atomicAdd(a.cursor, 1) : 0;
+    const int warp = (int)blockIdx.x * (kP2pThreads / 32) + (threadIdx.x >> 5);
+    int knext = a.each ? warp * a.each : lane == 0 ? atomicAdd(a.cursor, 1) : 0;
+    const int kend = a.each ? min(knext + a.each, total) : total;
     for (;;) {
         const int k = __shfl_sync(0xffffffffu, knext, 0);
-        if (k >= total) break;
-        if (lane == 0) knext = atomicAdd(a.cursor, 1);
+        if (k >= kend) break;
+        if (lane == 0) knext = a.each ? k + 1 : atomicAdd(a.cursor, 1);
         const int4 cl = __ldg(a.tab + k);
         const int first = cl.x, m = cl.y - cl.x, box = cl.z;
         const int tx = box & (side - 1), ty = box >> a.level;
@@ -536,7 +545,7 @@ __global__ void __launch_bounds__(kP2pThreads, kP2wCtas) fmm_p2p_warp_kernel(P2p
         }
     }
     // the last warp to finish returns the cursor slot to zero for its next use
-    if (lane == 0) {
+    if (lane == 0 && !a.each) {
         __threadfence();
         if (atomicAdd(a.cursor + 1, 1) == (int)gridDim.x * (kP2pThreads / 32) - 1) {
             atomicExch(a.cursor, 0);
@@ -604,13 +613,16 @@ extern "C" int fmm_p2p(int32_t level, const double* xy, const double* c, int64_t
     args.tperm = tgt_perm;
     args.tstart = tgt_start;
     args.phi = reinterpret_cast<float2*>(phi);
-    if (int rc = tile_counter(&args.cursor, st)) return rc;
+    const bool share = (flags & FMM_P2P_SHARE_SM) != 0;
+    args.cursor = nullptr;
+    if (!share)
+        if (int rc = tile_counter(&args.cursor, st)) return rc;
     if (int rc = device_error_word(&args.err)) return rc;
     const int nbox = 1 << (2 * level);
     const bool dense = nz >= (int64_t)kP2pDense * nbox || nbox < kP2wBoxes;
     const int run = dense ? kP2pRun : kP2wRun;
     // one buffer: the sources in box order, the claim table, the number of claims
-    const int64_t most = nz / run + nbox;  // claims can be no more
+    const int64_t most = nz / run + std::min<int64_t>(nbox, nz);  // claims can be no more
     float4* src = nullptr;
     if (int rc = p2p_source_buffer((size_t)(n + most + 1) * sizeof(float4), &src)) return rc;
     int4* tab = reinterpret_cast<int4*>(src + n);
@@ -627,28 +639,30 @@ extern "C" int fmm_p2p(int32_t level, const double* xy, const double* c, int64_t
     args.src = src;
     args.tab = tab;
     args.ntab = (int)most;
-    static int occ_cache[2];
-    static std::mutex mu;
     auto kern = dense ? fmm_p2p_kernel : fmm_p2p_warp_kernel;
-    int occ = 0;
-    {
-        std::lock_guard<std::mutex> lk(mu);
-        int& o = occ_cache[dense];
-        if (!o) {
-            FMM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, kern, kP2pThreads, 0));
-            if (o < 1) o = 1;
-        }
-        occ = o;
-    }
-    int sms = 0;
-    if (int rc = device_sm_count(&sms)) return rc;
-    // sharing the SMs with kernels of other streams: 8 CTAs (132 KB of shared memory, 1,024
-    // threads) per SM measured 1.5 % slower alone than the occupancy limit, and left room for
-    // the far field of the same FMM beside it (fewer starved the near field itself)
-    const int per_sm = (flags & FMM_P2P_SHARE_SM) ? std::min(occ, dense ? kP2pSharedCtas : kP2wSharedCtas) : occ;
     const int64_t ctas = dense ? most : (most + kP2pThreads / 32 - 1) / (kP2pThreads / 32);
-    const int grid = (int)std::min<int64_t>((int64_t)per_sm * sms, ctas);
-    kern<<<grid, kP2pThreads, 0, st>>>(args);
+    int64_t grid = 0;
+    args.each = 0;
+    if (share) {
+        args.each = (int)std::max<int64_t>(kP2pShareClaims, (ctas + kP2pShareGrid - 1) / kP2pShareGrid);
+        grid = (ctas + args.each - 1) / args.each;
+    } else {
+        static int occ_cache[2];
+        static std::mutex mu;
+        int sms = 0, occ = 0;
+        if (int rc = device_sm_count(&sms)) return rc;
+        {
+            std::lock_guard<std::mutex> lk(mu);
+            int& o = occ_cache[dense];
+            if (!o) {
+                FMM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, kern, kP2pThreads, 0));
+                if (o < 1) o = 1;
+            }
+            occ = o;
+        }
+        grid = std::min<int64_t>((int64_t)occ * sms, ctas);
+    }
+    kern<<<(unsigned)grid, kP2pThreads, 0, st>>>(args);
     FMM_CUDA_TRY(cudaGetLastError());
     return FMM_OK;
 }

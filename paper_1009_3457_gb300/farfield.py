@@ -114,12 +114,12 @@ class FmmPotential:
 
         phi(z) = sum_i c_i / (z - y_i)   (sources at exactly z skipped)
 
-    The near field and the far field up to L2L are independent: the near field runs on
-    a second stream (writing phi, with FMM_P2P_SHARE_SM so that the far-field kernels
-    find room on every SM), the far field on the current one, and L2P adds into phi
-    once both are done.  Buffers are allocated once; ``__call__`` enqueues the whole
-    evaluation, ending on the current stream (capturable as a CUDA graph after a
-    first call)."""
+    The near field and the far field up to L2L are independent: the near field runs on the
+    current stream (writing phi, with FMM_P2P_SHARE_SM so that its blocks end after a few
+    boxes), the far field on a second stream of higher priority, whose kernels take the places
+    that free up, and L2P adds into phi once both are done.  Buffers are allocated once;
+    ``__call__`` enqueues the whole evaluation, ending on the current stream (capturable as a
+    CUDA graph after a first call)."""
 
     def __init__(self, tree, p: int, xy: torch.Tensor, c: torch.Tensor, z: torch.Tensor, prec: int = 0):
         if tree.adaptive or tree.periodic or tree.max_level < 2:
@@ -142,19 +142,19 @@ class FmmPotential:
         fmmgb.fmm_bin_points(L, self.xy, self.sperm, self.sstart, work, stream=st)
         fmmgb.fmm_bin_points(L, self.z, self.tperm, self.tstart, work, stream=st)
         self.phi = torch.empty(nz, dtype=torch.complex64, device=dev)
-        self.side = torch.cuda.Stream(device=dev)
+        self.side = torch.cuda.Stream(device=dev, priority=-1)
 
     def __call__(self) -> torch.Tensor:
         p, L = self.p, self.L
         cur = torch.cuda.current_stream(self.phi.device)
-        st = fmmgb._stream(None)
-        self.side.wait_stream(cur)  # the inputs and phi are the current stream's until here
+        st, far = fmmgb._stream(None), self.side.cuda_stream
+        self.side.wait_stream(cur)  # the inputs and the expansions are the current stream's until here
         fmmgb.fmm_p2p(L, self.xy, self.c, self.sperm, self.sstart, self.z, self.tperm, self.tstart, self.phi,
-                      stream=self.side, share_sm=True)
-        fmmgb.fmm_p2m_binned(L, p, self.xy, self.c, self.sperm, self.sstart, self.Ms[-1], stream=st)
-        fmmgb._shift_levels(fmmgb.SHIFT_M2M, p, 2, self.Ms, st)
-        fmmgb.fmm_m2l_levels(self.tree, 2, p, self.Ms, self.Ls, prec=self.prec, stream=st)
-        fmmgb._shift_levels(fmmgb.SHIFT_L2L, p, 2, self.Ls, st)
+                      stream=st, share_sm=True)
+        fmmgb.fmm_p2m_binned(L, p, self.xy, self.c, self.sperm, self.sstart, self.Ms[-1], stream=far)
+        fmmgb._shift_levels(fmmgb.SHIFT_M2M, p, 2, self.Ms, far)
+        fmmgb.fmm_m2l_levels(self.tree, 2, p, self.Ms, self.Ls, prec=self.prec, stream=far)
+        fmmgb._shift_levels(fmmgb.SHIFT_L2L, p, 2, self.Ls, far)
         cur.wait_stream(self.side)
         fmmgb.fmm_l2p_binned(L, p, self.z, self.tperm, self.tstart, self.Ls[-1], self.phi, accumulate=True, stream=st)
         return self.phi
