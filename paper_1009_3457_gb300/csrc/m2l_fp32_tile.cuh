@@ -36,9 +36,9 @@
 // Cost per target: 10 p^2 packed multiply-adds and ~158 p additions instead of
 // 54 p^2 packed multiply-adds: 3.6x fewer cycles of the FP32 pipe at p = 16 (3.0x
 // at p = 8, 4.0x at p = 24).  Levels 2-8 of a 2^22-point tree (87,376 boxes):
-// p = 16 79.9 -> 31.1 us, where the pipe's own time for this count is 16.6 us
-// (53 % of it; 67 % at level 10, 394 us, where the launch, the first tile and the
-// last wave weigh less).  The rest is latency: 16 warps an SM, with the short
+// p = 16 79.9 -> 27.2 us back to back, where the pipe's own time for this count is
+// 16.6 us (61 % of it; 68 % at level 10, 391 us, where the launch, the first tile and
+// the last wave weigh less).  The rest is latency: 16 warps an SM, with the short
 // addition chains of the combinations between the multiply-adds.  The error
 // against 64 bits falls as well (2.9e-7 -> 1.6e-7): fewer terms are summed.
 //
@@ -58,7 +58,7 @@
 //     64 each warp takes both.  The two sums of a target meet in shared memory,
 //     from where the tile is written in whole rows of boxes.  Two warps a target
 //     are faster where a launch has only a few tiles per SM (p = 16, levels 2-8:
-//     31.1 against 33.6 us), one where it has many (40 trees of depth 4-9 in one
+//     31.1 against 33.6 us as ordinary launches), one where it has many (40 trees of depth 4-9 in one
 //     launch: 317 against 354 us), so the level kernel runs 128 threads and the
 //     batched one 64;
 //   - k runs in blocks of 4 (one period of r), so the code stays in the

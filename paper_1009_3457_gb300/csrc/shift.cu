@@ -17,9 +17,9 @@
 //
 // Threads are (box, index) pairs in index order, so every read and write of a coefficient row is
 // one coalesced run; a block's rows meet in shared memory.  Bound by memory at the finest levels and by the
-// launch at the coarse ones.  A 9-level tree at p = 16, seven launches a pass: M2M and L2L's transpose
-// together 253 -> 52 us, L2L and M2M's transpose 207 -> 58 us (a thread per output with its own
-// powers of z and a table read per term before).
+// launch at the coarse ones, which run as one (the chain below: four launches a pass instead of seven).
+// A 9-level tree at p = 16: M2M and L2L's transpose together 253 -> 57 us, L2L and M2M's transpose
+// 207 -> 60 us (a thread per output with its own powers of z and a table read per term before).
 #include <algorithm>
 
 #include "common.cuh"

@@ -56,11 +56,13 @@ def fgt_flops_per_box_separable(p: int, taps_x: int, taps_y: int) -> int:
     return 2 * p ** 3 * (taps_x + taps_y)
 
 
-def fgt_h2p_flops_per_pair(p: int) -> int:
-    """Eq. (hermite) for one target and one source box, as the bilinear form
-    h(t1)^T A h(t2): p^2 + p multiply-adds (the Hermite functions themselves are
-    not counted)."""
-    return 2 * (p * p + p)
+def fgt_h2p_cheb_flops(g: int, ncut: int, p: int, n: int, q: int = 12) -> int:
+    """Eq. (hermite) at n targets through q x q Chebyshev coefficients per target box: two contractions
+    along the grid's lines (p x p by p x q, then p x q by p x q per box and tap inside the grid), and
+    q^2 multiply-adds for each of the n targets."""
+    side = 1 << g
+    taps = sum(min(t + ncut, side - 1) - max(t - ncut, 0) + 1 for t in range(side)) * side
+    return 2 * taps * (p * p * q + p * q * q) + 2 * n * q * q
 
 
 def fgt_h2p_pairs(g: int, ncut: int, target_counts, source_nonempty) -> int:
@@ -83,25 +85,6 @@ def fgt_h2p_pairs(g: int, ncut: int, target_counts, source_nonempty) -> int:
                 x0, x1 = max(0, tx - ncut), min(n - 1, tx + ncut) + 1
                 total += int(t[ty, tx]) * int(c[y1, x1] - c[y0, x1] - c[y1, x0] + c[y0, x0])
     return total
-
-
-def fgt_h2p_tc_mma_flops(g: int, ncut: int, target_counts, products: int = 3, p: int = 16, rows: int = 128) -> int:
-    """Tensor-core flops that the tensor-core Hermite evaluation issues: per claim of up to
-    `rows` targets of a box, one [rows x p] x [p x (w p)] product per source row and precision
-    product, w x h the box's clipped neighbourhood (every box evaluated, full M tiles)."""
-    import numpy as np
-
-    n = 1 << g
-    t = np.asarray(target_counts, dtype=np.int64).reshape(n, n)
-    total = 0
-    for ty in range(n):
-        h = min(n - 1, ty + ncut) - max(0, ty - ncut) + 1
-        for tx in range(n):
-            if t[ty, tx]:
-                w = min(n - 1, tx + ncut) - max(0, tx - ncut) + 1
-                tiles = -(-int(t[ty, tx]) // rows)
-                total += tiles * h * 2 * rows * (w * p) * p
-    return total * products
 
 
 def p2p_pairs(level: int, target_counts, source_counts, self_pairs: int = 0) -> int:
