@@ -21,9 +21,9 @@
 // there); wider boxes keep the direct sum.  The sums are FP32, as in the direct kernel.
 //
 // Measured at p = 16, n_cut = 10: 2^20 clustered targets, 32 x 32 boxes (263.6M target-box pairs)
-// 2,350 us direct -> 50 us (table 6, contractions 7 and 6, evaluation 30, which is bound by the
+// 2,350 us direct -> 46 us (table 6, contractions 7 and 6, evaluation 26, which is bound by the
 // gathers of the targets and the scattered results); 3*10^5 targets, 16 x 16 boxes, against the
-// tensor-core form 128 -> 27 us.  Error against 64 bits on the same coefficients, mean of 20 draws:
+// tensor-core form 128 -> 26 us.  Error against 64 bits on the same coefficients, mean of 20 draws:
 // 2.7e-7 -> 1.6e-7 (3.4e-6 where BF16x3 is asked for): a target's value sums 144 terms instead of
 // 10^5.  A tap's P terms are summed apart before they join the sum over the taps: 1.9e-7 -> 1.6e-7, and
 // 173 -> 169 us for the whole transform.
@@ -259,6 +259,51 @@ __device__ __forceinline__ void cheb_sum(const float* __restrict__ c, const floa
     for (int r = 0; r < NR; ++r) out[r] = b1[r];
 }
 
+// Places base + 32 r + lane, r < NR, of the binned targets: tj[r] the target's index (-1: past the
+// end, or a perm entry out of range, which sets the error word), tb[r] the box of its coordinates
+// where that box holds the place, else -1, (o0, o1) its offset from that box's centre in box sides.
+// The loads of all rows are in flight together: index, coordinates and box range are three round
+// trips a warp instead of three a row (2^20 targets: 30 -> 26 us; fewer rows a lane, for more warps on an
+// SM, measured the same).
+template <int NR>
+__device__ __forceinline__ void binned_targets(const double* __restrict__ y, const int* __restrict__ perm,
+                                               const int* __restrict__ box_start, int g, int n, int64_t base, int* err,
+                                               int* tj, int* tb, float* o0, float* o1)
+{
+    double y0[NR], y1[NR];
+    int f[NR], e[NR];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) tj[r] = base + 32 * r < n ? __ldg(perm + base + 32 * r) : -1;
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+        const size_t j = (unsigned)tj[r] < (unsigned)n ? tj[r] : 0;
+        y0[r] = __ldg(y + 2 * j);
+        y1[r] = __ldg(y + 2 * j + 1);
+    }
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+        long long X0, X1;
+        tb[r] = -1;
+        o0[r] = o1[r] = 0.f;
+        if (grid_fixed31(y0[r], g, X0) && grid_fixed31(y1[r], g, X1)) {
+            tb[r] = ((int)(X1 >> 31) << g) + (int)(X0 >> 31);
+            o0[r] = cell_offset31(X0);
+            o1[r] = cell_offset31(X1);
+        }
+        f[r] = __ldg(box_start + max(tb[r], 0));
+        e[r] = __ldg(box_start + max(tb[r], 0) + 1);
+    }
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+        const int64_t pos = base + 32 * r;
+        if ((unsigned)tj[r] >= (unsigned)n) {
+            if (pos < n) atomicOr(err, DEV_ERR_CHECK);
+            tj[r] = tb[r] = -1;
+        } else if (tb[r] >= 0 && !(bin_range_ok(f[r], e[r], n) && f[r] <= pos && pos < e[r])) {
+            tb[r] = -1;
+        }
+    }
+}
 // A warp takes 32 kRows consecutive binned targets: together where they share a box (uniform
 // 16-byte loads of its coefficients, each feeding 4 kRows multiply-adds a lane), else a row of
 // 32 at a time with a box per lane.
@@ -276,29 +321,12 @@ __global__ void __launch_bounds__(kEvalThreads) cheb_eval_kernel(ChebEval a)
     if (base >= a.n) return;
     int tj[kRows], tb[kRows];  // target, its box (-1: evaluated apart)
     float x1[kRows], x2[kRows], out[kRows];
+    binned_targets<kRows>(a.y, a.perm, a.box_start, a.g, a.n, base + lane, a.err, tj, tb, x1, x2);
 #pragma unroll
     for (int r = 0; r < kRows; ++r) {
-        const int64_t pos = base + 32 * r + lane;
-        tj[r] = -1;
-        tb[r] = -1;
-        x1[r] = x2[r] = out[r] = 0.f;
-        if (pos >= a.n) continue;
-        const int j = __ldg(a.perm + pos);
-        if ((unsigned)j >= (unsigned)a.n) {
-            atomicOr(a.err, DEV_ERR_CHECK);
-            continue;
-        }
-        tj[r] = j;
-        const double y0 = __ldg(a.y + 2 * (size_t)j), y1 = __ldg(a.y + 2 * (size_t)j + 1);
-        long long X0, X1;
-        if (grid_fixed31(y0, a.g, X0) && grid_fixed31(y1, a.g, X1)) {
-            const int b = (int)(X1 >> 31) * side + (int)(X0 >> 31);
-            if (bin_holds(a.box_start, b, (int)pos, a.n)) {
-                tb[r] = b;
-                x1[r] = 2.f * cell_offset31(X0);
-                x2[r] = 2.f * cell_offset31(X1);
-            }
-        }
+        x1[r] *= 2.f;
+        x2[r] *= 2.f;
+        out[r] = 0.f;
     }
     const int b0 = __shfl_sync(0xffffffffu, tb[0], 0);
     bool same = b0 >= 0;
