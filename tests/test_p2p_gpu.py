@@ -266,3 +266,25 @@ def test_chains_of_launches_replay_from_a_graph(fmm, orc):
         box = ix[:, 1] * 2 ** level + ix[:, 0]
         assert torch.equal(torch.diff(start).long(), torch.bincount(box, minlength=4 ** level))
         assert torch.equal(box[perm.long()], torch.sort(box).values)
+
+
+@pytest.mark.parametrize("level,per_box", [(3, 100), (6, 8), (7, 0.3), (7, 20), (7, 40), (10, 0.6)])
+def test_p2p_short_lived_blocks_equal_persistent_ones(fmm, level, per_box):
+    """Both kernels, with blocks that end after a few claims (FMM_P2P_SHARE_SM; at level 10 more than
+    two, the grid being bounded) and with persistent ones: the same bits, twice."""
+    import torch
+
+    g = torch.Generator(device="cuda").manual_seed(level)
+    nz, n = int(per_box * 4 ** level), 20000
+    z, xy = (torch.rand((k, 2), dtype=torch.float64, device="cuda", generator=g) for k in (nz, n))
+    c = torch.rand(n, dtype=torch.float64, device="cuda", generator=g) - 0.5
+    (sp, ss), (tp, ts) = _bins(fmm, level, xy), _bins(fmm, level, z)
+    out = []
+    for share in (False, True, False, True):
+        phi = torch.full((nz,), float("nan"), dtype=torch.complex64, device="cuda")
+        fmm.fmm_p2p(level, xy, c, sp, ss, z, tp, ts, phi, share_sm=share)
+        fmm.fmm_sync_status()
+        assert bool(torch.isfinite(torch.view_as_real(phi)).all())
+        out.append(phi)
+    for phi in out[1:]:
+        assert torch.equal(torch.view_as_real(phi), torch.view_as_real(out[0]))
