@@ -211,64 +211,81 @@ __global__ void bin_scatter_kernel(int g, const double* __restrict__ y, int64_t 
 // atomics, and the global counters see one addition per box a block touches.
 constexpr int kBinSmemMaxLog2 = 7;
 
-// Calls f(i, box) for the points [i0, i1), kBinThreads apart from `first` on, the coordinates of
-// kBinLoads points in flight at a time (a load and a shared atomic in turn left a thread waiting
-// for each point's load: 7.7 -> 6.5 us to count 2^20 points, 14 -> 12.5 us to place them).
-constexpr int kBinLoads = 4;
-template <class F>
-__device__ __forceinline__ void for_boxes(const double* __restrict__ y, int g, int64_t first, int64_t i1, F f)
+// A block of T threads, LOADS points a thread in flight at a time (a load and a shared atomic in
+// turn left a thread waiting for each point's load).  fgt_bin_points takes
+//   - 1024 x 4 on grids of 4^6 boxes or more and 2^15 points or more: a histogram of 16 to 64 KB
+//     leaves room for few blocks, which then need their threads (2^20 points on 4^7 boxes 49 -> 33 us, 37
+//     with 512 threads; 2^18 on 4^6 20.5 -> 16.4);
+//   - 512 x 8 on smaller grids and 2^19 points or more (2^20 on 4^5 27 -> 22.5 us; 1024 threads 21, but
+//     they fill the SMs, and the next kernel's early part, the table of the Hermite evaluation, then waits:
+//     163 against 153 us for that transform);
+//   - 256 x 4 else: few blocks start and meet sooner (2^12 points 8.4 us against 9.6 with 1024
+//     threads; the Hermite transform of 3e5 points 79 us against 84 with 512).
+// Coordinates of the points first, first + T, ... (LOADS of them, below i1).
+template <int T, int LOADS>
+__device__ __forceinline__ void load_points(const double* __restrict__ y, int64_t first, int64_t i1,
+                                            double (&a)[LOADS], double (&b)[LOADS])
 {
-    for (int64_t i = first; i < i1; i += kBinLoads * kBinThreads) {
-        double a[kBinLoads], b[kBinLoads];
 #pragma unroll
-        for (int u = 0; u < kBinLoads; ++u) {
-            const int64_t k = i + u * kBinThreads;
-            a[u] = k < i1 ? __ldg(y + 2 * k) : 0.0;
-            b[u] = k < i1 ? __ldg(y + 2 * k + 1) : 0.0;
-        }
-#pragma unroll
-        for (int u = 0; u < kBinLoads; ++u) {
-            const int64_t k = i + u * kBinThreads;
-            if (k < i1) f(k, fgt_grid_box(a[u], b[u], g));
-        }
+    for (int u = 0; u < LOADS; ++u) {
+        const int64_t k = first + u * T;
+        a[u] = k < i1 ? __ldg(y + 2 * k) : 0.0;
+        b[u] = k < i1 ? __ldg(y + 2 * k + 1) : 0.0;
     }
 }
 
-__global__ void __launch_bounds__(kBinThreads) bin_count_smem_kernel(int g, const double* __restrict__ y, int64_t n,
-                                                                     int64_t chunk, int* __restrict__ counts)
+template <int T, int LOADS>
+__global__ void __launch_bounds__(T) bin_count_smem_kernel(int g, const double* __restrict__ y, int64_t n, int64_t chunk,
+                                                           int* __restrict__ counts)
 {
     after_go();
     extern __shared__ int s_cnt[];
     const int nbox = 1 << (2 * g);
-    for (int b = threadIdx.x; b < nbox; b += kBinThreads) s_cnt[b] = 0;
+    for (int b = threadIdx.x; b < nbox; b += T) s_cnt[b] = 0;
     __syncthreads();
     const int64_t i0 = (int64_t)blockIdx.x * chunk, i1 = i0 + chunk < n ? i0 + chunk : n;
-    for_boxes(y, g, i0 + threadIdx.x, i1, [&](int64_t, int b) { atomicAdd(&s_cnt[b], 1); });
+    for (int64_t i = i0 + threadIdx.x; i < i1; i += LOADS * T) {
+        double a[LOADS], b[LOADS];
+        load_points<T, LOADS>(y, i, i1, a, b);
+#pragma unroll
+        for (int u = 0; u < LOADS; ++u)
+            if (i + u * T < i1) atomicAdd(&s_cnt[fgt_grid_box(a[u], b[u], g)], 1);
+    }
     __syncthreads();
-    for (int b = threadIdx.x; b < nbox; b += kBinThreads)
+    for (int b = threadIdx.x; b < nbox; b += T)
         if (s_cnt[b]) atomicAdd(&counts[b], s_cnt[b]);
 }
 
-// The scatter over the same kind of chunks: recount the chunk, reserve each
-// touched box's range with one global atomic, then place the points with
-// shared-memory atomics.
-__global__ void __launch_bounds__(kBinThreads) bin_scatter_smem_kernel(int g, const double* __restrict__ y, int64_t n,
-                                                                       int64_t chunk, int* __restrict__ cursor,
-                                                                       int* __restrict__ perm)
+// The scatter over chunks of up to LOADS points a thread: the counting addition gives a point
+// its rank among the block's points of its box, which the thread keeps; the block reserves each
+// touched box's range with one global atomic, and a point goes to that range's start + rank.  The
+// coordinates are read once, with one shared atomic a point (a second pass over both before).
+template <int T, int LOADS>
+__global__ void __launch_bounds__(T) bin_scatter_smem_kernel(int g, const double* __restrict__ y, int64_t n, int64_t chunk,
+                                                             int* __restrict__ cursor, int* __restrict__ perm)
 {
     after_go();
     extern __shared__ int s_cnt[];
     const int nbox = 1 << (2 * g);
-    for (int b = threadIdx.x; b < nbox; b += kBinThreads) s_cnt[b] = 0;
+    for (int b = threadIdx.x; b < nbox; b += T) s_cnt[b] = 0;
     after_wait();
     __syncthreads();
-    const int64_t i0 = (int64_t)blockIdx.x * chunk, i1 = i0 + chunk < n ? i0 + chunk : n;
-    for_boxes(y, g, i0 + threadIdx.x, i1, [&](int64_t, int b) { atomicAdd(&s_cnt[b], 1); });
+    const int64_t i0 = (int64_t)blockIdx.x * chunk, i1 = i0 + chunk < n ? i0 + chunk : n, i = i0 + threadIdx.x;
+    double a[LOADS], b[LOADS];
+    load_points<T, LOADS>(y, i, i1, a, b);
+    int box[LOADS], rank[LOADS];
+#pragma unroll
+    for (int u = 0; u < LOADS; ++u) {
+        box[u] = fgt_grid_box(a[u], b[u], g);
+        if (i + u * T < i1) rank[u] = atomicAdd(&s_cnt[box[u]], 1);
+    }
     __syncthreads();
-    for (int b = threadIdx.x; b < nbox; b += kBinThreads)
-        if (s_cnt[b]) s_cnt[b] = atomicAdd(&cursor[b], s_cnt[b]);  // this block's first slot in box b
+    for (int c = threadIdx.x; c < nbox; c += T)
+        if (s_cnt[c]) s_cnt[c] = atomicAdd(&cursor[c], s_cnt[c]);  // this block's first slot in box c
     __syncthreads();
-    for_boxes(y, g, i0 + threadIdx.x, i1, [&](int64_t i, int b) { perm[atomicAdd(&s_cnt[b], 1)] = (int)i; });
+#pragma unroll
+    for (int u = 0; u < LOADS; ++u)
+        if (i + u * T < i1) perm[s_cnt[box[u]] + rank[u]] = (int)(i + u * T);
 }
 
 static int bin_grid(int64_t n)
@@ -916,21 +933,39 @@ extern "C" int fgt_bin_points(int32_t grid_log2, const double* y, int64_t n, int
     FMM_CUDA_TRY(cudaMemsetAsync(work, 0, sizeof(int) * (size_t)nbox, st));
     const bool smem = grid_log2 <= kBinSmemMaxLog2;
     const int smem_bytes = smem ? (int)sizeof(int) * nbox : 0;
+    // 0: 256 threads x 4 points, 1: 512 x 8, 2: 1024 x 4 (the lines: above the kernels)
+    const int form = grid_log2 >= 6 && n >= 1 << 15 ? 2 : grid_log2 < 6 && n >= 1 << 19 ? 1 : 0;
+    const int threads = 256 << form, most = form ? 4096 : 1024;
+    using Count = void (*)(int, const double*, int64_t, int64_t, int*);
+    using Scatter = void (*)(int, const double*, int64_t, int64_t, int*, int*);
+    static constexpr Count counts[] = {bin_count_smem_kernel<256, 4>, bin_count_smem_kernel<512, 8>,
+                                        bin_count_smem_kernel<1024, 4>};
+    static constexpr Scatter scatters[] = {bin_scatter_smem_kernel<256, 4>, bin_scatter_smem_kernel<512, 8>,
+                                           bin_scatter_smem_kernel<1024, 4>};
     int grid = bin_grid(n);
     int64_t chunk = 0;
     if (smem && n > 0) {
-        static unsigned long long opted[2];  // opted in once per device, for the largest such grid
-        constexpr int kMaxBytes = (int)sizeof(int) << (2 * kBinSmemMaxLog2);
-        if (int rc = smem_opt_in((const void*)bin_count_smem_kernel, kMaxBytes, &opted[0])) return rc;
-        if (int rc = smem_opt_in((const void*)bin_scatter_smem_kernel, kMaxBytes, &opted[1])) return rc;
+        // every form opted in by the first call on a device, for the largest such grid: no later call,
+        // in a capture or not, is a form's first
+        static unsigned long long all, opted[3][2];
+        int dev = 0;
+        FMM_CUDA_TRY(cudaGetDevice(&dev));
+        if (dev < 0 || dev >= 64 || !(__atomic_load_n(&all, __ATOMIC_ACQUIRE) >> dev & 1)) {
+            constexpr int kMaxBytes = (int)sizeof(int) << (2 * kBinSmemMaxLog2);
+            for (int f = 0; f < 3; ++f) {
+                if (int rc = smem_opt_in((const void*)counts[f], kMaxBytes, &opted[f][0])) return rc;
+                if (int rc = smem_opt_in((const void*)scatters[f], kMaxBytes, &opted[f][1])) return rc;
+            }
+            __atomic_fetch_or(&all, 1ull << dev, __ATOMIC_RELEASE);
+        }
         int sms = 0;
         if (device_sm_count(&sms) || sms <= 0) sms = 148;
-        grid = (int)std::min<int64_t>(2LL * sms, (n + kBinThreads - 1) / kBinThreads);
+        grid = (int)std::min<int64_t>(2LL * sms, (n + threads - 1) / threads);
         chunk = (n + grid - 1) / grid;
     }
     if (n > 0) {
         if (smem)
-            bin_count_smem_kernel<<<grid, kBinThreads, smem_bytes, st>>>(grid_log2, y, n, chunk, work);
+            counts[form]<<<grid, threads, smem_bytes, st>>>(grid_log2, y, n, chunk, work);
         else
             bin_count_kernel<<<grid, kBinThreads, 0, st>>>(grid_log2, y, n, work);
         FMM_CUDA_TRY(cudaGetLastError());
@@ -942,11 +977,13 @@ extern "C" int fgt_bin_points(int32_t grid_log2, const double* y, int64_t n, int
         FMM_CUDA_TRY(cudaMemcpyAsync(work, box_start, sizeof(int) * (size_t)nbox, cudaMemcpyDeviceToDevice, st));
     }
     if (n > 0) {
-        if (smem)
-            FMM_CUDA_TRY(launch_after(bin_scatter_smem_kernel, grid, kBinThreads, smem_bytes, st, grid_log2, y, n, chunk,
-                                      work, perm));
-        else
+        if (smem) {
+            chunk = std::min<int64_t>(chunk, most);  // points of a scatter block
+            FMM_CUDA_TRY(launch_after(scatters[form], (unsigned)((n + chunk - 1) / chunk), threads, smem_bytes, st, grid_log2, y, n,
+                                      chunk, work, perm));
+        } else {
             FMM_CUDA_TRY(launch_after(bin_scatter_kernel, grid, kBinThreads, 0, st, grid_log2, y, n, work, perm));
+        }
     }
     return FMM_OK;
 }

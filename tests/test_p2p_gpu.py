@@ -288,3 +288,20 @@ def test_p2p_short_lived_blocks_equal_persistent_ones(fmm, level, per_box):
         out.append(phi)
     for phi in out[1:]:
         assert torch.equal(torch.view_as_real(phi), torch.view_as_real(out[0]))
+
+
+@pytest.mark.parametrize("level", [0, 3, 7])
+@pytest.mark.parametrize("n", [1, 257, 32767, 32768, 4097 * 304, 1_300_001])
+def test_binning_at_the_edges_of_its_blocks(fmm, level, n):
+    """Both block widths, chunks of every length up to four points a thread and more blocks than
+    that: the boxes' counts, and every point once in its own box."""
+    import torch
+
+    g = torch.Generator(device="cuda").manual_seed(n)
+    pts = torch.rand((n, 2), dtype=torch.float64, device="cuda", generator=g) ** 2
+    perm, start = _bins(fmm, level, pts)
+    ix = (pts * 2 ** level).floor().long()
+    box = ix[:, 1] * 2 ** level + ix[:, 0]
+    assert torch.equal(torch.diff(start).long(), torch.bincount(box, minlength=4 ** level))
+    assert torch.equal(box[perm.long()], torch.sort(box).values)
+    assert torch.equal(torch.sort(perm).values.long(), torch.arange(n, device="cuda"))
