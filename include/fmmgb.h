@@ -574,10 +574,10 @@ int fgt_t2p_binned(int32_t grid_log2, int32_t p, double sigma, const float* C, c
  *   y, n, ...) of these targets; G: device float32 [n], indexed like y.
  *   n_cut 0..16, p 4, 8, 12 or 16, flags FMM_ACCUMULATE or 0.
  *   With two targets per box or more on average, grid_log2 <= 8 and a box side d =
- *   2^-g / (sqrt2 sigma) of up to 1.3 (p = 16; more below), every prec is served in FP32 on
- *   the CUDA cores through Chebyshev coefficients of each target box (12 or 16 per
- *   dimension, interpolation error below 3e-8 of a Hermite function's size): the sums over
- *   source boxes are taken once per target box.  Their workspace, 2 KiB per box, is allocated
+ *   2^-g / (sqrt2 sigma) of up to 1/2, every prec is served in FP32 on
+ *   the CUDA cores through Chebyshev coefficients of each target box (12 per dimension,
+ *   interpolation error below 4e-10 of a Hermite function's largest value): the sums over
+ *   source boxes are taken once per target box.  Their workspace, 1.3 KiB per box, is allocated
  *   per grid size and device on the first such call and kept; a first such call inside a
  *   stream capture takes the direct sums below instead, as every other call does.  Calls that
  *   overlap on the GPU share the workspace and must be serialised by the caller.

@@ -14,11 +14,14 @@
 //
 // Error.  The interpolant of h_a differs from it by at most
 //   2 (d/4)^Q / Q! max |h_a^(Q)|,  |h_a^(Q)| = |h_(a+Q)| <= 1.09 sqrt(2^(a+Q) (a+Q)!)
-// (Cramer's inequality), so relative to h_a's own size, 1.09 sqrt(2^a a!), by
-//   2 (d/4)^Q sqrt(2^Q (a+Q)!/a!) / Q!.
-// cheb_order takes the smallest Q of 12 and 16 that keeps this below 3e-8, half a unit of FP32's
-// last place, at a = p - 1 (Q = 12 for every grid with d <= 1/2 at p = 16; the bound is 4e-10
-// there); wider boxes keep the direct sum.  The sums are FP32, as in the direct kernel.
+// (Cramer's inequality), so relative to h_a's own largest value, 1.09 sqrt(2^a a!), by
+//   2 (d/4)^Q sqrt(2^Q (a+Q)!/a!) / Q!,
+// 4e-10 for Q = 12, a = 15 and d = 1/2, the widest box that is taken.  That bound, and the FP32
+// rounding of a box's sums, are relative to the largest values in the box; a target's own value can be
+// smaller: over a box k boxes away h(u + k d) falls by about exp(2 k d^2) in each dimension.  So
+// wider boxes keep the direct sum, which is accurate target by target (one source box (4, 4) boxes
+// away, d = 0.95, 99 of 100 targets: 4e-6 of their values direct, 3e-3 through 16 nodes).  The sums are FP32,
+// as in the direct kernel.
 //
 // Measured at p = 16, n_cut = 10: 2^20 clustered targets, 32 x 32 boxes (263.6M target-box pairs)
 // 2,350 us direct -> 46 us (table 6, contractions 7 and 6, evaluation 26, which is bound by the
@@ -29,11 +32,10 @@
 // 173 -> 169 us for the whole transform.
 //
 // The rule's other lines: at least 2 targets per box on average (the contractions cost a box
-// what the direct sum costs ~1 target) and grids of up to 256 x 256 boxes (128 MB of
+// what the direct sum costs ~1 target) and grids of up to 256 x 256 boxes (88 MB of
 // workspace; one allocation per grid size and device, kept).  A target outside its box
 // (coordinates outside the unit square, or a binning that assigns it elsewhere) is summed
 // directly.
-#include <cmath>
 #include <mutex>
 
 #include "fgt_hermite.cuh"
@@ -42,20 +44,9 @@ namespace fmmgb {
 
 constexpr int kChebMaxLog2 = 8;
 constexpr int kChebMaxCut = 16;
-constexpr int kChebMaxQ = 16;
-constexpr size_t kChebTableFloats = (size_t)(2 * kChebMaxCut + 1) * 16 * kChebMaxQ;
-
-// Nodes per dimension for order p and box side d (in sqrt2 sigma), 0: none keeps the bound.
-int cheb_order(int p, double d)
-{
-    for (int q : {12, 16}) {
-        // log of 2 (d/4)^q sqrt(2^q (p-1+q)! / (p-1)!) / q!
-        const double e = log(2.0) + q * log(0.25 * d) +
-                         0.5 * (q * log(2.0) + lgamma((double)(p + q)) - lgamma((double)p)) - lgamma(q + 1.0);
-        if (e <= log(3e-8)) return q;
-    }
-    return 0;
-}
+constexpr int kChebQ = 12;           // nodes per dimension
+constexpr double kChebMaxSide = 0.5;  // widest box, in sqrt2 sigma
+constexpr size_t kChebTableFloats = (size_t)(2 * kChebMaxCut + 1) * 16 * kChebQ;
 
 // W[k][a][m], k = 0..2 ncut for the offset (k - ncut) d: one CTA per offset, FP64.
 template <int P, int Q>
@@ -373,7 +364,7 @@ __global__ void __launch_bounds__(kEvalThreads) cheb_eval_kernel(ChebEval a)
         if (tj[r] >= 0) a.G[tj[r]] = a.accumulate ? a.G[tj[r]] + out[r] : out[r];
 }
 
-// Per device and grid size: table | X [4^g][16][16] | C [4^g][16][16], allocated on first use and
+// Per device and grid size: table | X [4^g][16][12] | C [4^g][12][12], allocated on first use and
 // kept (captured graphs hold its address).  NULL, without an error, when it would have to be
 // allocated inside a stream capture.
 static int cheb_workspace(int g, cudaStream_t st, float** out)
@@ -389,7 +380,7 @@ static int cheb_workspace(int g, cudaStream_t st, float** out)
         cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
         FMM_CUDA_TRY(cudaStreamIsCapturing(st, &cs));
         if (cs != cudaStreamCaptureStatusNone) return FMM_OK;
-        const size_t bytes = (kChebTableFloats + ((size_t)2 * 16 * kChebMaxQ << (2 * g))) * sizeof(float);
+        const size_t bytes = (kChebTableFloats + ((size_t)(16 + kChebQ) * kChebQ << (2 * g))) * sizeof(float);
         if (cudaMalloc(&buf[dev][g], bytes) != cudaSuccess) {
             (void)cudaGetLastError();
             buf[dev][g] = nullptr;
@@ -400,13 +391,13 @@ static int cheb_workspace(int g, cudaStream_t st, float** out)
     return FMM_OK;
 }
 
-template <int P, int Q>
+template <int P, int Q = kChebQ>
 static int cheb_launch(const ChebEval& e, float* ws, cudaStream_t st)
 {
     using C1 = ChebPass<P, P, Q>;
     using C2 = ChebPass<P, Q, Q>;
     const int side = 1 << e.g;
-    float *W = ws, *X = W + kChebTableFloats, *C = X + ((size_t)16 * kChebMaxQ << (2 * e.g));
+    float *W = ws, *X = W + kChebTableFloats, *C = X + ((size_t)16 * kChebQ << (2 * e.g));
     static unsigned long long opted[2];
     if (int rc = smem_opt_in((const void*)cheb_pass_kernel<P, P, Q>, (int)C1::smem(kChebMaxCut), &opted[0])) return rc;
     if (int rc = smem_opt_in((const void*)cheb_pass_kernel<P, Q, Q>, (int)C2::smem(kChebMaxCut), &opted[1])) return rc;
@@ -425,18 +416,17 @@ int launch_fgt_h2p_cheb(int g, int ncut, int p, double d, const float* A, const 
                         const int* box_start, float* G, bool accumulate, int* err, cudaStream_t st, bool* done)
 {
     *done = false;
-    const int q = cheb_order(p, d);
-    if (!q || g > kChebMaxLog2 || n < (2 << (2 * g))) return FMM_OK;
+    if (d > kChebMaxSide || g > kChebMaxLog2 || n < (2 << (2 * g))) return FMM_OK;
     float* ws = nullptr;
     if (int rc = cheb_workspace(g, st, &ws)) return rc;
     if (!ws) return FMM_OK;
     *done = true;
     const ChebEval e{g, ncut, n, accumulate ? 1 : 0, d, A, nullptr, y, perm, box_start, G, err};
     switch (p) {
-        case 4: return q == 12 ? cheb_launch<4, 12>(e, ws, st) : cheb_launch<4, 16>(e, ws, st);
-        case 8: return q == 12 ? cheb_launch<8, 12>(e, ws, st) : cheb_launch<8, 16>(e, ws, st);
-        case 12: return q == 12 ? cheb_launch<12, 12>(e, ws, st) : cheb_launch<12, 16>(e, ws, st);
-        default: return q == 12 ? cheb_launch<16, 12>(e, ws, st) : cheb_launch<16, 16>(e, ws, st);
+        case 4: return cheb_launch<4>(e, ws, st);
+        case 8: return cheb_launch<8>(e, ws, st);
+        case 12: return cheb_launch<12>(e, ws, st);
+        default: return cheb_launch<16>(e, ws, st);
     }
 }
 

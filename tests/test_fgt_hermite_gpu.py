@@ -374,7 +374,7 @@ def test_h2p_tc_agrees_with_fp32_path_at_full_size(fmm, orc):
 
 # ---------------------------------------------------------------------------
 # evaluation through per-box Chebyshev coefficients: taken at >= 2 targets per box on average, on
-# grids up to 256 x 256, for box sides whose interpolation bound holds
+# grids up to 256 x 256, for box sides of up to 1/2 (in sqrt2 sigma)
 # ---------------------------------------------------------------------------
 def _decaying(rng, nbox, p):
     import math
@@ -387,13 +387,13 @@ def _decaying(rng, nbox, p):
 
 
 @pytest.mark.parametrize("p,d", [(4, 0.5), (8, 0.4), (8, 0.95), (12, 0.79), (12, 0.82), (16, 0.26), (16, 0.72),
-                                 (16, 0.73), (16, 1.29), (16, 1.31)])
+                                 (16, 0.73), (16, 1.29), (16, 1.31), (16, 0.5), (16, 0.501)])
 def test_h2p_on_both_sides_of_the_chebyshev_rule(fmm, orc, p, d):
-    """Box sides d (in sqrt2 sigma) on both sides of the lines where 12 nodes, 16 nodes and the
-    direct sum are taken, and target counts on both sides of two per box; targets on box edges,
+    """Box sides d (in sqrt2 sigma) on both sides of the line (1/2) between the coefficients and the
+    direct sum, and target counts on both sides of two per box; targets on box edges,
     at 1.0 and outside the unit square (summed directly), and crowded into one box.  The bar is
-    the FP32 bar of the direct kernel: the interpolation adds at most 3e-8 of a Hermite function's
-    own size, against sums rounded to ~1e-7."""
+    the FP32 bar of the direct kernel: the interpolation adds at most 4e-10 of a Hermite function's
+    largest value, against sums rounded to ~1e-7."""
     import math
 
     g = 3
@@ -428,6 +428,40 @@ def test_h2p_chebyshev_grid_sizes(fmm, orc, g):
     got = _h2p(fmm, g, ncut, p, sigma, A32, y, G=G, accumulate=True)
     pick = rng.choice(len(y), min(800, len(y)), replace=False)
     _check(got[pick], orc.fgt_hermite_eval_grid(g, ncut, p, sigma, A32.astype(np.float64), y[pick]) + 0.25)
+
+
+def _per_target_terms(g, sigma, A, box, y):
+    """Sum over one source box of |A_a1a2 h_a1(t1) h_a2(t2)| at each target, and t1^2 + t2^2, in 64 bits."""
+    p, n = A.shape[-1], 1 << g
+    t = (y - (np.array([box % n, box // n]) + 0.5) / n) / (np.sqrt(2.0) * sigma)
+    h = [np.exp(-t * t), 2 * t * np.exp(-t * t)]
+    for m in range(1, p - 1):
+        h.append(2 * t * h[m] - 2 * m * h[m - 1])
+    h = np.abs(np.stack(h[:p]))
+    return np.einsum("ab,an,bn->n", np.abs(A.astype(np.float64)), h[:, :, 0], h[:, :, 1]), (t * t).sum(1)
+
+
+@pytest.mark.parametrize("p,d,g", [(16, 0.6, 3), (16, 1.0, 3), (16, 1.28, 3), (8, 0.95, 3), (12, 0.8, 3), (4, 1.9, 2)])
+def test_h2p_each_target_keeps_its_own_accuracy(fmm, orc, p, d, g):
+    """Sources in one corner box alone, targets all over the grid, down to values of 1e-30: each
+    target's error against the size of its own terms, not of the largest target's.  FP32: t1^2 + t2^2
+    are the exponents, whose rounding (two roundings of the argument, one of its scaling to a power of
+    2, each 2^-24 relative) is an absolute error of the logarithm; p-term recurrences and sums on both
+    axes and the function's own error: (4 p + 32 + 4 (t1^2 + t2^2)) units of 2^-24 (a 32-bit emulation
+    of the direct sum reaches 0.46 of that)."""
+    import math
+
+    n, rng = 1 << g, np.random.default_rng(int(100 * d) + p)
+    sigma = 2.0 ** -g / (math.sqrt(2.0) * d)
+    x = rng.random((60, 2)) / n
+    A32 = orc.fgt_p2h_grid(g, p, sigma, x, rng.random(60)).astype(np.float32)
+    y = rng.random((max(1500, 4 * n * n), 2))
+    ref = orc.fgt_hermite_eval_grid(g, 16, p, sigma, A32.astype(np.float64), y)
+    size, t2 = _per_target_terms(g, sigma, A32[0], 0, y)
+    got = _h2p(fmm, g, 16, p, sigma, A32, y)
+    ok = size > 1e-30
+    over = (np.abs(got - ref) / ((4 * p + 32 + 4 * t2) * 2.0 ** -24 * size))[ok]
+    assert over.max() <= 1.0, f"{over.max():.3g} of the bound, {int((over > 1).sum())} targets above it"
 
 
 def test_h2p_nan_coefficients_reach_their_neighbourhood_only(fmm, orc):
