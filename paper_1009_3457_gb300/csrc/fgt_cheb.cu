@@ -176,38 +176,73 @@ struct ChebEval {
     int* err;
 };
 
-// The direct sum for one target assigned to box (tx, ty), as the direct kernel takes it: every
-// source box of the neighbourhood that holds a non-zero coefficient.
+// The direct sum for one target assigned to `box`, as the direct kernel takes it (a source box without
+// a non-zero coefficient adds nothing): source boxes first, first + step, ... of the neighbourhood.
 template <int P>
-__device__ __noinline__ float cheb_direct(const ChebEval& a, int tx, int ty, double y0, double y1)
+__device__ __noinline__ float cheb_direct(const ChebEval& a, int box, double y0, double y1, int first, int step)
 {
-    const int side = 1 << a.g;
+    const int side = 1 << a.g, tx = box & (side - 1), ty = box >> a.g;
+    const int sx0 = max(tx - a.ncut, 0), w = min(tx + a.ncut, side - 1) - sx0 + 1;
+    const int sy0 = max(ty - a.ncut, 0), nb = w * (min(ty + a.ncut, side - 1) - sy0 + 1);
     const float u1 = (float)((y0 * side - (tx + 0.5)) * a.d), u2 = (float)((y1 * side - (ty + 0.5)) * a.d);
-    float acc = 0.f;
-    for (int sy = max(ty - a.ncut, 0); sy <= min(ty + a.ncut, side - 1); ++sy) {
-        float h2[P];
-        hermite_functions<P>(u2 + (float)((double)(ty - sy) * a.d), h2);
-        for (int sx = max(tx - a.ncut, 0); sx <= min(tx + a.ncut, side - 1); ++sx) {
-            float h1[P];
-            hermite_functions<P>(u1 + (float)((double)(tx - sx) * a.d), h1);
-            const float* Ab = a.A + ((size_t)sy * side + sx) * P * P;
-            bool nz = false;
-            float s = 0.f;
-#pragma unroll
-            for (int a1 = 0; a1 < P; ++a1) {
-                float t = 0.f;
-#pragma unroll
-                for (int a2 = 0; a2 < P; ++a2) {
-                    const float v = Ab[a1 * P + a2];
-                    nz |= v != 0.f;
-                    t = fmaf(v, h2[a2], t);
-                }
-                s = fmaf(h1[a1], t, s);
-            }
-            if (nz) acc += s;
+    float acc = 0.f, h2[P];
+    int row = -1;
+#pragma unroll 1
+    for (int i = first; i < nb; i += step) {
+        const int sx = sx0 + i % w, sy = sy0 + i / w;
+        if (sy != row) {
+            row = sy;
+            hermite_functions<P>(u2 + (float)((double)(ty - sy) * a.d), h2);
         }
+        // Clenshaw's backward recurrence over a1 for h_(a+1) = 2t h_a - 2a h_(a-1)
+        const float t1 = u1 + (float)((double)(tx - sx) * a.d), tt = t1 + t1;
+        const float4* Ab = reinterpret_cast<const float4*>(a.A + ((size_t)sy * side + sx) * P * P);
+        bool nz = false;
+        float c1 = 0.f, c2 = 0.f;
+#pragma unroll
+        for (int a1 = P - 1; a1 >= 0; --a1) {
+            float t = fmaf(tt, c1, -(float)(2 * (a1 + 1)) * c2);
+#pragma unroll
+            for (int q = 0; q < P / 4; ++q) {
+                const float4 v = __ldg(Ab + a1 * (P / 4) + q);
+                nz |= v.x != 0.f || v.y != 0.f || v.z != 0.f || v.w != 0.f;
+                t = fmaf(v.x, h2[4 * q], t);
+                t = fmaf(v.y, h2[4 * q + 1], t);
+                t = fmaf(v.z, h2[4 * q + 2], t);
+                t = fmaf(v.w, h2[4 * q + 3], t);
+            }
+            c2 = c1;
+            c1 = t;
+        }
+        if (nz) acc = fmaf(__expf(-t1 * t1), c1, acc);
     }
     return acc;
+}
+
+// The direct sums of a warp's targets (box < 0: none).  A few take the whole warp one after another, a
+// share of the source boxes a lane; many take a lane each.  2^20 targets on 32 x 32 boxes, n_cut = 10,
+// 61 us with none outside the unit square: with one 1,842 us a lane each always, 86 us so; with one in a
+// hundred (crowded into the edge boxes) 7.4 ms and 2.7 ms, where the direct kernel takes 4.4 ms for all.
+constexpr int kApartShared = 15;
+template <int P>
+__device__ __noinline__ float cheb_apart(const ChebEval& a, int box, double y0, double y1)
+{
+    unsigned todo = __ballot_sync(0xffffffffu, box >= 0);
+    float out = 0.f;
+    if (__popc(todo) > kApartShared) {
+        if (box >= 0) out = cheb_direct<P>(a, box, y0, y1, 0, 1);
+        return out;
+    }
+    const int lane = threadIdx.x & 31;
+    for (; todo; todo &= todo - 1) {
+        const int l = __ffs(todo) - 1;
+        float s = cheb_direct<P>(a, __shfl_sync(0xffffffffu, box, l), __shfl_sync(0xffffffffu, y0, l),
+                                 __shfl_sync(0xffffffffu, y1, l), lane, 32);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == l) out = s;
+    }
+    return out;
 }
 
 // sum_{m,l} c[m][l] T_m(x1) T_l(x2) for NR targets of one box (or, with NR = 1, of a box per lane).
@@ -339,17 +374,22 @@ __global__ void __launch_bounds__(kEvalThreads) cheb_eval_kernel(ChebEval a)
                     b = tb[k];
                     j = tj[k];
                 }
-            if (b >= 0) {
-                cheb_sum<Q, 1>(a.C + (size_t)b * Q * Q, &u1, &u2, &v);
-            } else if (j >= 0) {
-                const int lo = bin_find(a.box_start, nbox, (int)(base + 32 * r + lane), a.n);  // the assigned box
-                if (lo >= 0) {
-                    v = cheb_direct<P>(a, lo & (side - 1), lo >> a.g, __ldg(a.y + 2 * (size_t)j),
-                                       __ldg(a.y + 2 * (size_t)j + 1));
-                } else {  // box_start does not bin [0, n)
-                    atomicOr(a.err, DEV_ERR_CHECK);
-                    j = -1;
+            if (b >= 0) cheb_sum<Q, 1>(a.C + (size_t)b * Q * Q, &u1, &u2, &v);
+            if (__any_sync(0xffffffffu, b < 0 && j >= 0)) {
+                int lo = -1;  // the assigned box
+                double y0 = 0.0, y1 = 0.0;
+                if (b < 0 && j >= 0) {
+                    lo = bin_find(a.box_start, nbox, (int)(base + 32 * r + lane), a.n);
+                    if (lo >= 0) {
+                        y0 = __ldg(a.y + 2 * (size_t)j);
+                        y1 = __ldg(a.y + 2 * (size_t)j + 1);
+                    } else {  // box_start does not bin [0, n)
+                        atomicOr(a.err, DEV_ERR_CHECK);
+                        j = -1;
+                    }
                 }
+                const float w = cheb_apart<P>(a, lo, y0, y1);
+                if (lo >= 0) v = w;
             }
 #pragma unroll
             for (int k = 0; k < kRows; ++k)

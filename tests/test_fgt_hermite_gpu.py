@@ -430,6 +430,25 @@ def test_h2p_chebyshev_grid_sizes(fmm, orc, g):
     _check(got[pick], orc.fgt_hermite_eval_grid(g, ncut, p, sigma, A32.astype(np.float64), y[pick]) + 0.25)
 
 
+@pytest.mark.parametrize("p", [4, 8, 12, 16])
+@pytest.mark.parametrize("g,k", [(1, 1), (1, 10), (1, 15), (1, 16), (1, 40), (3, 150), (5, 3)])
+def test_h2p_targets_outside_the_unit_square(fmm, orc, p, g, k):
+    """k targets outside the unit square (the nearest box's, summed directly) among those of the boxes:
+    few of a warp's targets (the warp shares the source boxes of each) and many (a lane each), with
+    neighbourhoods of one box and of the whole grid."""
+    import math
+
+    rng = np.random.default_rng(100 * g + k)
+    sigma = 2.0 ** -g / (math.sqrt(2.0) * 0.45)
+    A32 = _decaying(rng, 4 ** g, p)
+    y = rng.random((max(32 - k, 4 * 4 ** g), 2))
+    out = rng.choice(len(y), min(k, len(y)), replace=False)
+    y[out, 0] = np.where(rng.random(len(out)) < 0.5, 1.0 + 0.05 * rng.random(len(out)), -0.05 * rng.random(len(out)))
+    for ncut in (0, 16):
+        _check(_h2p(fmm, g, ncut, p, sigma, A32, y),
+               orc.fgt_hermite_eval_grid(g, ncut, p, sigma, A32.astype(np.float64), y))
+
+
 def _per_target_terms(g, sigma, A, box, y):
     """Sum over one source box of |A_a1a2 h_a1(t1) h_a2(t2)| at each target, and t1^2 + t2^2, in 64 bits."""
     p, n = A.shape[-1], 1 << g
