@@ -577,7 +577,9 @@ int fgt_t2p_binned(int32_t grid_log2, int32_t p, double sigma, const float* C, c
  *   2^-g / (sqrt2 sigma) of up to 1/2, every prec is served in FP32 on
  *   the CUDA cores through Chebyshev coefficients of each target box (12 per dimension,
  *   interpolation error below 4e-10 of a Hermite function's largest value): the sums over
- *   source boxes are taken once per target box.  Their workspace, 1.3 KiB per box, is allocated
+ *   source boxes are taken once per target box.  Targets outside the unit square, and
+ *   boxes over which the field falls by more than e^5 (sources far away only), are summed
+ *   directly in the same call, so that each value keeps its own FP32 accuracy.  The workspace, 1.4 KiB per box, is allocated
  *   per grid size and device on the first such call and kept; a first such call inside a
  *   stream capture takes the direct sums below instead, as every other call does.  Calls that
  *   overlap on the GPU share the workspace and must be serialised by the caller.

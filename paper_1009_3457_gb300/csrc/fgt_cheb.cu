@@ -20,8 +20,16 @@
 // rounding of a box's sums, are relative to the largest values in the box; a target's own value can be
 // smaller: over a box k boxes away h(u + k d) falls by about exp(2 k d^2) in each dimension.  So
 // wider boxes keep the direct sum, which is accurate target by target (one source box (4, 4) boxes
-// away, d = 0.95, 99 of 100 targets: 4e-6 of their values direct, 3e-3 through 16 nodes).  The sums are FP32,
-// as in the direct kernel.
+// away, d = 0.95, 99 of 100 targets: 4e-6 of their values direct, 3e-3 through 16 nodes), and so do the
+// boxes that the sources reach from afar only (d = 1/2, (10, 10) boxes away: 6e-6 direct, 2e-4).
+// The contractions carry two limits of ln |field| over each target box besides, with m_B the largest
+// coefficient of a source box: max_B (ln m_B - r^2) for the distance r to B's centre of the
+// box's nearest point and of its farthest, per axis (|k| -+ 1/2) d.  Boxes where they lie more than
+// kChebLoss apart are listed and summed directly.  In 32-bit emulation of random
+// source boxes (1 to 6 of them up to 10 away, strengths over 8 decades) the rms error relative to a target's
+// own terms is at most the direct sum's up to 5 (at 4 to 5: 3.2e-7 against 6.7e-7, d = 0.44; at 6 to 8 2.9e-6
+// against 1.3e-6).
+// The sums are FP32, as in the direct kernel.
 //
 // Measured at p = 16, n_cut = 10: 2^20 clustered targets, 32 x 32 boxes (263.6M target-box pairs)
 // 2,350 us direct -> 46 us (table 6, contractions 7 and 6, evaluation 26, which is bound by the
@@ -35,7 +43,8 @@
 // what the direct sum costs ~1 target) and grids of up to 256 x 256 boxes (88 MB of
 // workspace; one allocation per grid size and device, kept).  A target outside its box
 // (coordinates outside the unit square, or a binning that assigns it elsewhere) is summed
-// directly.
+// directly too.
+#include <algorithm>
 #include <mutex>
 
 #include "fgt_hermite.cuh"
@@ -46,15 +55,44 @@ constexpr int kChebMaxLog2 = 8;
 constexpr int kChebMaxCut = 16;
 constexpr int kChebQ = 12;           // nodes per dimension
 constexpr double kChebMaxSide = 0.5;  // widest box, in sqrt2 sigma
+constexpr float kChebLoss = 5.f;      // largest fall of ln |field| over a box (see above)
 constexpr size_t kChebTableFloats = (size_t)(2 * kChebMaxCut + 1) * 16 * kChebQ;
 
-// W[k][a][m], k = 0..2 ncut for the offset (k - ncut) d: one CTA per offset, FP64.
+// What the contractions and the listed boxes read (see above).
+struct ChebLimits {
+    float2* box;           // [sy][sx]: ln of the largest |coefficient| of the source box, twice
+    float2* line;          // [tx][sy]: the limits contracted along x, (nearest, farthest)
+    unsigned char* nz;     // [box] any non-zero coefficient
+    unsigned char* apart;  // [box] summed directly
+    H2pList list;
+};
+
+// The first 2 ncut + 1 CTAs: W[k][a][m] for the offset (k - ncut) d, one CTA each, FP64.  The others:
+// the source boxes' l.box and l.nz, a warp each.
 template <int P, int Q>
-__global__ void __launch_bounds__(256) cheb_table_kernel(int ncut, double d, float* __restrict__ W)
+__global__ void __launch_bounds__(256) cheb_table_kernel(int ncut, double d, int nbox, const float* A, float* __restrict__ W,
+                                                         ChebLimits l)
 {
     __shared__ double s_h[P][Q], s_cos[4 * Q];
     const int tid = threadIdx.x, k = blockIdx.x;
     after_go();
+    if (k > 2 * ncut) {
+        after_wait();
+        const int b = (k - 2 * ncut - 1) * 8 + tid / 32, lane = tid % 32;
+        if (b >= nbox) return;
+        unsigned m = 0;
+        for (int i = lane; i < P * P / 4; i += 32) {
+            const float4 v = reinterpret_cast<const float4*>(A + (size_t)b * P * P)[i];
+            m = max(m, max(max(__float_as_uint(v.x) & 0x7FFFFFFFu, __float_as_uint(v.y) & 0x7FFFFFFFu),
+                           max(__float_as_uint(v.z) & 0x7FFFFFFFu, __float_as_uint(v.w) & 0x7FFFFFFFu)));
+        }
+        m = __reduce_max_sync(0xffffffffu, m);
+        if (lane) return;
+        const float ln = m < 0x7F800000u ? logf(__uint_as_float(m)) : INFINITY;  // infinite: not finite
+        l.box[b] = make_float2(ln, ln);
+        l.nz[b] = m != 0;
+        return;
+    }
     if (tid < 4 * Q) s_cos[tid] = cospi((double)tid / (2.0 * Q));
     __syncthreads();
     if (tid < Q) {
@@ -70,7 +108,8 @@ __global__ void __launch_bounds__(256) cheb_table_kernel(int ncut, double d, flo
         }
     }
     __syncthreads();
-    after_wait();  // an earlier call may still read the table
+    after_wait();  // an earlier call may still read the table and the list
+    if (k == 0 && tid == 0) *l.list.count = 0;
     for (int e = tid; e < P * Q; e += 256) {
         const int a = e / Q, m = e % Q;
         double s = 0.0;
@@ -86,8 +125,11 @@ __global__ void __launch_bounds__(256) cheb_table_kernel(int ncut, double d, flo
 // kSeg + 2 n_cut source boxes and the table; a thread owns (box, r) and all Q outputs, over
 // every kTaps-th tap, so a step is one scalar and Q/4 broadcast 16-byte shared loads for Q
 // multiply-adds; the taps' sums are added in registers and the groups' meet in shared memory.
+// The limits of ln |field| (see above) are contracted beside them, max for sum: along x from l.box into
+// l.line, along y (LAST) into the list of the boxes summed directly, whose first coefficient becomes NaN.
 constexpr int kSeg = 4;
 constexpr int kTaps = 4;
+constexpr int kEvalThreads = 128;  // of the evaluation's CTAs, and targets of a listed box per claim
 
 template <int P, int R, int Q>
 struct ChebPass {
@@ -101,10 +143,20 @@ struct ChebPass {
     }
 };
 
-template <int P, int R, int Q>
-__global__ void __launch_bounds__(kSeg* kTaps* R)
-    cheb_pass_kernel(int side, int ncut, const float* __restrict__ in, const float* __restrict__ W, float* __restrict__ out)
+// The order of floats as that of integers (NaN aside), and back.
+__device__ __forceinline__ int float_key(float x)
 {
+    const int i = __float_as_int(x);
+    return i ^ (i >> 31 & 0x7FFFFFFF);
+}
+
+template <int P, int R, int Q, bool LAST>
+__global__ void __launch_bounds__(kSeg* kTaps* R)
+    cheb_pass_kernel(int side, int ncut, const float* __restrict__ in, const float* __restrict__ W, float* __restrict__ out,
+                     float d, ChebLimits l, const int* box_start)
+{
+    __shared__ float2 s_lim[kSeg + 2 * kChebMaxCut];  // of the window's boxes
+    __shared__ bool s_apart[kSeg];
     using C = ChebPass<P, R, Q>;
     extern __shared__ float4 cheb_smem[];
     const int taps = 2 * ncut + 1;
@@ -113,15 +165,20 @@ __global__ void __launch_bounds__(kSeg* kTaps* R)
     const int tid = threadIdx.x, line = blockIdx.y, t0 = blockIdx.x * kSeg;
     after_go();
     after_wait();
+    const int nwin = kSeg + 2 * ncut;
+    static_assert(C::THREADS >= kSeg + 2 * kChebMaxCut);
     for (int i = tid; i < taps * P * Q / 4; i += C::THREADS)
         reinterpret_cast<float4*>(s_tab)[i] = __ldg(reinterpret_cast<const float4*>(W) + i);
+    float2 lim = make_float2(-INFINITY, -INFINITY);
+    if (const int s = t0 - ncut + tid; tid < nwin && s >= 0 && s < side) lim = (LAST ? l.line : l.box)[line * side + s];
     constexpr int B4 = P * R / 4;
-    for (int i = tid; i < (kSeg + 2 * ncut) * B4; i += C::THREADS) {
+    for (int i = tid; i < nwin * B4; i += C::THREADS) {
         const int b = i / B4, s = t0 - ncut + b;
         float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
         if (s >= 0 && s < side) v = __ldg(reinterpret_cast<const float4*>(in + ((size_t)line * side + s) * P * R) + i % B4);
         *reinterpret_cast<float4*>(s_win + b * C::BOX + 4 * (i % B4)) = v;
     }
+    if (tid < nwin) s_lim[tid] = lim;
     __syncthreads();
     const int group = tid / (kSeg * R), e = tid % (kSeg * R), seg = e / R, r = e % R;
     float sum[Q];
@@ -148,6 +205,36 @@ __global__ void __launch_bounds__(kSeg* kTaps* R)
 #pragma unroll
         for (int m = 0; m < Q; ++m) sum[m] += acc[m];
     }
+    // the limits, after the sums (before them the first pass took 2 us more); the last warps have fewer taps
+    for (int t = C::THREADS / 32 - 1 - tid / 32; t < kSeg; t += C::THREADS / 32) {
+        const int lane = tid & 31;
+        int hi = float_key(-INFINITY), lo = hi;
+        for (int j = lane; j < taps; j += 32) {
+            const float2 m = s_lim[t + j];
+            const float k = (float)abs(j - ncut), near = fmaxf(k - 0.5f, 0.f) * d, far = (k + 0.5f) * d;
+            hi = max(hi, float_key(m.x - near * near));
+            lo = max(lo, float_key(m.y - far * far));
+        }
+        hi = __reduce_max_sync(0xffffffffu, hi);
+        lo = __reduce_max_sync(0xffffffffu, lo);
+        const int b = (t0 + t) * side + line;
+        if (lane || t0 + t >= side) continue;
+        const float2 m = make_float2(__int_as_float(hi ^ (hi >> 31 & 0x7FFFFFFF)), __int_as_float(lo ^ (lo >> 31 & 0x7FFFFFFF)));
+        if constexpr (!LAST) {
+            l.line[b] = m;
+        } else {
+            // m.x = -inf: no source box holds anything; inf - inf: a coefficient is not finite
+            const bool apart = m.x > -INFINITY && !(m.x - m.y <= kChebLoss);
+            l.apart[b] = s_apart[t] = apart;
+            const int n = apart ? box_start[b + 1] - box_start[b] : 0;
+            if (n > 0) {
+                const unsigned long long old =
+                    atomicAdd(l.list.count, (1ull << 32) | (unsigned)((n + kEvalThreads - 1) / kEvalThreads));
+                l.list.box[old >> 32] = b;
+                l.list.claim[old >> 32] = (int)old;
+            }
+        }
+    }
     __syncthreads();
 #pragma unroll
     for (int q = 0; q < Q / 4; ++q)
@@ -160,24 +247,19 @@ __global__ void __launch_bounds__(kSeg* kTaps* R)
         float v = 0.f;
 #pragma unroll
         for (int k = 0; k < kTaps; ++k) v += s_win[k * C::OUT + i];
+        if (LAST && i % (R * Q) == 0 && s_apart[i / (R * Q)]) v = NAN;
         out[((size_t)t * side + line) * (R * Q) + i % (R * Q)] = v;
     }
 }
 
-struct ChebEval {
-    int g, ncut, n, accumulate;
-    double d;
-    const float* A;
+struct ChebEval : H2pSums {
     const float* C;
-    const double* y;
-    const int* perm;
-    const int* box_start;
-    float* G;
-    int* err;
+    const unsigned char* apart;  // of ChebLimits
+    H2pList list;
 };
 
-// The direct sum for one target assigned to `box`, as the direct kernel takes it (a source box without
-// a non-zero coefficient adds nothing): source boxes first, first + step, ... of the neighbourhood.
+// The direct sum for one target assigned to `box`, as the direct kernel takes it (source boxes without
+// a non-zero coefficient are skipped): source boxes first, first + step, ... of the neighbourhood.
 template <int P>
 __device__ __noinline__ float cheb_direct(const ChebEval& a, int box, double y0, double y1, int first, int step)
 {
@@ -190,6 +272,7 @@ __device__ __noinline__ float cheb_direct(const ChebEval& a, int box, double y0,
 #pragma unroll 1
     for (int i = first; i < nb; i += step) {
         const int sx = sx0 + i % w, sy = sy0 + i / w;
+        if (!a.nz[sy * side + sx]) continue;
         if (sy != row) {
             row = sy;
             hermite_functions<P>(u2 + (float)((double)(ty - sy) * a.d), h2);
@@ -197,7 +280,6 @@ __device__ __noinline__ float cheb_direct(const ChebEval& a, int box, double y0,
         // Clenshaw's backward recurrence over a1 for h_(a+1) = 2t h_a - 2a h_(a-1)
         const float t1 = u1 + (float)((double)(tx - sx) * a.d), tt = t1 + t1;
         const float4* Ab = reinterpret_cast<const float4*>(a.A + ((size_t)sy * side + sx) * P * P);
-        bool nz = false;
         float c1 = 0.f, c2 = 0.f;
 #pragma unroll
         for (int a1 = P - 1; a1 >= 0; --a1) {
@@ -205,7 +287,6 @@ __device__ __noinline__ float cheb_direct(const ChebEval& a, int box, double y0,
 #pragma unroll
             for (int q = 0; q < P / 4; ++q) {
                 const float4 v = __ldg(Ab + a1 * (P / 4) + q);
-                nz |= v.x != 0.f || v.y != 0.f || v.z != 0.f || v.w != 0.f;
                 t = fmaf(v.x, h2[4 * q], t);
                 t = fmaf(v.y, h2[4 * q + 1], t);
                 t = fmaf(v.z, h2[4 * q + 2], t);
@@ -214,7 +295,7 @@ __device__ __noinline__ float cheb_direct(const ChebEval& a, int box, double y0,
             c2 = c1;
             c1 = t;
         }
-        if (nz) acc = fmaf(__expf(-t1 * t1), c1, acc);
+        acc = fmaf(__expf(-t1 * t1), c1, acc);
     }
     return acc;
 }
@@ -334,17 +415,11 @@ __device__ __forceinline__ void binned_targets(const double* __restrict__ y, con
 // 16-byte loads of its coefficients, each feeding 4 kRows multiply-adds a lane), else a row of
 // 32 at a time with a box per lane.
 constexpr int kRows = 4;
-constexpr int kEvalThreads = 128;
 
 template <int P, int Q>
-__global__ void __launch_bounds__(kEvalThreads) cheb_eval_kernel(ChebEval a)
+__device__ __forceinline__ void cheb_eval_warp(const ChebEval& a, int64_t base)
 {
     const int lane = threadIdx.x & 31, side = 1 << a.g, nbox = side * side;
-    after_go();
-    after_wait();
-    const int64_t base = ((int64_t)blockIdx.x * (kEvalThreads / 32) + (threadIdx.x >> 5)) * (32 * kRows);
-    bin_check(a.box_start, nbox, a.n, a.err);
-    if (base >= a.n) return;
     int tj[kRows], tb[kRows];  // target, its box (-1: evaluated apart)
     float x1[kRows], x2[kRows], out[kRows];
     binned_targets<kRows>(a.y, a.perm, a.box_start, a.g, a.n, base + lane, a.err, tj, tb, x1, x2);
@@ -380,7 +455,9 @@ __global__ void __launch_bounds__(kEvalThreads) cheb_eval_kernel(ChebEval a)
                 double y0 = 0.0, y1 = 0.0;
                 if (b < 0 && j >= 0) {
                     lo = bin_find(a.box_start, nbox, (int)(base + 32 * r + lane), a.n);
-                    if (lo >= 0) {
+                    if (lo >= 0 && a.apart[lo]) {
+                        lo = j = -1;
+                    } else if (lo >= 0) {
                         y0 = __ldg(a.y + 2 * (size_t)j);
                         y1 = __ldg(a.y + 2 * (size_t)j + 1);
                     } else {  // box_start does not bin [0, n)
@@ -401,10 +478,41 @@ __global__ void __launch_bounds__(kEvalThreads) cheb_eval_kernel(ChebEval a)
     }
 #pragma unroll
     for (int r = 0; r < kRows; ++r)
-        if (tj[r] >= 0) a.G[tj[r]] = a.accumulate ? a.G[tj[r]] + out[r] : out[r];
+        // NaN of a box that is summed directly: left to that sum
+        if (tj[r] >= 0 && !(isnan(out[r]) && tb[r] >= 0 && a.apart[tb[r]])) a.G[tj[r]] = a.accumulate ? a.G[tj[r]] + out[r] : out[r];
 }
 
-// Per device and grid size: table | X [4^g][16][12] | C [4^g][12][12], allocated on first use and
+// A CTA that has evaluated its own targets takes its share of the claims on the listed boxes, 128
+// targets each, one a thread.  (A launch of the direct kernel after this one cost 7 us more for an empty list,
+// and so did CTAs of their own before the others.)
+template <int P, int Q>
+__global__ void __launch_bounds__(kEvalThreads) cheb_eval_kernel(ChebEval a)
+{
+    __shared__ H2pShared<kEvalThreads> sh;
+    __shared__ int s_claim[3];
+    extern __shared__ float4 cheb_smem[];
+    const int nbox = 1 << (2 * a.g);
+    after_go();
+    after_wait();
+    const int64_t base = ((int64_t)blockIdx.x * (kEvalThreads / 32) + (threadIdx.x >> 5)) * (32 * kRows);
+    bin_check(a.box_start, nbox, a.n, a.err);
+    const unsigned long long count = *a.list.count;
+    if (base < a.n) cheb_eval_warp<P, Q>(a, base);
+    if (blockIdx.x >= (unsigned)count) return;
+    h2p_offsets(sh, a);
+    for (unsigned k = blockIdx.x; k < (unsigned)count; k += gridDim.x) {
+        if (threadIdx.x == 0)
+            h2p_claim_range_ordered(a.list.claim, a.list.box, a.box_start, nbox, (int)(count >> 32), a.n, kEvalThreads, k,
+                                    s_claim, s_claim + 1, s_claim + 2);
+        __syncthreads();
+        const int first = s_claim[0], end = s_claim[1], box = s_claim[2];
+        if (first < end) h2p_run<P, 1, kEvalThreads>(a, sh, reinterpret_cast<float*>(cheb_smem), first, end, box);
+        __syncthreads();  // the claim has been read
+    }
+}
+
+// Per device and grid size: table | X [4^g][16][12] | C [4^g][12][12] | the list's count | l.box, l.line
+// [4^g] | the list's boxes and claims [4^g] | nz, apart [4^g] (bytes), allocated on first use and
 // kept (captured graphs hold its address).  NULL, without an error, when it would have to be
 // allocated inside a stream capture.
 static int cheb_workspace(int g, cudaStream_t st, float** out)
@@ -420,7 +528,7 @@ static int cheb_workspace(int g, cudaStream_t st, float** out)
         cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
         FMM_CUDA_TRY(cudaStreamIsCapturing(st, &cs));
         if (cs != cudaStreamCaptureStatusNone) return FMM_OK;
-        const size_t bytes = (kChebTableFloats + ((size_t)(16 + kChebQ) * kChebQ << (2 * g))) * sizeof(float);
+        const size_t bytes = (kChebTableFloats + 2 + ((size_t)((16 + kChebQ) * kChebQ + 7) << (2 * g))) * sizeof(float);
         if (cudaMalloc(&buf[dev][g], bytes) != cudaSuccess) {
             (void)cudaGetLastError();
             buf[dev][g] = nullptr;
@@ -432,23 +540,42 @@ static int cheb_workspace(int g, cudaStream_t st, float** out)
 }
 
 template <int P, int Q = kChebQ>
-static int cheb_launch(const ChebEval& e, float* ws, cudaStream_t st)
+static int cheb_launch(const H2pSums& e, float* ws, cudaStream_t st)
 {
     using C1 = ChebPass<P, P, Q>;
     using C2 = ChebPass<P, Q, Q>;
     const int side = 1 << e.g;
     float *W = ws, *X = W + kChebTableFloats, *C = X + ((size_t)16 * kChebQ << (2 * e.g));
     static unsigned long long opted[2];
-    if (int rc = smem_opt_in((const void*)cheb_pass_kernel<P, P, Q>, (int)C1::smem(kChebMaxCut), &opted[0])) return rc;
-    if (int rc = smem_opt_in((const void*)cheb_pass_kernel<P, Q, Q>, (int)C2::smem(kChebMaxCut), &opted[1])) return rc;
-    FMM_CUDA_TRY(launch_after(cheb_table_kernel<P, Q>, 2 * e.ncut + 1, 256, 0, st, e.ncut, e.d, W));
+    if (int rc = smem_opt_in((const void*)cheb_pass_kernel<P, P, Q, false>, (int)C1::smem(kChebMaxCut), &opted[0])) return rc;
+    if (int rc = smem_opt_in((const void*)cheb_pass_kernel<P, Q, Q, true>, (int)C2::smem(kChebMaxCut), &opted[1])) return rc;
+    const size_t nbox = (size_t)1 << (2 * e.g);
+    ChebLimits l;
+    l.list.count = reinterpret_cast<unsigned long long*>(C + kChebQ * kChebQ * nbox);
+    l.box = reinterpret_cast<float2*>(l.list.count + 1);
+    l.line = l.box + nbox;
+    l.list.box = reinterpret_cast<int*>(l.line + nbox);
+    l.list.claim = l.list.box + nbox;
+    l.nz = reinterpret_cast<unsigned char*>(l.list.claim + nbox);
+    l.apart = l.nz + nbox;
+    FMM_CUDA_TRY(launch_after(cheb_table_kernel<P, Q>, 2 * e.ncut + 1 + (unsigned)(nbox + 7) / 8, 256, 0, st, e.ncut, e.d, (int)nbox, e.A, W, l));
     const dim3 grid((side + kSeg - 1) / kSeg, side);
-    FMM_CUDA_TRY(launch_after(cheb_pass_kernel<P, P, Q>, grid, C1::THREADS, C1::smem(e.ncut), st, side, e.ncut, e.A, W, X));
-    FMM_CUDA_TRY(launch_after(cheb_pass_kernel<P, Q, Q>, grid, C2::THREADS, C2::smem(e.ncut), st, side, e.ncut, X, W, C));
-    ChebEval a = e;
+    FMM_CUDA_TRY(launch_after(cheb_pass_kernel<P, P, Q, false>, grid, C1::THREADS, C1::smem(e.ncut), st, side, e.ncut, e.A, W, X,
+                              (float)e.d, l, e.box_start));
+    FMM_CUDA_TRY(launch_after(cheb_pass_kernel<P, Q, Q, true>, grid, C2::THREADS, C2::smem(e.ncut), st, side, e.ncut, X, W, C,
+                              (float)e.d, l, e.box_start));
+    ChebEval a;
+    static_cast<H2pSums&>(a) = e;
+    a.nz = l.nz;
     a.C = C;
-    const unsigned blocks = bin_blocks(a.n, kEvalThreads * kRows, (int64_t)1 << (2 * e.g), kEvalThreads);
-    FMM_CUDA_TRY(launch_after(cheb_eval_kernel<P, Q>, blocks, kEvalThreads, 0, st, a));
+    a.apart = l.apart;
+    a.list = l.list;
+    int sms = 0;
+    if (int rc = device_sm_count(&sms)) return rc;
+    // with few targets, CTAs enough for the listed boxes (a list of 800 boxes of 16 targets: 150 -> 70 us)
+    const unsigned blocks = std::max(bin_blocks(a.n, kEvalThreads * kRows, (int64_t)nbox, kEvalThreads),
+                                     (unsigned)std::min<size_t>(nbox, 2 * (size_t)sms));
+    FMM_CUDA_TRY(launch_after(cheb_eval_kernel<P, Q>, blocks, kEvalThreads, H2pSmem<P>::bytes, st, a));
     return FMM_OK;
 }
 
@@ -461,7 +588,7 @@ int launch_fgt_h2p_cheb(int g, int ncut, int p, double d, const float* A, const 
     if (int rc = cheb_workspace(g, st, &ws)) return rc;
     if (!ws) return FMM_OK;
     *done = true;
-    const ChebEval e{g, ncut, n, accumulate ? 1 : 0, d, A, nullptr, y, perm, box_start, G, err};
+    const H2pSums e{g, ncut, n, d, A, y, perm, box_start, nullptr, G, accumulate ? 1 : 0, err};
     switch (p) {
         case 4: return cheb_launch<4>(e, ws, st);
         case 8: return cheb_launch<8>(e, ws, st);

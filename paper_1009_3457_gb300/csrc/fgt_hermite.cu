@@ -433,39 +433,21 @@ __global__ void __launch_bounds__(kP2hPoints) fgt_p2h_binned_kernel(int g, doubl
 // ---------------------------------------------------------------------------
 // Hermite evaluation at binned targets
 // ---------------------------------------------------------------------------
-constexpr int kH2pThreads = 128;
-constexpr int kH2pWarps = kH2pThreads / 32;
-constexpr int kH2pMaxCut = 16;
-constexpr int kH2pMaxBoxes = (2 * kH2pMaxCut + 1) * (2 * kH2pMaxCut + 1);
-constexpr int kH2pBatch = 8;                  // source boxes per shared-memory stage
-constexpr int kH2pStages = 3;                 // ring depth (two batches in flight)
-
 template <int P>
 struct H2pCfg {
     // 4 targets per thread: each broadcast 16-byte load of A feeds 16 FMAs; 64-thread CTAs at
     // p >= 12 keep a claim at 256 targets (a box's last claim is partly idle)
     static constexpr int R = 4;                        // targets per thread
     static constexpr int THREADS = P >= 12 ? 64 : 128;
-    static constexpr int WARPS = THREADS / 32;
     static constexpr int CH = THREADS * R;             // targets per claim
     static constexpr int PP = P * P;
-    static constexpr size_t smem = (size_t)kH2pStages * kH2pBatch * PP * sizeof(float);
+    static constexpr size_t smem = H2pSmem<P>::bytes;
 };
 
-struct H2pArgs {
-    int g, ncut, n;
-    double d;  // box side / (sqrt2 sigma)
-    const float* A;
-    const double* y;
-    const int* perm;
-    const int* box_start;
-    const unsigned char* nz;  // per source box: any non-zero coefficient
+struct H2pArgs : H2pSums {
     const int* claims;        // [nbox + 1] claim-index prefix over the boxes in `order`
     const int* order;         // [nbox] the boxes, heaviest neighbourhood first (h2p_order_*)
-    float* G;
-    int accumulate;
     int* cursor;  // [0] next claim index, [1] CTAs finished
-    int* err;
 };
 
 // flag[b] = any coefficient of box b is non-zero (one warp per box)
@@ -478,16 +460,6 @@ __global__ void fgt_box_flags_kernel(const float* __restrict__ A, int nbox, int 
     nz = __any_sync(0xffffffffu, nz);
     if (lane == 0) flag[b] = nz ? 1 : 0;
 }
-
-__device__ __forceinline__ void cp_async_16(void* smem, const void* gmem)
-{
-    const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
-
 
 // claims[0..nbox]: exclusive scan of ceil(targets of box b / ch), the table that maps a claim
 // index to its box; a box_start that decreases counts as empty and is reported.
@@ -657,7 +629,7 @@ __device__ bool h2p_claim(const H2pArgs& a, int nbox, int ch, int* first, int* e
     const int total = __ldg(a.claims + nbox);
     const int k = atomicAdd(a.cursor, 1);
     if (k >= total) return false;
-    h2p_claim_range_ordered(a.claims, a.order, a.box_start, nbox, a.n, ch, k, first, end, box);
+    h2p_claim_range_ordered(a.claims, a.order, a.box_start, nbox, nbox, a.n, ch, k, first, end, box);
     if (*first >= *end) atomicOr(a.err, DEV_ERR_CHECK);  // box_start does not bin [0, n)
     return true;
 }
@@ -666,20 +638,11 @@ template <int P>
 __global__ void __launch_bounds__(H2pCfg<P>::THREADS) fgt_h2p_kernel(H2pArgs a)
 {
     using C = H2pCfg<P>;
-    constexpr int R = C::R;
-    constexpr int PP = C::PP;
-    constexpr int NT = C::THREADS;
     extern __shared__ float4 h2p_smem[];
-    float* sA = reinterpret_cast<float*>(h2p_smem);  // [kH2pStages][kH2pBatch][P][P]
-    __shared__ float s_off[2 * kH2pMaxCut + 1];       // k d, k = -ncut .. ncut
-    __shared__ short s_list[kH2pMaxBoxes];            // non-empty source boxes, row-major, as (dy + ncut) * 64 + dx + ncut
-    __shared__ int s_warp_cnt[C::WARPS];
+    __shared__ H2pShared<C::THREADS> sh;
     __shared__ int s_claim[4];
-
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int side = 1 << a.g, nbox = side * side;
-    const int wmax = 2 * a.ncut + 1;
-    if (tid < wmax) s_off[tid] = (float)((double)(tid - a.ncut) * a.d);
+    const int tid = threadIdx.x, side = 1 << a.g, nbox = side * side;
+    h2p_offsets(sh, a);
 
     for (;;) {
         if (tid == 0) {
@@ -696,133 +659,7 @@ __global__ void __launch_bounds__(H2pCfg<P>::THREADS) fgt_h2p_kernel(H2pArgs a)
             __syncthreads();
             continue;
         }
-        const int tx = box & (side - 1), ty = box >> a.g;
-        const int x0 = max(tx - a.ncut, 0), x1 = min(tx + a.ncut, side - 1);
-        const int y0 = max(ty - a.ncut, 0), y1 = min(ty + a.ncut, side - 1);
-        const int w = x1 - x0 + 1, nb = w * (y1 - y0 + 1);
-
-        // ordered compaction of the neighbourhood's non-empty source boxes (row-major)
-        int total = 0;
-        for (int base = 0; base < nb; base += NT) {
-            const int i = base + tid;
-            bool keep = false;
-            int code = 0;
-            if (i < nb) {
-                const int sx = x0 + i % w, sy = y0 + i / w;
-                keep = __ldg(a.nz + sy * side + sx) != 0;
-                code = (sy - ty + a.ncut) * 64 + (sx - tx + a.ncut);
-            }
-            const unsigned bal = __ballot_sync(0xffffffffu, keep);
-            if (lane == 0) s_warp_cnt[warp] = __popc(bal);
-            __syncthreads();
-            int off = total;
-            for (int q = 0; q < warp; ++q) off += s_warp_cnt[q];
-            if (keep) s_list[off + __popc(bal & ((1u << lane) - 1))] = (short)code;
-            for (int q = 0; q < C::WARPS; ++q) total += s_warp_cnt[q];
-            __syncthreads();
-        }
-
-        // this thread's targets and their offsets u within the box
-        int tj[R];
-        float u1[R], u2[R], acc[R];
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int pos = first + warp * 32 * R + r * 32 + lane;  // a warp's 32 R targets
-            tj[r] = -1;
-            u1[r] = u2[r] = acc[r] = 0.f;
-            if (pos < end) {
-                const int j = __ldg(a.perm + pos);
-                if ((unsigned)j < (unsigned)a.n) {
-                    tj[r] = j;
-                    u1[r] = (float)((__ldg(a.y + 2 * (size_t)j) * side - (tx + 0.5)) * a.d);
-                    u2[r] = (float)((__ldg(a.y + 2 * (size_t)j + 1) * side - (ty + 0.5)) * a.d);
-                } else {
-                    atomicOr(a.err, DEV_ERR_CHECK);
-                }
-            }
-        }
-        const bool active = first + warp * 32 * R < end;  // warp-uniform
-
-        const int nbatch = (total + kH2pBatch - 1) / kH2pBatch;
-        auto stage = [&](int k) {
-            if (k < nbatch) {
-                float4* dst = reinterpret_cast<float4*>(sA + (size_t)(k % kH2pStages) * kH2pBatch * PP);
-                const int cnt = min(kH2pBatch, total - k * kH2pBatch) * (PP / 4);
-                for (int i = tid; i < cnt; i += NT) {
-                    const int code = s_list[k * kH2pBatch + i / (PP / 4)];
-                    const int sx = tx + (code & 63) - a.ncut, sy = ty + (code >> 6) - a.ncut;
-                    cp_async_16(dst + i, reinterpret_cast<const float4*>(a.A + ((size_t)sy * side + sx) * PP) +
-                                             i % (PP / 4));
-                }
-            }
-            cp_async_commit();  // an empty group past the end keeps the wait counts uniform
-        };
-        stage(0);
-        stage(1);
-        int cur_dy = -1;
-        float h2[R][P];
-        for (int k = 0; k < nbatch; ++k) {
-            cp_async_wait<1>();
-            __syncthreads();  // batch k landed; everyone is done with batch k - 1's stage
-            stage(k + 2);
-            if (active) {
-                const float* sb = sA + (size_t)(k % kH2pStages) * kH2pBatch * PP;
-                const int nk = min(kH2pBatch, total - k * kH2pBatch);
-#pragma unroll 1
-                for (int e = 0; e < nk; ++e) {
-                    const int code = s_list[k * kH2pBatch + e];
-                    const int dy = code >> 6, dx = code & 63;  // source offset + ncut
-                    if (dy != cur_dy) {
-                        cur_dy = dy;
-#pragma unroll
-                        for (int r = 0; r < R; ++r) hermite_functions<P>(u2[r] + s_off[2 * a.ncut - dy], h2[r]);
-                    }
-                    // sum_a1 h_a1(t1) T[a1], T[a1] = sum_a2 A[a1][a2] h_a2(t2), by Clenshaw's backward
-                    // recurrence for h_{a+1} = 2t h_a - 2a h_{a-1}:
-                    //   c_a = T[a] + 2t c_{a+1} - 2(a+1) c_{a+2},  c_p = c_{p+1} = 0,  sum = h_0(t1) c_0,
-                    // two multiply-adds per a1 beside the p of T[a1] (the forward recurrence and the
-                    // accumulation take three)
-                    float c1[R], c2[R], tt[R], e0[R];
-#pragma unroll
-                    for (int r = 0; r < R; ++r) {
-                        const float t = u1[r] + s_off[2 * a.ncut - dx];
-                        tt[r] = t + t;
-                        e0[r] = __expf(-t * t);
-                        c1[r] = c2[r] = 0.f;
-                    }
-                    const float4* Ab = reinterpret_cast<const float4*>(sb + e * PP);
-#pragma unroll
-                    for (int a1 = P - 1; a1 >= 0; --a1) {
-                        float t[R];
-#pragma unroll
-                        for (int r = 0; r < R; ++r) t[r] = fmaf(tt[r], c1[r], -(float)(2 * (a1 + 1)) * c2[r]);
-#pragma unroll
-                        for (int qd = 0; qd < P / 4; ++qd) {
-                            const float4 v = Ab[a1 * (P / 4) + qd];
-#pragma unroll
-                            for (int r = 0; r < R; ++r) {
-                                t[r] = fmaf(v.x, h2[r][4 * qd], t[r]);
-                                t[r] = fmaf(v.y, h2[r][4 * qd + 1], t[r]);
-                                t[r] = fmaf(v.z, h2[r][4 * qd + 2], t[r]);
-                                t[r] = fmaf(v.w, h2[r][4 * qd + 3], t[r]);
-                            }
-                        }
-#pragma unroll
-                        for (int r = 0; r < R; ++r) {
-                            c2[r] = c1[r];
-                            c1[r] = t[r];
-                        }
-                    }
-#pragma unroll
-                    for (int r = 0; r < R; ++r) acc[r] = fmaf(e0[r], c1[r], acc[r]);
-                }
-            }
-        }
-        cp_async_wait<0>();
-        __syncthreads();  // the ring and the list are free for the next claim
-#pragma unroll
-        for (int r = 0; r < R; ++r)
-            if (tj[r] >= 0) a.G[tj[r]] = a.accumulate ? a.G[tj[r]] + acc[r] : acc[r];
+        h2p_run<P, C::R, C::THREADS>(a, sh, reinterpret_cast<float*>(h2p_smem), first, end, box);
     }
     // the last CTA to finish returns the cursor slot to zero for its next use
     if (tid == 0) {

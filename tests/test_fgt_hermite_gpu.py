@@ -460,7 +460,8 @@ def _per_target_terms(g, sigma, A, box, y):
     return np.einsum("ab,an,bn->n", np.abs(A.astype(np.float64)), h[:, :, 0], h[:, :, 1]), (t * t).sum(1)
 
 
-@pytest.mark.parametrize("p,d,g", [(16, 0.6, 3), (16, 1.0, 3), (16, 1.28, 3), (8, 0.95, 3), (12, 0.8, 3), (4, 1.9, 2)])
+@pytest.mark.parametrize("p,d,g", [(16, 0.6, 3), (16, 1.0, 3), (16, 1.28, 3), (8, 0.95, 3), (12, 0.8, 3), (4, 1.9, 2),
+                                   (16, 0.5, 4), (12, 0.5, 4), (8, 0.44, 4), (4, 0.5, 4), (16, 0.36, 5)])
 def test_h2p_each_target_keeps_its_own_accuracy(fmm, orc, p, d, g):
     """Sources in one corner box alone, targets all over the grid, down to values of 1e-30: each
     target's error against the size of its own terms, not of the largest target's.  FP32: t1^2 + t2^2
