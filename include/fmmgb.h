@@ -638,7 +638,8 @@ int fgt_h2p(int32_t grid_log2, int32_t n_cut, int32_t p, int32_t prec, double si
  *   1e-30 is added to every squared distance, so a source at exactly a
  *   target's position (e.g. the points themselves) contributes nothing
  *   (strengths |c| < 3e8) and other pairs change by a relative 1e-30 / r^2.  Uses a
- *   per-device buffer grown on demand (calls that overlap on the GPU must be serialised).  A
+ *   per-device buffer grown on demand (calls that overlap on the GPU must be serialised; graphs
+ *   captured with a smaller one keep it).  A
  *   permutation entry outside range or inconsistent box starts set the device
  *   error word's check bit; the affected pairs are skipped.
  * ------------------------------------------------------------------------- */

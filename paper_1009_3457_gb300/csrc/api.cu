@@ -151,6 +151,39 @@ int tile_counter(int** out, cudaStream_t st)
     return FMM_OK;
 }
 
+cudaError_t capture_safe_malloc(void** out, size_t bytes)
+{
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaError_t e = cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e != cudaSuccess) return e;
+    e = cudaMalloc(out, bytes);
+    if (e != cudaSuccess) {
+        (void)cudaGetLastError();
+        *out = nullptr;
+    }
+    const cudaError_t back = cudaThreadExchangeStreamCaptureMode(&mode);
+    return e != cudaSuccess ? e : back;
+}
+
+int kept_buffer(KeptBuffer& b, size_t bytes, void** out)
+{
+    int dev = 0;
+    FMM_CUDA_TRY(cudaGetDevice(&dev));
+    if (dev < 0 || dev >= 64) return fail(FMM_EUNSUPPORTED, "device ordinal %d above 63", dev);
+    std::lock_guard<std::mutex> lk(b.mu);
+    if (b.bytes[dev] < bytes) {
+        void* p = nullptr;
+        size_t want = bytes < 2 * b.bytes[dev] ? 2 * b.bytes[dev] : bytes;
+        cudaError_t e = capture_safe_malloc(&p, want);
+        if (e == cudaErrorMemoryAllocation && want > bytes) e = capture_safe_malloc(&p, want = bytes);
+        if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(scratch)");
+        b.ptr[dev] = p;
+        b.bytes[dev] = want;
+    }
+    *out = b.ptr[dev];
+    return FMM_OK;
+}
+
 int fgt_flag_buffer(unsigned char** out)
 {
     std::lock_guard<std::mutex> lk(g_mu);

@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <mutex>
+
 #include "fmmgb.h"
 
 namespace fmmgb {
@@ -117,6 +119,18 @@ inline cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, siz
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
+
+// Per-device scratch grown on demand, to twice its size at least where that fits.  Nothing is freed:
+// captured graphs hold the address that they were recorded with, and the buffers outgrown add up to less
+// than the present one.  May be called while a stream is being captured (nothing is enqueued).
+struct KeptBuffer {
+    std::mutex mu;
+    void* ptr[64] = {};
+    size_t bytes[64] = {};
+};
+int kept_buffer(KeptBuffer& b, size_t bytes, void** out);
+// cudaMalloc, while a stream is being captured too.
+cudaError_t capture_safe_malloc(void** out, size_t bytes);
 
 // Number of SMs of the current device (cached).
 int device_sm_count(int* out);

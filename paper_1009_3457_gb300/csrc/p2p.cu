@@ -554,30 +554,8 @@ __global__ void __launch_bounds__(kP2pThreads, kP2wCtas) fmm_p2p_warp_kernel(P2p
     }
 }
 
-// Per-device buffer of sorted sources (grown on demand).
-static std::mutex g_src_mu;
-static float4* g_src[64];
-static size_t g_src_bytes[64];
-
-static int p2p_source_buffer(size_t bytes, float4** out)
-{
-    int dev = 0;
-    FMM_CUDA_TRY(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= 64) return fail(FMM_EUNSUPPORTED, "fmm_p2p: device ordinal %d above 63", dev);
-    std::lock_guard<std::mutex> lk(g_src_mu);
-    if (g_src_bytes[dev] < bytes) {
-        if (g_src[dev]) {
-            FMM_CUDA_TRY(cudaDeviceSynchronize());
-            cudaFree(g_src[dev]);
-            g_src[dev] = nullptr;
-            g_src_bytes[dev] = 0;
-        }
-        FMM_CUDA_TRY(cudaMalloc(&g_src[dev], bytes));
-        g_src_bytes[dev] = bytes;
-    }
-    *out = g_src[dev];
-    return FMM_OK;
-}
+// The sources in box order and the claim table of a call.
+static KeptBuffer g_p2p_buffer;
 
 }  // namespace fmmgb
 
@@ -624,7 +602,7 @@ extern "C" int fmm_p2p(int32_t level, const double* xy, const double* c, int64_t
     // one buffer: the sources in box order, the claim table, the number of claims
     const int64_t most = nz / run + std::min<int64_t>(nbox, nz);  // claims can be no more
     float4* src = nullptr;
-    if (int rc = p2p_source_buffer((size_t)(n + most + 1) * sizeof(float4), &src)) return rc;
+    if (int rc = kept_buffer(g_p2p_buffer, (size_t)(n + most + 1) * sizeof(float4), (void**)&src)) return rc;
     int4* tab = reinterpret_cast<int4*>(src + n);
     int* nclaim = reinterpret_cast<int*>(tab + most);
     args.nclaim = nclaim;

@@ -305,3 +305,39 @@ def test_binning_at_the_edges_of_its_blocks(fmm, level, n):
     assert torch.equal(torch.diff(start).long(), torch.bincount(box, minlength=4 ** level))
     assert torch.equal(box[perm.long()], torch.sort(box).values)
     assert torch.equal(torch.sort(perm).values.long(), torch.arange(n, device="cuda"))
+
+
+def test_p2p_graph_keeps_its_buffer(fmm):
+    """The per-device buffer grows inside a capture (more targets, then more sources, than any call
+    before), and a graph captured before it grew replays what it did."""
+    import torch
+
+    level = 7
+    g = torch.Generator(device="cuda").manual_seed(3)
+
+    def problem(n, nz):
+        xy, z = (torch.rand((k, 2), dtype=torch.float64, device="cuda", generator=g) for k in (n, nz))
+        c = torch.rand(n, dtype=torch.float64, device="cuda", generator=g) - 0.5
+        phi = torch.empty(nz, dtype=torch.complex64, device="cuda")
+        (sp, ss), (tp, ts) = _bins(fmm, level, xy), _bins(fmm, level, z)
+        return phi, lambda: fmm.fmm_p2p(level, xy, c, sp, ss, z, tp, ts, phi)
+
+    torch.cuda.synchronize()
+    grow = 6_000_000  # beyond every other call of these tests
+    problems = [problem(1000, 2000), problem(1000, grow), problem(2 * grow, 2000), problem(8 * grow, 3000)]
+    problems[0][1]()
+    torch.cuda.synchronize()
+    graphs = []
+    for phi, call in problems:
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, capture_error_mode="thread_local"):
+            call()
+        graphs.append(graph)
+    for graph, (phi, call) in zip(graphs, problems):
+        call()
+        fmm.fmm_sync_status()
+        want = phi.clone()
+        phi.fill_(float("nan"))
+        graph.replay()
+        fmm.fmm_sync_status()
+        assert torch.equal(torch.view_as_real(phi), torch.view_as_real(want))
