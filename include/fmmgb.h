@@ -580,8 +580,8 @@ int fgt_t2p_binned(int32_t grid_log2, int32_t p, double sigma, const float* C, c
  *   source boxes are taken once per target box.  Targets outside the unit square, and
  *   boxes over which the field falls by more than e^5 (sources far away only), are summed
  *   directly in the same call, so that each value keeps its own FP32 accuracy.  The workspace, 1.4 KiB per box, is allocated
- *   per grid size and device on the first such call and kept; a first such call inside a
- *   stream capture takes the direct sums below instead, as every other call does.  Calls that
+ *   per grid size and device on the first such call, in a stream capture or not, and kept
+ *   (where there is no room for it the call takes the direct sums below, as every other call does).  Calls that
  *   overlap on the GPU share the workspace and must be serialised by the caller.
  *   prec FMM_FP32: CUDA cores.  Source boxes whose coefficients are all zero
  *   are skipped: a first kernel writes one flag per box.  The targets are
@@ -589,7 +589,8 @@ int fgt_t2p_binned(int32_t grid_log2, int32_t p, double sigma, const float* C, c
  *   source boxes within n_cut first (an order built on the device in every
  *   call; G does not depend on it).  Flags, claim order and claim table live
  *   in a ~17 MiB per-device scratch that the library allocates on the first
- *   call (or in fmm_prepare; make one of them before any stream capture);
+ *   call that needs it, in a stream capture or not (a first fgt_h2p call of any kind, or fmm_prepare,
+ *   must come before any capture);
  *   calls that overlap on the GPU (different streams) share it and must be
  *   serialised by the caller.  A perm
  *   entry outside [0, n) or a box_start that does not bin [0, n) sets the
@@ -602,8 +603,7 @@ int fgt_t2p_binned(int32_t grid_log2, int32_t p, double sigma, const float* C, c
  *   FP32 accumulation, BF16 operands split into hi + lo (three products,
  *   ~16 significant bits each) or hi only.  Every box of the neighbourhood
  *   is evaluated (no skipping).  A BF16 copy of A (1 KiB per box) lives in a
- *   per-device buffer grown on demand (the first call of a grid size
- *   allocates: make it before any stream capture).
+ *   per-device buffer grown on demand, in a stream capture or not.
  * ------------------------------------------------------------------------- */
 int fgt_bin_points(int32_t grid_log2, const double* y, int64_t n, int32_t* perm, int32_t* box_start, int32_t* work,
                    void* stream);

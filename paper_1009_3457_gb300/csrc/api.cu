@@ -190,7 +190,7 @@ int fgt_flag_buffer(unsigned char** out)
     DeviceState* s = nullptr;
     int rc = current_state(&s);
     if (rc) return rc;
-    if (!s->fgt_flags) FMM_CUDA_TRY(cudaMalloc(&s->fgt_flags, kFgtScratchBytes));
+    if (!s->fgt_flags) FMM_CUDA_TRY(capture_safe_malloc((void**)&s->fgt_flags, kFgtScratchBytes));
     *out = s->fgt_flags;
     return FMM_OK;
 }

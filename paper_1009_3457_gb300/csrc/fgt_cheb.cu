@@ -513,9 +513,8 @@ __global__ void __launch_bounds__(kEvalThreads) cheb_eval_kernel(ChebEval a)
 
 // Per device and grid size: table | X [4^g][16][12] | C [4^g][12][12] | the list's count | l.box, l.line
 // [4^g] | the list's boxes and claims [4^g] | nz, apart [4^g] (bytes), allocated on first use and
-// kept (captured graphs hold its address).  NULL, without an error, when it would have to be
-// allocated inside a stream capture.
-static int cheb_workspace(int g, cudaStream_t st, float** out)
+// kept (captured graphs hold its address).  NULL, without an error, when there is no room for it.
+static int cheb_workspace(int g, float** out)
 {
     static std::mutex mu;
     static float* buf[64][kChebMaxLog2 + 1];
@@ -525,15 +524,8 @@ static int cheb_workspace(int g, cudaStream_t st, float** out)
     if (dev < 0 || dev >= 64) return FMM_OK;  // the direct sum serves it
     std::lock_guard<std::mutex> lk(mu);
     if (!buf[dev][g]) {
-        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-        FMM_CUDA_TRY(cudaStreamIsCapturing(st, &cs));
-        if (cs != cudaStreamCaptureStatusNone) return FMM_OK;
         const size_t bytes = (kChebTableFloats + 2 + ((size_t)((16 + kChebQ) * kChebQ + 7) << (2 * g))) * sizeof(float);
-        if (cudaMalloc(&buf[dev][g], bytes) != cudaSuccess) {
-            (void)cudaGetLastError();
-            buf[dev][g] = nullptr;
-            return FMM_OK;
-        }
+        if (capture_safe_malloc((void**)&buf[dev][g], bytes) != cudaSuccess) return FMM_OK;
     }
     *out = buf[dev][g];
     return FMM_OK;
@@ -585,7 +577,7 @@ int launch_fgt_h2p_cheb(int g, int ncut, int p, double d, const float* A, const 
     *done = false;
     if (d > kChebMaxSide || g > kChebMaxLog2 || n < (2 << (2 * g))) return FMM_OK;
     float* ws = nullptr;
-    if (int rc = cheb_workspace(g, st, &ws)) return rc;
+    if (int rc = cheb_workspace(g, &ws)) return rc;
     if (!ws) return FMM_OK;
     *done = true;
     const H2pSums e{g, ncut, n, d, A, y, perm, box_start, nullptr, G, accumulate ? 1 : 0, err};

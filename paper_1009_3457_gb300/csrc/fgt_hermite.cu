@@ -900,13 +900,13 @@ extern "C" int fgt_h2p(int32_t grid_log2, int32_t n_cut, int32_t p, int32_t prec
     args.accumulate = (flags & FMM_ACCUMULATE) ? 1 : 0;
     cudaStream_t st = (cudaStream_t)stream;
     if (int rc = device_error_word(&args.err)) return rc;
+    if (int rc = tile_counter(&args.cursor, st)) return rc;  // whichever form serves a first call, a captured one may take the other
     // every precision: the Chebyshev form is FP32 throughout and faster than either direct form
     bool done = false;
     if (int rc = launch_fgt_h2p_cheb(grid_log2, n_cut, p, args.d, A, y, args.n, perm, box_start, G,
                                      args.accumulate != 0, args.err, st, &done))
         return rc;
     if (done) return FMM_OK;
-    if (int rc = tile_counter(&args.cursor, st)) return rc;
     unsigned char* nzbuf = nullptr;
     if (int rc = fgt_flag_buffer(&nzbuf)) return rc;
     args.nz = nzbuf;

@@ -396,54 +396,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) fgt_h2p_tc_kernel(H2pTcArgs a)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
 }
 
-// Per-device BF16 image of A (grown on demand).
-static std::mutex g_img_mu;
-static unsigned char* g_img[64];
-static size_t g_img_bytes[64];
-
-static int tc_image_buffer(size_t bytes, unsigned char** out)
-{
-    int dev = 0;
-    FMM_CUDA_TRY(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= 64) return fail(FMM_EUNSUPPORTED, "fgt_h2p: device ordinal %d above 63", dev);
-    std::lock_guard<std::mutex> lk(g_img_mu);
-    if (g_img_bytes[dev] < bytes) {
-        if (g_img[dev]) {
-            FMM_CUDA_TRY(cudaDeviceSynchronize());
-            cudaFree(g_img[dev]);
-            g_img[dev] = nullptr;
-            g_img_bytes[dev] = 0;
-        }
-        FMM_CUDA_TRY(cudaMalloc(&g_img[dev], bytes));
-        g_img_bytes[dev] = bytes;
-    }
-    *out = g_img[dev];
-    return FMM_OK;
-}
-
-// Per-device tile table (grown on demand).
-static unsigned char* g_tiles[64];
-static size_t g_tiles_bytes[64];
-
-static int tc_tile_buffer(size_t bytes, int4** out)
-{
-    int dev = 0;
-    FMM_CUDA_TRY(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= 64) return fail(FMM_EUNSUPPORTED, "fgt_h2p: device ordinal %d above 63", dev);
-    std::lock_guard<std::mutex> lk(g_img_mu);
-    if (g_tiles_bytes[dev] < bytes) {
-        if (g_tiles[dev]) {
-            FMM_CUDA_TRY(cudaDeviceSynchronize());
-            cudaFree(g_tiles[dev]);
-            g_tiles[dev] = nullptr;
-            g_tiles_bytes[dev] = 0;
-        }
-        FMM_CUDA_TRY(cudaMalloc(&g_tiles[dev], bytes));
-        g_tiles_bytes[dev] = bytes;
-    }
-    *out = reinterpret_cast<int4*>(g_tiles[dev]);
-    return FMM_OK;
-}
+// The BF16 image of A and the tile table.
+static KeptBuffer g_image, g_tiles;
 
 int launch_fgt_h2p_tc(int g, int ncut, double d, bool split, const float* A, const double* y, int n, const int* perm,
                       const int* box_start, const int* claims, float* G, bool accumulate, int* err, cudaStream_t st)
@@ -451,7 +405,7 @@ int launch_fgt_h2p_tc(int g, int ncut, double d, bool split, const float* A, con
     if (ncut > kTcMaxCut) return fail(FMM_EUNSUPPORTED, "fgt_h2p: tensor-core form needs n_cut <= %d", kTcMaxCut);
     const int nbox = 1 << (2 * g);
     unsigned char* img = nullptr;
-    if (int rc = tc_image_buffer((size_t)nbox * 2 * kTcBoxBytes, &img)) return rc;
+    if (int rc = kept_buffer(g_image, (size_t)nbox * 2 * kTcBoxBytes, (void**)&img)) return rc;
     const int64_t elems = (int64_t)nbox * 256;
     fgt_tc_image_kernel<<<(unsigned)((elems + 255) / 256), 256, 0, st>>>(A, nbox, img);
     FMM_CUDA_TRY(cudaGetLastError());
@@ -463,7 +417,7 @@ int launch_fgt_h2p_tc(int g, int ncut, double d, bool split, const float* A, con
     if (smem < kTcMinSmem) smem = kTcMinSmem;
     const int max_claims = (int)std::min<int64_t>((int64_t)n / kTcRows + nbox, INT32_MAX);
     int4* tiles = nullptr;
-    if (int rc = tc_tile_buffer((size_t)max_claims * sizeof(int4), &tiles)) return rc;
+    if (int rc = kept_buffer(g_tiles, (size_t)max_claims * sizeof(int4), (void**)&tiles)) return rc;
     h2p_tiles_kernel<<<(max_claims + 255) / 256, 256, 0, st>>>(claims, box_start, nbox, n, max_claims, tiles);
     FMM_CUDA_TRY(cudaGetLastError());
     int sms = 0;

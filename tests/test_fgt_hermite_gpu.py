@@ -508,8 +508,8 @@ def test_h2p_nan_coefficients_reach_their_neighbourhood_only(fmm, orc):
 
 
 def test_h2p_first_call_of_a_grid_size_inside_a_capture(fmm, orc):
-    """The coefficients' workspace of a grid size is allocated on its first use; a first use inside
-    a stream capture takes the direct sum instead, and the graph replays beside later calls."""
+    """The coefficients' workspace of a grid size is allocated on its first use, inside a stream capture
+    too: the graph replays what direct calls give, beside them."""
     import math
     import torch
 
@@ -545,6 +545,54 @@ def test_h2p_first_call_of_a_grid_size_inside_a_capture(fmm, orc):
     ref = orc.fgt_hermite_eval_grid(g, ncut, p, sigma, A32.astype(np.float64), y[pick])
     for t in (first, second, G):
         _check(t.cpu().numpy().astype(np.float64)[pick], ref)
+    assert torch.equal(first, second) and torch.equal(first, G)
+
+
+@pytest.mark.parametrize("prec", ["fp32", "bf16x3", "bf16"])
+def test_h2p_captures_after_a_call_of_the_other_form(prec):
+    """A program whose only call was served through the Chebyshev coefficients captures one that takes the
+    direct sums (their scratch, and the tensor cores' image and tile table, come inside the
+    capture), and one of a grid not used before: in a process of its own, where nothing else
+    has been allocated."""
+    import os
+    import subprocess
+    import sys
+
+    code = f"""
+import math, torch
+from paper_1009_3457_gb300 import fmmgb as fmm
+prec = {{"fp32": fmm.FMM_FP32, "bf16x3": fmm.FMM_TC_BF16X3, "bf16": fmm.FMM_TC_BF16}}[{prec!r}]
+torch.manual_seed(1)
+def problem(g, n):
+    y = torch.rand((n, 2), dtype=torch.float64, device="cuda")
+    i = dict(dtype=torch.int32, device="cuda")
+    perm, start, work = torch.empty(n, **i), torch.empty(4 ** g + 1, **i), torch.empty(4 ** g, **i)
+    fmm.fgt_bin_points(g, y, perm, start, work)
+    A, G = torch.rand((4 ** g, 16, 16), device="cuda"), torch.empty(n, device="cuda")
+    A *= 0.1 ** torch.arange(16, device="cuda")[:, None] * 0.1 ** torch.arange(16, device="cuda")
+    sigma = 2.0 ** -g / (math.sqrt(2.0) * 0.45)
+    return G, lambda: fmm.fgt_h2p(g, 3, 16, sigma, A, y, perm, start, G, prec=prec)
+problem(4, 2000)[1]()
+todo = [problem(4, 300), problem(5, 700), problem(5, 4000)]
+torch.cuda.synchronize()
+graphs = []
+for G, call in todo:
+    graphs.append(torch.cuda.CUDAGraph())
+    with torch.cuda.graph(graphs[-1], capture_error_mode="thread_local"):
+        call()
+for graph, (G, call) in zip(graphs, todo):
+    graph.replay()
+    fmm.fmm_sync_status()
+    got = G.clone()
+    G.fill_(float("nan"))
+    call()
+    fmm.fmm_sync_status()
+    assert torch.equal(got, G) and bool(torch.isfinite(G).all())
+print("captured")
+"""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and "captured" in r.stdout, r.stdout + r.stderr
 
 
 @pytest.mark.parametrize("p", [4, 8, 12, 16])
