@@ -95,7 +95,9 @@ __device__ __forceinline__ float pow2_neg(int k) { return __int_as_float((127 - 
 // launch).  A kernel launched by launch_after calls after_wait() before it touches global memory
 // that anything before it in the stream may write or read, and every thread of it does.  What a
 // wait releases is complete and visible, and so is everything before it: each kernel of a chain
-// waits for its own predecessor.  Without after_go() in its predecessor such a kernel is set up while
+// waits for its own predecessor.  Such a kernel, and what it calls, reads by plain (or .cg) loads: the
+// non-coherent ones (__ldg, const __restrict__ parameters) are for data that does not change while the grid
+// runs, and the grid starts before its predecessor ends.  Without after_go() in its predecessor such a kernel is set up while
 // that one ends, with it as soon as all of that one's CTAs have started: only the short kernels of the
 // FGT and of the binning call it, since CTAs that wait hold their registers (in the whole FMM, where
 // the far field runs beside the near field, calling it in the M2L and shift kernels cost 2 %).

@@ -152,8 +152,8 @@ __device__ __forceinline__ int float_key(float x)
 
 template <int P, int R, int Q, bool LAST>
 __global__ void __launch_bounds__(kSeg* kTaps* R)
-    cheb_pass_kernel(int side, int ncut, const float* __restrict__ in, const float* __restrict__ W, float* __restrict__ out,
-                     float d, ChebLimits l, const int* box_start)
+    cheb_pass_kernel(int side, int ncut, const float* in, const float* W, float* __restrict__ out, float d, ChebLimits l,
+                     const int* box_start)
 {
     __shared__ float2 s_lim[kSeg + 2 * kChebMaxCut];  // of the window's boxes
     __shared__ bool s_apart[kSeg];
@@ -168,14 +168,14 @@ __global__ void __launch_bounds__(kSeg* kTaps* R)
     const int nwin = kSeg + 2 * ncut;
     static_assert(C::THREADS >= kSeg + 2 * kChebMaxCut);
     for (int i = tid; i < taps * P * Q / 4; i += C::THREADS)
-        reinterpret_cast<float4*>(s_tab)[i] = __ldg(reinterpret_cast<const float4*>(W) + i);
+        reinterpret_cast<float4*>(s_tab)[i] = reinterpret_cast<const float4*>(W)[i];
     float2 lim = make_float2(-INFINITY, -INFINITY);
     if (const int s = t0 - ncut + tid; tid < nwin && s >= 0 && s < side) lim = (LAST ? l.line : l.box)[line * side + s];
     constexpr int B4 = P * R / 4;
     for (int i = tid; i < nwin * B4; i += C::THREADS) {
         const int b = i / B4, s = t0 - ncut + b;
         float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (s >= 0 && s < side) v = __ldg(reinterpret_cast<const float4*>(in + ((size_t)line * side + s) * P * R) + i % B4);
+        if (s >= 0 && s < side) v = reinterpret_cast<const float4*>(in + ((size_t)line * side + s) * P * R)[i % B4];
         *reinterpret_cast<float4*>(s_win + b * C::BOX + 4 * (i % B4)) = v;
     }
     if (tid < nwin) s_lim[tid] = lim;
@@ -286,7 +286,7 @@ __device__ __noinline__ float cheb_direct(const ChebEval& a, int box, double y0,
             float t = fmaf(tt, c1, -(float)(2 * (a1 + 1)) * c2);
 #pragma unroll
             for (int q = 0; q < P / 4; ++q) {
-                const float4 v = __ldg(Ab + a1 * (P / 4) + q);
+                const float4 v = Ab[a1 * (P / 4) + q];
                 t = fmaf(v.x, h2[4 * q], t);
                 t = fmaf(v.y, h2[4 * q + 1], t);
                 t = fmaf(v.z, h2[4 * q + 2], t);
@@ -328,7 +328,7 @@ __device__ __noinline__ float cheb_apart(const ChebEval& a, int box, double y0, 
 
 // sum_{m,l} c[m][l] T_m(x1) T_l(x2) for NR targets of one box (or, with NR = 1, of a box per lane).
 template <int Q, int NR>
-__device__ __forceinline__ void cheb_sum(const float* __restrict__ c, const float* x1, const float* x2, float* out)
+__device__ __forceinline__ void cheb_sum(const float* c, const float* x1, const float* x2, float* out)
 {
     float T[NR][Q], b1[NR], b2[NR];
 #pragma unroll
@@ -347,7 +347,7 @@ __device__ __forceinline__ void cheb_sum(const float* __restrict__ c, const floa
         for (int r = 0; r < NR; ++r) row[r] = fmaf(m ? x1[r] + x1[r] : x1[r], b1[r], -b2[r]);
 #pragma unroll
         for (int q = 0; q < Q / 4; ++q) {
-            const float4 v = __ldg(c4 + m * (Q / 4) + q);
+            const float4 v = c4[m * (Q / 4) + q];
 #pragma unroll
             for (int r = 0; r < NR; ++r) {
                 row[r] = fmaf(v.x, T[r][4 * q], row[r]);
@@ -373,19 +373,18 @@ __device__ __forceinline__ void cheb_sum(const float* __restrict__ c, const floa
 // trips a warp instead of three a row (2^20 targets: 30 -> 26 us; fewer rows a lane, for more warps on an
 // SM, measured the same).
 template <int NR>
-__device__ __forceinline__ void binned_targets(const double* __restrict__ y, const int* __restrict__ perm,
-                                               const int* __restrict__ box_start, int g, int n, int64_t base, int* err,
-                                               int* tj, int* tb, float* o0, float* o1)
+__device__ __forceinline__ void binned_targets(const double* y, const int* perm, const int* box_start, int g, int n,
+                                               int64_t base, int* err, int* tj, int* tb, float* o0, float* o1)
 {
     double y0[NR], y1[NR];
     int f[NR], e[NR];
 #pragma unroll
-    for (int r = 0; r < NR; ++r) tj[r] = base + 32 * r < n ? __ldg(perm + base + 32 * r) : -1;
+    for (int r = 0; r < NR; ++r) tj[r] = base + 32 * r < n ? perm[base + 32 * r] : -1;
 #pragma unroll
     for (int r = 0; r < NR; ++r) {
         const size_t j = (unsigned)tj[r] < (unsigned)n ? tj[r] : 0;
-        y0[r] = __ldg(y + 2 * j);
-        y1[r] = __ldg(y + 2 * j + 1);
+        y0[r] = y[2 * j];
+        y1[r] = y[2 * j + 1];
     }
 #pragma unroll
     for (int r = 0; r < NR; ++r) {
@@ -397,8 +396,8 @@ __device__ __forceinline__ void binned_targets(const double* __restrict__ y, con
             o0[r] = cell_offset31(X0);
             o1[r] = cell_offset31(X1);
         }
-        f[r] = __ldg(box_start + max(tb[r], 0));
-        e[r] = __ldg(box_start + max(tb[r], 0) + 1);
+        f[r] = box_start[max(tb[r], 0)];
+        e[r] = box_start[max(tb[r], 0) + 1];
     }
 #pragma unroll
     for (int r = 0; r < NR; ++r) {
@@ -458,8 +457,8 @@ __device__ __forceinline__ void cheb_eval_warp(const ChebEval& a, int64_t base)
                     if (lo >= 0 && a.apart[lo]) {
                         lo = j = -1;
                     } else if (lo >= 0) {
-                        y0 = __ldg(a.y + 2 * (size_t)j);
-                        y1 = __ldg(a.y + 2 * (size_t)j + 1);
+                        y0 = a.y[2 * (size_t)j];
+                        y1 = a.y[2 * (size_t)j + 1];
                     } else {  // box_start does not bin [0, n)
                         atomicOr(a.err, DEV_ERR_CHECK);
                         j = -1;

@@ -65,13 +65,13 @@ constexpr int kT2pRows = 4;
 template <bool VEC>
 __device__ __forceinline__ float4 t2p_load4(const float* c)
 {
-    if constexpr (VEC) return __ldg(reinterpret_cast<const float4*>(c));
-    return make_float4(__ldg(c), __ldg(c + 1), __ldg(c + 2), __ldg(c + 3));
+    if constexpr (VEC) return *reinterpret_cast<const float4*>(c);
+    return make_float4(c[0], c[1], c[2], c[3]);
 }
 
 // sum_{b1,b2} c[b1][b2] t1^b1 t2^b2 by Horner's rule, NR targets of one box (NR = 1: a box per lane)
 template <int P, int NR, bool VEC>
-__device__ __forceinline__ void t2p_sum(const float* __restrict__ c, const float* t1, const float* t2, float* out)
+__device__ __forceinline__ void t2p_sum(const float* c, const float* t1, const float* t2, float* out)
 {
 #pragma unroll
     for (int r = 0; r < NR; ++r) out[r] = 0.f;
@@ -98,10 +98,8 @@ __device__ __forceinline__ void t2p_sum(const float* __restrict__ c, const float
 
 template <int P, bool VEC>
 __global__ void __launch_bounds__(kT2pThreads) fgt_t2p_binned_kernel(int g, double inv_scale, float dcell,
-                                                                     const float* __restrict__ C, int n,
-                                                                     const double* __restrict__ y,
-                                                                     const int* __restrict__ perm,
-                                                                     const int* __restrict__ box_start,
+                                                                     const float* C, int n, const double* y,
+                                                                     const int* perm, const int* box_start,
                                                                      float* __restrict__ G, int accumulate, int* err)
 {
     const int lane = threadIdx.x & 31, side = 1 << g, nbox = side * side;
@@ -117,12 +115,12 @@ __global__ void __launch_bounds__(kT2pThreads) fgt_t2p_binned_kernel(int g, doub
         tj[r] = tb[r] = -1;
         t1[r] = t2[r] = out[r] = 0.f;
         if (pos >= n) continue;
-        const int j = __ldg(perm + pos);
+        const int j = perm[pos];
         if ((unsigned)j >= (unsigned)n) {
             atomicOr(err, DEV_ERR_CHECK);
             continue;
         }
-        const double y0 = __ldg(y + 2 * (size_t)j), y1 = __ldg(y + 2 * (size_t)j + 1);
+        const double y0 = y[2 * (size_t)j], y1 = y[2 * (size_t)j + 1];
         long long X0, X1;
         if (grid_fixed31(y0, g, X0) && grid_fixed31(y1, g, X1)) {
             const int b = (int)(X1 >> 31) * side + (int)(X0 >> 31);

@@ -136,7 +136,7 @@ __global__ void __launch_bounds__(kScanThreads) bin_scan_kernel(int nbox, int* c
 // 735 -> 95 us.
 constexpr int kScanTile = 4096;
 
-__global__ void __launch_bounds__(kScanThreads) bin_scan_tiles_kernel(int nbox, const int* __restrict__ counts,
+__global__ void __launch_bounds__(kScanThreads) bin_scan_tiles_kernel(int nbox, const int* counts,
                                                                       int* __restrict__ box_start)
 {
     __shared__ int s_warp[kScanThreads / 32], s_before;
@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(kScanThreads) bin_scan_tiles_kernel(int nbox, 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, first = blockIdx.x * kScanTile;
     int before = 0;
 #pragma unroll 4
-    for (int i = tid; i < first; i += kScanThreads) before += __ldg(counts + i);
+    for (int i = tid; i < first; i += kScanThreads) before += counts[i];
     before = __reduce_add_sync(0xffffffffu, before);
     if (lane == 0) s_warp[warp] = before;
     __syncthreads();
@@ -158,7 +158,7 @@ __global__ void __launch_bounds__(kScanThreads) bin_scan_tiles_kernel(int nbox, 
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         const int i = first + 4 * tid + k;
-        c[k] = i < nbox ? __ldg(counts + i) : 0;
+        c[k] = i < nbox ? counts[i] : 0;
         sum += c[k];
     }
     int x = sum;
@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(kScanThreads) bin_scan_tiles_kernel(int nbox, 
     }
 }
 
-__global__ void bin_scatter_kernel(int g, const double* __restrict__ y, int64_t n, int* __restrict__ cursor,
+__global__ void bin_scatter_kernel(int g, const double* y, int64_t n, int* __restrict__ cursor,
                                    int* __restrict__ perm)
 {
     after_go();
@@ -200,7 +200,7 @@ __global__ void bin_scatter_kernel(int g, const double* __restrict__ y, int64_t 
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t w = w0; 32 * w < n; w += nw) {
         const int64_t i = 32 * w + lane;
-        const int key = i < n ? fgt_grid_box(__ldg(y + 2 * i), __ldg(y + 2 * i + 1), g) : -1;
+        const int key = i < n ? fgt_grid_box(y[2 * i], y[2 * i + 1], g) : -1;
         const int slot = warp_box_claim(cursor, key);
         if (slot >= 0) perm[slot] = (int)i;
     }
@@ -223,14 +223,14 @@ constexpr int kBinSmemMaxLog2 = 7;
 //     threads; the Hermite transform of 3e5 points 79 us against 84 with 512).
 // Coordinates of the points first, first + T, ... (LOADS of them, below i1).
 template <int T, int LOADS>
-__device__ __forceinline__ void load_points(const double* __restrict__ y, int64_t first, int64_t i1,
+__device__ __forceinline__ void load_points(const double* y, int64_t first, int64_t i1,
                                             double (&a)[LOADS], double (&b)[LOADS])
 {
 #pragma unroll
     for (int u = 0; u < LOADS; ++u) {
         const int64_t k = first + u * T;
-        a[u] = k < i1 ? __ldg(y + 2 * k) : 0.0;
-        b[u] = k < i1 ? __ldg(y + 2 * k + 1) : 0.0;
+        a[u] = k < i1 ? y[2 * k] : 0.0;
+        b[u] = k < i1 ? y[2 * k + 1] : 0.0;
     }
 }
 
@@ -261,7 +261,7 @@ __global__ void __launch_bounds__(T) bin_count_smem_kernel(int g, const double* 
 // touched box's range with one global atomic, and a point goes to that range's start + rank.  The
 // coordinates are read once, with one shared atomic a point (a second pass over both before).
 template <int T, int LOADS>
-__global__ void __launch_bounds__(T) bin_scatter_smem_kernel(int g, const double* __restrict__ y, int64_t n, int64_t chunk,
+__global__ void __launch_bounds__(T) bin_scatter_smem_kernel(int g, const double* y, int64_t n, int64_t chunk,
                                                              int* __restrict__ cursor, int* __restrict__ perm)
 {
     after_go();

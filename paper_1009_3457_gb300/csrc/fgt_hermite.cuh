@@ -21,24 +21,24 @@ __device__ __forceinline__ void hermite_functions(float t, float (&h)[P])
 // Binned targets taken by place rather than by box.  bin_check (all threads of the grid): a box
 // whose start or end lies outside [0, n] or that ends before it starts sets the error word.
 __device__ __forceinline__ bool bin_range_ok(int first, int end, int n) { return 0 <= first && first <= end && end <= n; }
-__device__ __forceinline__ void bin_check(const int* __restrict__ box_start, int nbox, int n, int* err)
+__device__ __forceinline__ void bin_check(const int* box_start, int nbox, int n, int* err)
 {
     for (int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; b < nbox; b += (int64_t)gridDim.x * blockDim.x)
-        if (!bin_range_ok(__ldg(box_start + b), __ldg(box_start + b + 1), n)) atomicOr(err, DEV_ERR_CHECK);
+        if (!bin_range_ok(box_start[b], box_start[b + 1], n)) atomicOr(err, DEV_ERR_CHECK);
 }
 // Whether place pos lies in box b's run.
-__device__ __forceinline__ bool bin_holds(const int* __restrict__ box_start, int b, int pos, int n)
+__device__ __forceinline__ bool bin_holds(const int* box_start, int b, int pos, int n)
 {
-    const int f = __ldg(box_start + b), e = __ldg(box_start + b + 1);
+    const int f = box_start[b], e = box_start[b + 1];
     return bin_range_ok(f, e, n) && f <= pos && pos < e;
 }
 // The box whose run holds place pos (by bisection), -1 if none does.
-__device__ __forceinline__ int bin_find(const int* __restrict__ box_start, int nbox, int pos, int n)
+__device__ __forceinline__ int bin_find(const int* box_start, int nbox, int pos, int n)
 {
     int lo = 0, hi = nbox;
     while (hi - lo > 1) {
         const int mid = (lo + hi) >> 1;
-        if (__ldg(box_start + mid) <= pos) lo = mid;
+        if (box_start[mid] <= pos) lo = mid;
         else hi = mid;
     }
     return bin_holds(box_start, lo, pos, n) ? lo : -1;
@@ -182,11 +182,11 @@ __device__ __forceinline__ void h2p_run(const H2pSums& a, H2pShared<NT>& sh, flo
         tj[r] = -1;
         u1[r] = u2[r] = acc[r] = 0.f;
         if (pos < end) {
-            const int j = __ldg(a.perm + pos);
+            const int j = a.perm[pos];
             if ((unsigned)j < (unsigned)a.n) {
                 tj[r] = j;
-                u1[r] = (float)((__ldg(a.y + 2 * (size_t)j) * side - (tx + 0.5)) * a.d);
-                u2[r] = (float)((__ldg(a.y + 2 * (size_t)j + 1) * side - (ty + 0.5)) * a.d);
+                u1[r] = (float)((a.y[2 * (size_t)j] * side - (tx + 0.5)) * a.d);
+                u2[r] = (float)((a.y[2 * (size_t)j + 1] * side - (ty + 0.5)) * a.d);
             } else {
                 atomicOr(a.err, DEV_ERR_CHECK);
             }

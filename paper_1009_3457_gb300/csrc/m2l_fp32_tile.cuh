@@ -452,7 +452,7 @@ __device__ __forceinline__ void m2l_tile(unsigned char* raw, const TileGeom& g, 
             }
             if constexpr (ADAPTIVE)
                 if (in && g.exists) in = g.exists[(size_t)iy * g.side + ix] != 0;  // V-list: existing sources only
-            if (in) v[u] = __ldg(M4 + ((size_t)iy * g.side + ix) * Q + q);
+            if (in) v[u] = __ldcg(M4 + ((size_t)iy * g.side + ix) * Q + q);
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
@@ -546,8 +546,8 @@ __device__ __forceinline__ void m2l_tile(unsigned char* raw, const TileGeom& g, 
 // ---------------------------------------------------------------------------
 template <int P, bool ADAPTIVE>
 __global__ void __launch_bounds__(M2LCfg<P>::THREADS, M2LCfg<P>::MIN_CTAS)
-    m2l_fp32_kernel(const __grid_constant__ M2LLaunch job, const float* __restrict__ ascale,
-                    const float* __restrict__ bscale, int total, int* __restrict__ counter)
+    m2l_fp32_kernel(const __grid_constant__ M2LLaunch job, const float* ascale,
+                    const float* bscale, int total, int* __restrict__ counter)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int s_next;

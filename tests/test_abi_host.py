@@ -358,3 +358,42 @@ def test_wait_probe_rejects_bad_arguments(fmm):
     assert lib.fmm_wait_probe((1 << 22) + 1, 0, None) == fmm.FMM_EINVAL
     assert "cap" in fmm.fmm_last_error()
     assert lib.fmm_wait_probe(8, 2, None) == fmm.FMM_EINVAL
+
+
+def _device_functions():
+    """{name: (signature, body)} of the functions of csrc, comments removed."""
+    src = os.path.join(ROOT, "paper_1009_3457_gb300", "csrc")
+    out = {}
+    for fn in sorted(os.listdir(src)):
+        if not fn.endswith((".cu", ".cuh")):
+            continue
+        text = re.sub(r"//[^\n]*", "", open(os.path.join(src, fn)).read())
+        for m in re.finditer(r"__(?:global|device)__[^;{}=]*?(?:__launch_bounds__\([^{;]*?\)\s*)?(\w+)\(([^{};]*)\)\s*\{", text):
+            depth, end = 1, m.end()
+            while depth:
+                depth += {"{": 1, "}": -1}.get(text[end], 0)
+                end += 1
+            out.setdefault(m.group(1), []).append((m.group(2), text[m.end():end]))
+    return out
+
+
+def test_kernels_that_start_early_read_coherently():
+    """A kernel launched by launch_after starts while its predecessor runs and waits inside, so
+    what it reads after the wait was written while its grid was up: neither it nor what it calls may use
+    the non-coherent loads (__ldg; const __restrict__ parameters), which are for data that stays
+    as it is for the whole grid."""
+    funcs = _device_functions()
+    early = {n for n, defs in funcs.items() if any("after_wait();" in b for _, b in defs)}
+    assert {"cheb_eval_kernel", "cheb_pass_kernel", "bin_scatter_smem_kernel", "m2l_fp32_kernel", "shift_kernel",
+            "fgt_t2p_binned_kernel"} <= early
+    reached, todo = set(), list(early)
+    while todo:
+        n = todo.pop()
+        if n in reached:
+            continue
+        reached.add(n)
+        for _, body in funcs[n]:
+            todo += [w for w in re.findall(r"\b(\w+)\s*(?:<[^;(){}]*>)?\(", body) if w in funcs]
+    bad = [n for n in sorted(reached) if any("__ldg(" in b for _, b in funcs[n])]
+    bad += [n for n in sorted(early) if any(re.search(r"const \w+\* __restrict__", s) for s, _ in funcs[n])]
+    assert not bad, bad
