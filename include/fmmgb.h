@@ -630,7 +630,7 @@ int fgt_h2p(int32_t grid_log2, int32_t n_cut, int32_t p, int32_t prec, double si
  *   fmm_bin_points(level, z, nz, ...); phi: device complex64 [nz], indexed
  *   like z.  level 0..10, n and nz < 2^31.
  *   flags   FMM_ACCUMULATE; FMM_P2P_SHARE_SM: thread blocks that end after
- *           two runs of targets instead of staying to the end, so that kernels
+ *           one or two runs of targets instead of staying to the end, so that kernels
  *           of a stream of higher priority find room on the SMs (the far
  *           field of the same FMM: 1.24 -> 1.16 ms for the whole potential at
  *           2^22 points).  The result is the same, bit for bit.

@@ -42,8 +42,12 @@ constexpr int kP2pBatch = 1024;                 // sources per shared-memory bat
 // a stream of higher priority take its place; a persistent CTA would hold its registers to the end.  The
 // potential of 2^22 points with the far field beside it: 1,240 us with persistent CTAs (8 per SM), 1,167 /
 // 1,157 / 1,163 / 1,169 with 1 / 2 / 3 / 4 claims; the near field alone 923 us persistent, 925 with 2.  A warp a claim
-// loses more alone (2^22 points at level 9 689 -> 731), so that without the flag CTAs persist.
+// loses more alone (2^22 points at level 9 689 -> 731), so that without the flag CTAs persist; but a few claims
+// go to a CTA each in any case: where some are heavy, one waits behind another in a persistent CTA,
+// and where two went to a CTA the SMs stood idle (us, persistent / two / one a CTA: 2^17 clustered points at level 6
+// 218 / 243 / 186, 2^15 at level 5 73 / 80 / 57, 2^15 uniform 24 / 24 / 22).
 constexpr int kP2pShareClaims = 2;
+constexpr int kP2pShareOne = 1 << 14;           // a CTA (warp) each for fewer claims
 constexpr int kP2pShareGrid = 1 << 16;          // more claims a CTA rather than more CTAs (most find none)
 // The warp kernel takes calls of fewer than kP2pDense targets a box on average, on kP2wBoxes boxes or
 // more (fewer claims than warps otherwise).  us, CTA / warp: 16 a box at level 5 26 / 35, level 6 31 / 35,
@@ -591,10 +595,7 @@ extern "C" int fmm_p2p(int32_t level, const double* xy, const double* c, int64_t
     args.tperm = tgt_perm;
     args.tstart = tgt_start;
     args.phi = reinterpret_cast<float2*>(phi);
-    const bool share = (flags & FMM_P2P_SHARE_SM) != 0;
     args.cursor = nullptr;
-    if (!share)
-        if (int rc = tile_counter(&args.cursor, st)) return rc;
     if (int rc = device_error_word(&args.err)) return rc;
     const int nbox = 1 << (2 * level);
     const bool dense = nz >= (int64_t)kP2pDense * nbox || nbox < kP2wBoxes;
@@ -619,12 +620,14 @@ extern "C" int fmm_p2p(int32_t level, const double* xy, const double* c, int64_t
     args.ntab = (int)most;
     auto kern = dense ? fmm_p2p_kernel : fmm_p2p_warp_kernel;
     const int64_t ctas = dense ? most : (most + kP2pThreads / 32 - 1) / (kP2pThreads / 32);
+    const bool share = (flags & FMM_P2P_SHARE_SM) || (dense && ctas <= kP2pShareOne);
     int64_t grid = 0;
     args.each = 0;
     if (share) {
-        args.each = (int)std::max<int64_t>(kP2pShareClaims, (ctas + kP2pShareGrid - 1) / kP2pShareGrid);
+        args.each = ctas <= kP2pShareOne ? 1 : (int)std::max<int64_t>(kP2pShareClaims, (ctas + kP2pShareGrid - 1) / kP2pShareGrid);
         grid = (ctas + args.each - 1) / args.each;
     } else {
+        if (int rc = tile_counter(&args.cursor, st)) return rc;
         static int occ_cache[2];
         static std::mutex mu;
         int sms = 0, occ = 0;
