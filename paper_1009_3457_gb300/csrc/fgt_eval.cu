@@ -59,8 +59,11 @@ static int t2p_p(int g, double sigma, const float* C, int64_t n, const double* y
 // multiply-add is gone.  Target offsets are read off the bits of the FP64 coordinates.
 // 2^20 uniform targets on 32 x 32 boxes, p = 16: 40 -> 26 us, bound by the gathers and the
 // scattered results.
+// Fewer than kT2pWide targets leave the SMs warps to spare: one target a lane, since four rows
+// one after the other are four times the latency (p = 16, 32 x 32 boxes, us, one / four: 300 targets 7.0 / 16.7,
+// 10^4 4.7 / 12.3, 2*10^5 9.5 / 11.3, 3*10^5 14.1 / 12.0, 2^20 38 / 26).
 constexpr int kT2pThreads = 128;
-constexpr int kT2pRows = 4;
+constexpr int64_t kT2pWide = 1 << 18;
 
 template <bool VEC>
 __device__ __forceinline__ float4 t2p_load4(const float* c)
@@ -75,7 +78,7 @@ __device__ __forceinline__ void t2p_sum(const float* c, const float* t1, const f
 {
 #pragma unroll
     for (int r = 0; r < NR; ++r) out[r] = 0.f;
-#pragma unroll 4
+#pragma unroll (NR == 1 ? P : 4)
     for (int b1 = P - 1; b1 >= 0; --b1) {
         float inner[NR];
 #pragma unroll
@@ -96,7 +99,7 @@ __device__ __forceinline__ void t2p_sum(const float* c, const float* t1, const f
     }
 }
 
-template <int P, bool VEC>
+template <int P, bool VEC, int ROWS>
 __global__ void __launch_bounds__(kT2pThreads) fgt_t2p_binned_kernel(int g, double inv_scale, float dcell,
                                                                      const float* C, int n, const double* y,
                                                                      const int* perm, const int* box_start,
@@ -104,13 +107,13 @@ __global__ void __launch_bounds__(kT2pThreads) fgt_t2p_binned_kernel(int g, doub
 {
     const int lane = threadIdx.x & 31, side = 1 << g, nbox = side * side;
     after_wait();
-    const int64_t base = ((int64_t)blockIdx.x * (kT2pThreads / 32) + (threadIdx.x >> 5)) * (32 * kT2pRows);
+    const int64_t base = ((int64_t)blockIdx.x * (kT2pThreads / 32) + (threadIdx.x >> 5)) * (32 * ROWS);
     bin_check(box_start, nbox, n, err);
     if (base >= n) return;
-    int tj[kT2pRows], tb[kT2pRows];
-    float t1[kT2pRows], t2[kT2pRows], out[kT2pRows];
+    int tj[ROWS], tb[ROWS];
+    float t1[ROWS], t2[ROWS], out[ROWS];
 #pragma unroll
-    for (int r = 0; r < kT2pRows; ++r) {
+    for (int r = 0; r < ROWS; ++r) {
         const int64_t pos = base + 32 * r + lane;
         tj[r] = tb[r] = -1;
         t1[r] = t2[r] = out[r] = 0.f;
@@ -146,16 +149,16 @@ __global__ void __launch_bounds__(kT2pThreads) fgt_t2p_binned_kernel(int g, doub
     const int b0 = __shfl_sync(0xffffffffu, tb[0], 0);
     bool same = b0 >= 0;
 #pragma unroll
-    for (int r = 0; r < kT2pRows; ++r) same &= tb[r] == b0 || base + 32 * r + lane >= n;
+    for (int r = 0; r < ROWS; ++r) same &= tb[r] == b0 || base + 32 * r + lane >= n;
     if (__all_sync(0xffffffffu, same)) {
-        t2p_sum<P, kT2pRows, VEC>(C + (size_t)b0 * P * P, t1, t2, out);
+        t2p_sum<P, ROWS, VEC>(C + (size_t)b0 * P * P, t1, t2, out);
     } else {
 #pragma unroll
-        for (int r = 0; r < kT2pRows; ++r)
+        for (int r = 0; r < ROWS; ++r)
             if (tb[r] >= 0) t2p_sum<P, 1, VEC>(C + (size_t)tb[r] * P * P, t1 + r, t2 + r, out + r);
     }
 #pragma unroll
-    for (int r = 0; r < kT2pRows; ++r)
+    for (int r = 0; r < ROWS; ++r)
         if (tj[r] >= 0) G[tj[r]] = accumulate ? G[tj[r]] + out[r] : out[r];
 }
 
@@ -165,8 +168,10 @@ static int t2p_binned_p(int g, double sigma, const float* C, int n, const double
 {
     const double inv_scale = 1.0 / (sqrt(2.0) * sigma);
     const float dcell = (float)(ldexp(1.0, -g) * inv_scale);
-    const unsigned grid = bin_blocks(n, kT2pThreads * kT2pRows, (int64_t)1 << (2 * g), kT2pThreads);
-    auto kern = ((uintptr_t)C & 15) == 0 ? fgt_t2p_binned_kernel<P, true> : fgt_t2p_binned_kernel<P, false>;
+    const bool wide = n >= kT2pWide, vec = ((uintptr_t)C & 15) == 0;
+    const unsigned grid = bin_blocks(n, kT2pThreads * (wide ? 4 : 1), (int64_t)1 << (2 * g), kT2pThreads);
+    auto kern = wide ? (vec ? fgt_t2p_binned_kernel<P, true, 4> : fgt_t2p_binned_kernel<P, false, 4>)
+                     : (vec ? fgt_t2p_binned_kernel<P, true, 1> : fgt_t2p_binned_kernel<P, false, 1>);
     FMM_CUDA_TRY(launch_after(kern, grid, kT2pThreads, 0, st, g, inv_scale, dcell, C, n, y, perm, box_start, G, acc ? 1 : 0,
                               err));
     return FMM_OK;

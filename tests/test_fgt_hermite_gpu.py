@@ -625,6 +625,31 @@ def test_p2h_and_t2p_binned_runs_and_alignments(fmm, orc, p):
         _check(G.cpu().numpy().astype(np.float64), ev)
 
 
+@pytest.mark.parametrize("p", [4, 8, 12, 16])
+@pytest.mark.parametrize("g,n", [(0, 1), (0, 33), (2, 31), (2, 129), (5, 1000), (5, 2 ** 18 - 1), (5, 2 ** 18), (8, 3000)])
+def test_t2p_binned_one_and_four_targets_a_lane(fmm, orc, p, g, n):
+    """T2P on both sides of the line between one and four targets a lane, from coefficients 16-byte aligned and
+    not, added and written: boxes of one target and of many, the last warp ragged."""
+    import torch
+
+    rng = np.random.default_rng(1000 * g + p)
+    sigma = 2.0 ** -g / (np.sqrt(2.0) * 0.4)
+    C = rng.standard_normal((4 ** g, p, p)).astype(np.float32)
+    y = np.concatenate([rng.random((n - n // 3, 2)), 0.3 + 0.2 * rng.random((n // 3, 2))])
+    pick = rng.choice(n, min(n, 500), replace=False)
+    ref = orc.fgt_taylor_eval_grid(g, p, sigma, C.astype(np.float64), y[pick])
+    yd = torch.from_numpy(y).cuda()
+    perm, start = _bin(fmm, g, yd)
+    for shift in (0, 1):
+        Cd = torch.empty(C.size + 1, device="cuda")[shift:shift + C.size].view(C.shape)
+        Cd.copy_(torch.from_numpy(C))
+        for acc in (False, True):
+            G = torch.full((n,), 0.5, dtype=torch.float32, device="cuda")
+            fmm.fgt_t2p_binned(g, p, sigma, Cd, yd, perm, start, G, accumulate=acc)
+            fmm.fmm_sync_status()
+            _check(G.cpu().numpy().astype(np.float64)[pick], ref + (0.5 if acc else 0.0))
+
+
 def test_t2p_and_h2p_report_a_bad_box_start(fmm):
     """A box start out of range, or a box that ends before it starts, sets the error word; the other
     boxes' targets are evaluated."""
