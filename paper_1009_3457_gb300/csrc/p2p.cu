@@ -11,13 +11,13 @@
 // only the exact offset between box centres (-1, 0 or 1) -- no FP64
 // arithmetic per staged source or per claim.  Runs of targets of one box are
 // claimed from a table; two kernels take them:
-//   - fmm_p2p_kernel, dense boxes or few of them: a CTA of 128 threads a claim of
+//   - fmm_p2p_kernel, dense or crowded boxes, or few boxes: a CTA of 128 threads a claim of
 //     up to 96 targets.  It gathers the sources of the 3 x 3 neighbourhood
 //     into shared memory in batches, and each warp sums the run's targets (one to
 //     three rows of 32, as many as the run fills, one target per lane and row)
 //     against a quarter of every batch; the four partial sums of a target meet in
 //     shared memory;
-//   - fmm_p2p_warp_kernel, many sparse boxes: a warp a claim of up to 64 targets, eight
+//   - fmm_p2p_warp_kernel, the sparse boxes where they are many: a warp a claim of up to 64 targets, eight
 //     lanes for the targets and four for the sources, so that a run of 16 targets
 //     fills the warp (a row of 32 lanes was half empty), and no barrier.
 // In FP32:
@@ -38,7 +38,8 @@ constexpr int kP2pWarps = kP2pThreads / 32;     // each takes a quarter of the s
 constexpr int kP2pR = 3;                        // targets per lane (rows of 32 targets per claim)
 constexpr int kP2pRun = 32 * kP2pR;             // targets per claim
 constexpr int kP2pBatch = 1024;                 // sources per shared-memory batch
-// With FMM_P2P_SHARE_SM a CTA (a warp of it in the warp kernel) ends after this many claims, and kernels of
+// With FMM_P2P_SHARE_SM a CTA (a warp of it in the warp kernel) ends after its share of the claims, one
+// or two, and kernels of
 // a stream of higher priority take its place; a persistent CTA would hold its registers to the end.  The
 // potential of 2^22 points with the far field beside it: 1,240 us with persistent CTAs (8 per SM), 1,167 /
 // 1,157 / 1,163 / 1,169 with 1 / 2 / 3 / 4 claims; the near field alone 923 us persistent, 925 with 2.  A warp a claim
@@ -46,14 +47,21 @@ constexpr int kP2pBatch = 1024;                 // sources per shared-memory bat
 // go to a CTA each in any case: where some are heavy, one waits behind another in a persistent CTA,
 // and where two went to a CTA the SMs stood idle (us, persistent / two / one a CTA: 2^17 clustered points at level 6
 // 218 / 243 / 186, 2^15 at level 5 73 / 80 / 57, 2^15 uniform 24 / 24 / 22).
-constexpr int kP2pShareClaims = 2;
 constexpr int kP2pShareOne = 1 << 14;           // a CTA (warp) each for fewer claims
 constexpr int kP2pShareGrid = 1 << 16;          // more claims a CTA rather than more CTAs (most find none)
+constexpr int kP2pSplitGrid = 64;               // CTAs per SM of the CTA kernel beside the warp kernel
 // The warp kernel takes calls of fewer than kP2pDense targets a box on average, on kP2wBoxes boxes or
 // more (fewer claims than warps otherwise).  us, CTA / warp: 16 a box at level 5 26 / 35, level 6 31 / 35,
 // level 7 68 / 62, level 8 216 / 170, level 9 914 / 676; 32 a box at level 6 41 / 55, level 7 105 / 110,
 // level 8 374 / 344; 64 a box at level 8 931 / 1,038.
 constexpr int kP2pDense = 32, kP2wBoxes = 1 << 14;
+// And of such a call only the boxes with fewer than kP2wBoxTargets targets and kP2wSources sources around
+// them; the others go to the CTA kernel, beside it.  (All boxes to the warp kernel left its warps waiting
+// for the crowded ones; us, before the warp kernel / that / so, Gaussian mixtures: 2^18 points at level 7 250 / 450 / 243,
+// at level 8 153 / 213 / 97, 2^20 at level 8 709 / 1,004 / 670, at level 9 501 / 430 / 260.  32 / 48 / 64 targets
+// with ordinary launches: 264 / 275 / 302, 133 / 143 / 172, 682 / 706 / 743, 319 / 341 / 418; 512 to 2,048 sources
+// measured alike.)
+constexpr int kP2wBoxTargets = 32, kP2wSources = 1024;
 // the warp kernel
 constexpr int kP2wLanes = 8;                    // target lanes; the other factor 4 splits the sources
 constexpr int kP2wSplit = 32 / kP2wLanes;
@@ -82,7 +90,8 @@ struct P2pArgs {
     int ntab;
     float2* phi;
     int* cursor;  // [0] next claim index, [1] CTAs finished
-    int each;     // 0, or claims per CTA (warp): consecutive places of the table, no cursor
+    int share;    // every CTA (warp) takes every gridDim-th place of the table and ends; no cursor
+    int go;       // the other kernel may start beside this one
     int* err;
 };
 
@@ -217,11 +226,42 @@ __device__ __forceinline__ void p2p_batch(const float4* __restrict__ s_src, int 
 // which claims are taken.  Places past `cap`, or a box_start that does not bin [0, nz), set the
 // error word (and those runs are skipped).  (A scan of the boxes' counts by one block, to give every
 // run a place of its own, took 73 us at 256 x 256 boxes and 290 us at 512 x 512.)
-__global__ void p2p_claim_table_kernel(int nbox, const int* __restrict__ tstart, int nz, int most, int cap,
-                                       int* nclaim, int4* __restrict__ tab, int* err)
+struct P2pTable {
+    int most, cap;
+    int* nclaim;
+    int4* tab;
+};
+
+// The whole warp: the runs of its boxes (n of [f, e) each) into the table.
+__device__ __forceinline__ void p2p_append(const P2pTable& t, int n, int f, int e, int b, int* err)
 {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
-    int f = 0, e = 0, n = 0;
+    const int lane = threadIdx.x & 31;
+    int x = n;  // inclusive scan over the warp
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += v;
+    }
+    int at = 0;
+    if (lane == 31 && x > 0) at = atomicAdd(t.nclaim, x);
+    at = __shfl_sync(0xffffffffu, at, 31) + x - n;
+    if (n <= 0) return;
+    const int run = (e - f + n - 1) / n;
+    for (int k = 0; k < n; ++k) {
+        if ((unsigned)(at + k) >= (unsigned)t.cap) {
+            atomicOr(err, DEV_ERR_CHECK);
+            return;
+        }
+        t.tab[at + k] = make_int4(f + k * run, min(f + (k + 1) * run, e), b, 0);
+    }
+}
+
+// cta: the runs of the CTA kernel; warp: of the warp kernel (cap 0: every box to the CTA kernel).
+__global__ void p2p_claim_table_kernel(int level, const int* __restrict__ tstart, int nz, const int* __restrict__ sstart,
+                                       P2pTable cta, P2pTable warp, int* err)
+{
+    const int b = blockIdx.x * blockDim.x + threadIdx.x, side = 1 << level, nbox = side * side;
+    int f = 0, e = 0;
     if (b < nbox) {
         f = tstart[b];
         e = tstart[b + 1];
@@ -230,26 +270,21 @@ __global__ void p2p_claim_table_kernel(int nbox, const int* __restrict__ tstart,
             e = min(e, nz);
             if (f < 0 || f > e) f = e = 0;
         }
-        n = (e - f + most - 1) / most;
     }
-    int x = n;  // inclusive scan over the warp
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += t;
-    }
-    int at = 0;
-    if (lane == 31 && x > 0) at = atomicAdd(nclaim, x);
-    at = __shfl_sync(0xffffffffu, at, 31) + x - n;
-    if (n <= 0) return;
-    const int run = (e - f + n - 1) / n;
-    for (int k = 0; k < n; ++k) {
-        if ((unsigned)(at + k) >= (unsigned)cap) {
-            atomicOr(err, DEV_ERR_CHECK);
-            return;
+    const int m = e - f;
+    bool sparse = false;
+    if (warp.cap) {
+        sparse = m < kP2wBoxTargets;
+        if (sparse && m > 0) {  // the sources of the 3 x 3 neighbourhood: a run of boxes a row
+            const int tx = b & (side - 1), ty = b >> level;
+            int64_t src = 0;
+            for (int y = max(ty - 1, 0); y <= min(ty + 1, side - 1); ++y)
+                src += (int64_t)sstart[y * side + min(tx + 1, side - 1) + 1] - sstart[y * side + max(tx - 1, 0)];
+            sparse = src < kP2wSources;
         }
-        tab[at + k] = make_int4(f + k * run, min(f + (k + 1) * run, e), b, 0);
+        p2p_append(warp, sparse ? (m + warp.most - 1) / warp.most : 0, f, e, b, err);
     }
+    p2p_append(cta, sparse ? 0 : (m + cta.most - 1) / cta.most, f, e, b, err);
 }
 
 __global__ void __launch_bounds__(kP2pThreads) fmm_p2p_kernel(P2pArgs a)
@@ -262,16 +297,17 @@ __global__ void __launch_bounds__(kP2pThreads) fmm_p2p_kernel(P2pArgs a)
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int side = 1 << a.level;
+    if (a.go) after_go();
     const int total = min(__ldg(a.nclaim), a.ntab);
+    if (total <= 0) return;  // the same for every CTA
     // thread 0 fetches the index of the CTA's next claim one claim ahead
-    int knext = a.each ? (int)blockIdx.x * a.each : tid == 0 ? atomicAdd(a.cursor, 1) : 0;
-    const int kend = a.each ? min(knext + a.each, total) : total;
+    int knext = a.share ? (int)blockIdx.x : tid == 0 ? atomicAdd(a.cursor, 1) : 0;
 
     for (;;) {
         if (tid == 0) {
             const int k = knext;
-            s_claim = k < kend ? __ldg(a.tab + k) : make_int4(-1, -1, 0, 0);
-            if (k < kend) knext = a.each ? k + 1 : atomicAdd(a.cursor, 1);
+            s_claim = k < total ? __ldg(a.tab + k) : make_int4(-1, -1, 0, 0);
+            if (k < total) knext = a.share ? k + (int)gridDim.x : atomicAdd(a.cursor, 1);
         }
         __syncthreads();
         const int4 cl = s_claim;
@@ -386,7 +422,7 @@ __global__ void __launch_bounds__(kP2pThreads) fmm_p2p_kernel(P2pArgs a)
         }
     }
     // the last CTA to finish returns the cursor slot to zero for its next use
-    if (tid == 0 && !a.each) {
+    if (tid == 0 && !a.share) {
         __threadfence();
         if (atomicAdd(a.cursor + 1, 1) == (int)gridDim.x - 1) {
             atomicExch(a.cursor, 0);
@@ -416,7 +452,7 @@ __device__ __forceinline__ void p2p_claim(const P2pArgs& a, int first, int m, in
     unsigned long long zx[NP], zy[NP], re[NP], im[NP];
     auto target = [&](int k) {  // index of the lane's target k (-1: none)
         const int t = kP2wLanes * k + tl;
-        const int j = t < m ? __ldg(a.tperm + first + t) : -1;
+        const int j = t < m ? a.tperm[first + t] : -1;
         return (unsigned)j < (unsigned)a.nz ? j : -1;
     };
 #pragma unroll
@@ -430,7 +466,7 @@ __device__ __forceinline__ void p2p_claim(const P2pArgs& a, int first, int m, in
                 if (kP2wLanes * (2 * p + h) + tl < m) atomicOr(a.err, DEV_ERR_CHECK);
                 continue;
             }
-            const double x = __ldg(a.z + 2 * (size_t)j), y = __ldg(a.z + 2 * (size_t)j + 1);
+            const double x = a.z[2 * (size_t)j], y = a.z[2 * (size_t)j + 1];
             long long X, Y;
             if (grid_fixed31(x, a.level, X) && grid_fixed31(y, a.level, Y) && (int)(X >> 31) == tx &&
                 (int)(Y >> 31) == ty) {
@@ -510,22 +546,23 @@ __device__ __forceinline__ void p2p_claim(const P2pArgs& a, int first, int m, in
     }
 }
 
+// Runs beside the CTA kernel of the same call, in the room that one leaves (nothing it reads is
+// written by that kernel).
 __global__ void __launch_bounds__(kP2pThreads, kP2wCtas) fmm_p2p_warp_kernel(P2pArgs a)
 {
     __shared__ float4 s_src[kP2pThreads / 32][2 * kP2wChunk];  // two staging buffers a warp
     const int lane = threadIdx.x & 31;
     float4* buf = s_src[threadIdx.x >> 5];
     const int side = 1 << a.level;
-    const int total = min(__ldg(a.nclaim), a.ntab);
+    const int total = min(*a.nclaim, a.ntab);
     // lane 0 fetches the index of the warp's next claim one claim ahead
-    const int warp = (int)blockIdx.x * (kP2pThreads / 32) + (threadIdx.x >> 5);
-    int knext = a.each ? warp * a.each : lane == 0 ? atomicAdd(a.cursor, 1) : 0;
-    const int kend = a.each ? min(knext + a.each, total) : total;
+    const int warp = (int)blockIdx.x * (kP2pThreads / 32) + (threadIdx.x >> 5), nwarp = (int)gridDim.x * (kP2pThreads / 32);
+    int knext = a.share ? warp : lane == 0 ? atomicAdd(a.cursor, 1) : 0;
     for (;;) {
         const int k = __shfl_sync(0xffffffffu, knext, 0);
-        if (k >= kend) break;
-        if (lane == 0) knext = a.each ? k + 1 : atomicAdd(a.cursor, 1);
-        const int4 cl = __ldg(a.tab + k);
+        if (k >= total) break;
+        if (lane == 0) knext = a.share ? k + nwarp : atomicAdd(a.cursor, 1);
+        const int4 cl = a.tab[k];
         const int first = cl.x, m = cl.y - cl.x, box = cl.z;
         const int tx = box & (side - 1), ty = box >> a.level;
         int b0 = 0, n = 0;
@@ -533,8 +570,8 @@ __global__ void __launch_bounds__(kP2pThreads, kP2wCtas) fmm_p2p_warp_kernel(P2p
             const int sx = tx + lane % 3 - 1, sy = ty + lane / 3 - 1;
             if (sx >= 0 && sy >= 0 && sx < side && sy < side) {
                 const int b = sy * side + sx;
-                b0 = __ldg(a.sstart + b);
-                n = __ldg(a.sstart + b + 1) - b0;
+                b0 = a.sstart[b];
+                n = a.sstart[b + 1] - b0;
                 if (n < 0 || b0 < 0 || b0 + n > a.n) {
                     atomicOr(a.err, DEV_ERR_CHECK);
                     b0 = n = 0;
@@ -549,17 +586,62 @@ __global__ void __launch_bounds__(kP2pThreads, kP2wCtas) fmm_p2p_warp_kernel(P2p
         }
     }
     // the last warp to finish returns the cursor slot to zero for its next use
-    if (lane == 0 && !a.each) {
+    if (lane == 0 && !a.share) {
         __threadfence();
         if (atomicAdd(a.cursor + 1, 1) == (int)gridDim.x * (kP2pThreads / 32) - 1) {
             atomicExch(a.cursor, 0);
             atomicExch(a.cursor + 1, 0);
         }
     }
+    after_wait();  // what follows in the stream waits for the CTA kernel too
 }
 
 // The sources in box order and the claim table of a call.
 static KeptBuffer g_p2p_buffer;
+
+// The claims of a table, at most `ctas` CTAs of them at one a CTA (warp); warp: by the warp kernel, else by
+// the CTA kernel, alone or (split) before the warp kernel.
+static int p2p_launch(bool warp, bool split, P2pArgs& a, const P2pTable& t, bool share, cudaStream_t st)
+{
+    auto kern = warp ? fmm_p2p_warp_kernel : fmm_p2p_kernel;
+    const int64_t ctas = warp ? ((int64_t)t.cap + kP2pThreads / 32 - 1) / (kP2pThreads / 32) : t.cap;
+    int sms = 0;
+    if (int rc = device_sm_count(&sms)) return rc;
+    a.go = split;
+    if (!warp && !split && ctas <= kP2pShareOne) share = true;
+    a.nclaim = t.nclaim;
+    a.tab = t.tab;
+    a.ntab = t.cap;
+    a.share = share;
+    a.cursor = nullptr;
+    int64_t grid = 0;
+    if (share) {
+        grid = split ? std::min<int64_t>(ctas, kP2pSplitGrid * sms)
+                     : (ctas <= kP2pShareOne ? ctas : std::min<int64_t>((ctas + 1) / 2, kP2pShareGrid));
+    } else {
+        if (int rc = tile_counter(&a.cursor, st)) return rc;
+        static int occ_cache[2];
+        static std::mutex mu;
+        int occ = 0;
+        {
+            std::lock_guard<std::mutex> lk(mu);
+            int& o = occ_cache[warp];
+            if (!o) {
+                FMM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, kern, kP2pThreads, 0));
+                if (o < 1) o = 1;
+            }
+            occ = o;
+        }
+        grid = std::min<int64_t>((int64_t)occ * sms, ctas);
+    }
+    if (warp) {
+        FMM_CUDA_TRY(launch_after(kern, (unsigned)grid, kP2pThreads, 0, st, a));
+    } else {
+        kern<<<(unsigned)grid, kP2pThreads, 0, st>>>(a);
+        FMM_CUDA_TRY(cudaGetLastError());
+    }
+    return FMM_OK;
+}
 
 }  // namespace fmmgb
 
@@ -595,55 +677,29 @@ extern "C" int fmm_p2p(int32_t level, const double* xy, const double* c, int64_t
     args.tperm = tgt_perm;
     args.tstart = tgt_start;
     args.phi = reinterpret_cast<float2*>(phi);
-    args.cursor = nullptr;
     if (int rc = device_error_word(&args.err)) return rc;
     const int nbox = 1 << (2 * level);
+    // every box to the CTA kernel, or the sparse ones to the warp kernel (the lines: above)
     const bool dense = nz >= (int64_t)kP2pDense * nbox || nbox < kP2wBoxes;
-    const int run = dense ? kP2pRun : kP2wRun;
-    // one buffer: the sources in box order, the claim table, the number of claims
-    const int64_t most = nz / run + std::min<int64_t>(nbox, nz);  // claims can be no more
+    // one buffer: the sources in box order, the claim tables, the numbers of claims
+    const int64_t boxes = std::min<int64_t>(nbox, nz);
+    P2pTable cta{kP2pRun, (int)(nz / kP2pRun + boxes)}, warp{kP2wRun, dense ? 0 : (int)(nz / kP2wRun + boxes)};  // claims can be no more
     float4* src = nullptr;
-    if (int rc = kept_buffer(g_p2p_buffer, (size_t)(n + most + 1) * sizeof(float4), (void**)&src)) return rc;
-    int4* tab = reinterpret_cast<int4*>(src + n);
-    int* nclaim = reinterpret_cast<int*>(tab + most);
-    args.nclaim = nclaim;
-    FMM_CUDA_TRY(cudaMemsetAsync(nclaim, 0, sizeof(int), st));
-    p2p_claim_table_kernel<<<(unsigned)((nbox + 255) / 256), 256, 0, st>>>(nbox, tgt_start, (int)nz, run, (int)most,
-                                                                          nclaim, tab, args.err);
+    if (int rc = kept_buffer(g_p2p_buffer, (size_t)(n + cta.cap + warp.cap + 1) * sizeof(float4), (void**)&src)) return rc;
+    cta.tab = reinterpret_cast<int4*>(src + n);
+    warp.tab = cta.tab + cta.cap;
+    cta.nclaim = reinterpret_cast<int*>(warp.tab + warp.cap);
+    warp.nclaim = cta.nclaim + 1;
+    FMM_CUDA_TRY(cudaMemsetAsync(cta.nclaim, 0, 2 * sizeof(int), st));
+    p2p_claim_table_kernel<<<(unsigned)((nbox + 255) / 256), 256, 0, st>>>(level, tgt_start, (int)nz, src_start, cta, warp,
+                                                                          args.err);
     FMM_CUDA_TRY(cudaGetLastError());
     if (n > 0) {
         p2p_sort_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(level, xy, c, src_perm, (int)n, src, args.err);
         FMM_CUDA_TRY(cudaGetLastError());
     }
     args.src = src;
-    args.tab = tab;
-    args.ntab = (int)most;
-    auto kern = dense ? fmm_p2p_kernel : fmm_p2p_warp_kernel;
-    const int64_t ctas = dense ? most : (most + kP2pThreads / 32 - 1) / (kP2pThreads / 32);
-    const bool share = (flags & FMM_P2P_SHARE_SM) || (dense && ctas <= kP2pShareOne);
-    int64_t grid = 0;
-    args.each = 0;
-    if (share) {
-        args.each = ctas <= kP2pShareOne ? 1 : (int)std::max<int64_t>(kP2pShareClaims, (ctas + kP2pShareGrid - 1) / kP2pShareGrid);
-        grid = (ctas + args.each - 1) / args.each;
-    } else {
-        if (int rc = tile_counter(&args.cursor, st)) return rc;
-        static int occ_cache[2];
-        static std::mutex mu;
-        int sms = 0, occ = 0;
-        if (int rc = device_sm_count(&sms)) return rc;
-        {
-            std::lock_guard<std::mutex> lk(mu);
-            int& o = occ_cache[dense];
-            if (!o) {
-                FMM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, kern, kP2pThreads, 0));
-                if (o < 1) o = 1;
-            }
-            occ = o;
-        }
-        grid = std::min<int64_t>((int64_t)occ * sms, ctas);
-    }
-    kern<<<(unsigned)grid, kP2pThreads, 0, st>>>(args);
-    FMM_CUDA_TRY(cudaGetLastError());
-    return FMM_OK;
+    const bool share = (flags & FMM_P2P_SHARE_SM) != 0;
+    if (int rc = p2p_launch(false, !dense, args, cta, share, st)) return rc;
+    return dense ? FMM_OK : p2p_launch(true, false, args, warp, share, st);
 }

@@ -307,6 +307,43 @@ def test_binning_at_the_edges_of_its_blocks(fmm, level, n):
     assert torch.equal(torch.sort(perm).values.long(), torch.arange(n, device="cuda"))
 
 
+@pytest.mark.parametrize("level", [7, 8])
+def test_p2p_crowded_boxes_among_sparse_ones(fmm, orc, level):
+    """A call whose sparse boxes go to the warp kernel and whose dense or crowded ones to the CTA kernel:
+    boxes of 1, 31, 32, 33, 97 and 500 targets, and few targets beside 1,023, 1,024 and 3,000 sources
+    (in the box, and in its neighbours), at corners and inside, every such target against the oracle;
+    the same bits with short-lived blocks."""
+    import torch
+
+    rng = np.random.default_rng(level)
+    side = 2 ** level
+    at = lambda bx, by, k: (np.array([bx, by]) + 0.02 + 0.96 * rng.random((k, 2))) / side
+    z, xy = [rng.random((side * side // 8, 2))], [rng.random((2000, 2))]
+    for i, m in enumerate((1, 31, 32, 33, 97, 500)):
+        z.append(at(4 * i, 0 if i % 2 else side - 1, m))
+        xy.append(at(4 * i, 0 if i % 2 else side - 1, 7))
+    for i, k in enumerate((1023, 1024, 3000)):
+        z.append(at(10 * i + 3, side // 2, 5))
+        xy.append(at(10 * i + 3 + i % 2, side // 2 + (i == 2), k))
+    z, xy = np.concatenate(z), np.concatenate(xy)
+    c = rng.uniform(-1, 1, len(xy))
+    zz = z[:, 0] + 1j * z[:, 1]
+    ref = orc.p2p_uniform(level, xy, c, zz)
+    zd, xyd, cd = (torch.from_numpy(v).cuda() for v in (z, xy, c))
+    (sp, ss), (tp, ts) = _bins(fmm, level, xyd), _bins(fmm, level, zd)
+    out = []
+    for share in (False, True):
+        phi = torch.full((len(z),), float("nan"), dtype=torch.complex64, device="cuda")
+        fmm.fmm_p2p(level, xyd, cd, sp, ss, zd, tp, ts, phi, share_sm=share)
+        fmm.fmm_sync_status()
+        out.append(phi)
+    assert torch.equal(torch.view_as_real(out[0]), torch.view_as_real(out[1]))
+    got = out[0].cpu().numpy().astype(np.complex128)
+    # the bars of the coarse levels, as for the other crowded boxes above
+    assert np.linalg.norm(got - ref) <= 1e-4 * np.linalg.norm(ref)
+    assert np.abs(got - ref).max() <= 2e-4 * np.abs(ref).max()
+
+
 def test_p2p_graph_keeps_its_buffer(fmm):
     """The per-device buffer grows inside a capture (more targets, then more sources, than any call
     before), and a graph captured before it grew replays what it did."""
