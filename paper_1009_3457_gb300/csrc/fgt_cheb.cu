@@ -410,20 +410,22 @@ __device__ __forceinline__ void binned_targets(const double* y, const int* perm,
         }
     }
 }
-// A warp takes 32 kRows consecutive binned targets: together where they share a box (uniform
-// 16-byte loads of its coefficients, each feeding 4 kRows multiply-adds a lane), else a row of
-// 32 at a time with a box per lane.
-constexpr int kRows = 4;
+// A warp takes 32 ROWS consecutive binned targets: together where they share a box (uniform
+// 16-byte loads of its coefficients, each feeding 4 ROWS multiply-adds a lane), else a row of
+// 32 at a time with a box per lane.  ROWS is 4, or 1 for fewer than kEvalWide targets, which leave the SMs
+// warps to spare (whole calls on 1 to 4^7 boxes, p = 8 and 16, n_cut = 0 to 10, one row against four: 0.73 of the
+// time for 2,000 targets, 0.85 for 10^5, 1.00 for 2*10^5, 1.13 for 3*10^5).
+constexpr int64_t kEvalWide = 1 << 17;
 
-template <int P, int Q>
+template <int P, int Q, int ROWS>
 __device__ __forceinline__ void cheb_eval_warp(const ChebEval& a, int64_t base)
 {
     const int lane = threadIdx.x & 31, side = 1 << a.g, nbox = side * side;
-    int tj[kRows], tb[kRows];  // target, its box (-1: evaluated apart)
-    float x1[kRows], x2[kRows], out[kRows];
-    binned_targets<kRows>(a.y, a.perm, a.box_start, a.g, a.n, base + lane, a.err, tj, tb, x1, x2);
+    int tj[ROWS], tb[ROWS];  // target, its box (-1: evaluated apart)
+    float x1[ROWS], x2[ROWS], out[ROWS];
+    binned_targets<ROWS>(a.y, a.perm, a.box_start, a.g, a.n, base + lane, a.err, tj, tb, x1, x2);
 #pragma unroll
-    for (int r = 0; r < kRows; ++r) {
+    for (int r = 0; r < ROWS; ++r) {
         x1[r] *= 2.f;
         x2[r] *= 2.f;
         out[r] = 0.f;
@@ -431,17 +433,17 @@ __device__ __forceinline__ void cheb_eval_warp(const ChebEval& a, int64_t base)
     const int b0 = __shfl_sync(0xffffffffu, tb[0], 0);
     bool same = b0 >= 0;
 #pragma unroll
-    for (int r = 0; r < kRows; ++r) same &= tb[r] == b0 || base + 32 * r + lane >= a.n;
+    for (int r = 0; r < ROWS; ++r) same &= tb[r] == b0 || base + 32 * r + lane >= a.n;
     if (__all_sync(0xffffffffu, same)) {
-        cheb_sum<Q, kRows>(a.C + (size_t)b0 * Q * Q, x1, x2, out);
+        cheb_sum<Q, ROWS>(a.C + (size_t)b0 * Q * Q, x1, x2, out);
     } else {
 #pragma unroll 1
-        for (int r = 0; r < kRows; ++r) {
+        for (int r = 0; r < ROWS; ++r) {
             // registers indexed by constants only
             float u1 = 0.f, u2 = 0.f, v = 0.f;
             int b = -1, j = -1;
 #pragma unroll
-            for (int k = 0; k < kRows; ++k)
+            for (int k = 0; k < ROWS; ++k)
                 if (k == r) {
                     u1 = x1[k];
                     u2 = x2[k];
@@ -468,7 +470,7 @@ __device__ __forceinline__ void cheb_eval_warp(const ChebEval& a, int64_t base)
                 if (lo >= 0) v = w;
             }
 #pragma unroll
-            for (int k = 0; k < kRows; ++k)
+            for (int k = 0; k < ROWS; ++k)
                 if (k == r) {
                     out[k] = v;
                     tj[k] = j;
@@ -476,7 +478,7 @@ __device__ __forceinline__ void cheb_eval_warp(const ChebEval& a, int64_t base)
         }
     }
 #pragma unroll
-    for (int r = 0; r < kRows; ++r)
+    for (int r = 0; r < ROWS; ++r)
         // NaN of a box that is summed directly: left to that sum
         if (tj[r] >= 0 && !(isnan(out[r]) && tb[r] >= 0 && a.apart[tb[r]])) a.G[tj[r]] = a.accumulate ? a.G[tj[r]] + out[r] : out[r];
 }
@@ -484,7 +486,7 @@ __device__ __forceinline__ void cheb_eval_warp(const ChebEval& a, int64_t base)
 // A CTA that has evaluated its own targets takes its share of the claims on the listed boxes, 128
 // targets each, one a thread.  (A launch of the direct kernel after this one cost 7 us more for an empty list,
 // and so did CTAs of their own before the others.)
-template <int P, int Q>
+template <int P, int Q, int ROWS>
 __global__ void __launch_bounds__(kEvalThreads) cheb_eval_kernel(ChebEval a)
 {
     __shared__ H2pShared<kEvalThreads> sh;
@@ -493,10 +495,10 @@ __global__ void __launch_bounds__(kEvalThreads) cheb_eval_kernel(ChebEval a)
     const int nbox = 1 << (2 * a.g);
     after_go();
     after_wait();
-    const int64_t base = ((int64_t)blockIdx.x * (kEvalThreads / 32) + (threadIdx.x >> 5)) * (32 * kRows);
+    const int64_t base = ((int64_t)blockIdx.x * (kEvalThreads / 32) + (threadIdx.x >> 5)) * (32 * ROWS);
     bin_check(a.box_start, nbox, a.n, a.err);
     const unsigned long long count = *a.list.count;
-    if (base < a.n) cheb_eval_warp<P, Q>(a, base);
+    if (base < a.n) cheb_eval_warp<P, Q, ROWS>(a, base);
     if (blockIdx.x >= (unsigned)count) return;
     h2p_offsets(sh, a);
     for (unsigned k = blockIdx.x; k < (unsigned)count; k += gridDim.x) {
@@ -563,10 +565,12 @@ static int cheb_launch(const H2pSums& e, float* ws, cudaStream_t st)
     a.list = l.list;
     int sms = 0;
     if (int rc = device_sm_count(&sms)) return rc;
+    const bool wide = a.n >= kEvalWide;
     // with few targets, CTAs enough for the listed boxes (a list of 800 boxes of 16 targets: 150 -> 70 us)
-    const unsigned blocks = std::max(bin_blocks(a.n, kEvalThreads * kRows, (int64_t)nbox, kEvalThreads),
+    const unsigned blocks = std::max(bin_blocks(a.n, kEvalThreads * (wide ? 4 : 1), (int64_t)nbox, kEvalThreads),
                                      (unsigned)std::min<size_t>(nbox, 2 * (size_t)sms));
-    FMM_CUDA_TRY(launch_after(cheb_eval_kernel<P, Q>, blocks, kEvalThreads, H2pSmem<P>::bytes, st, a));
+    auto eval = wide ? cheb_eval_kernel<P, Q, 4> : cheb_eval_kernel<P, Q, 1>;
+    FMM_CUDA_TRY(launch_after(eval, blocks, kEvalThreads, H2pSmem<P>::bytes, st, a));
     return FMM_OK;
 }
 
@@ -579,6 +583,7 @@ int launch_fgt_h2p_cheb(int g, int ncut, int p, double d, const float* A, const 
     if (int rc = cheb_workspace(g, &ws)) return rc;
     if (!ws) return FMM_OK;
     *done = true;
+    ncut = std::min(ncut, (1 << g) - 1);  // no more offsets than the grid has (1 box, n_cut = 10: 16.7 -> 11 us)
     const H2pSums e{g, ncut, n, d, A, y, perm, box_start, nullptr, G, accumulate ? 1 : 0, err};
     switch (p) {
         case 4: return cheb_launch<4>(e, ws, st);

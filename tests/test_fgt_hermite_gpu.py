@@ -449,6 +449,23 @@ def test_h2p_targets_outside_the_unit_square(fmm, orc, p, g, k):
                orc.fgt_hermite_eval_grid(g, ncut, p, sigma, A32.astype(np.float64), y))
 
 
+@pytest.mark.parametrize("p", [4, 16])
+@pytest.mark.parametrize("g,ncut,n", [(0, 0, 5), (0, 16, 5), (0, 16, 700), (1, 16, 9), (1, 2, 500), (2, 15, 800),
+                                      (3, 7, 2 ** 17 - 1), (3, 10, 2 ** 17)])
+def test_h2p_neighbourhoods_wider_than_the_grid(fmm, orc, p, g, ncut, n):
+    """n_cut beyond the grid's side (as many offsets as the grid has), and both sides of the line between one
+    and four targets a lane; 500 targets against the oracle."""
+    import math
+
+    rng = np.random.default_rng(10 * g + ncut)
+    sigma = 2.0 ** -g / (math.sqrt(2.0) * 0.45)
+    A32 = _decaying(rng, 4 ** g, p)
+    y = rng.random((n, 2))
+    pick = rng.choice(n, min(n, 500), replace=False)
+    _check(_h2p(fmm, g, ncut, p, sigma, A32, y)[pick],
+           orc.fgt_hermite_eval_grid(g, ncut, p, sigma, A32.astype(np.float64), y[pick]))
+
+
 def _per_target_terms(g, sigma, A, box, y):
     """Sum over one source box of |A_a1a2 h_a1(t1) h_a2(t2)| at each target, and t1^2 + t2^2, in 64 bits."""
     p, n = A.shape[-1], 1 << g
