@@ -629,11 +629,12 @@ int fgt_h2p(int32_t grid_log2, int32_t n_cut, int32_t p, int32_t prec, double si
  *   z: device float64 [nz][2] targets; tgt_perm, tgt_start:
  *   fmm_bin_points(level, z, nz, ...); phi: device complex64 [nz], indexed
  *   like z.  level 0..10, n and nz < 2^31.
- *   flags   FMM_ACCUMULATE; FMM_P2P_SHARE_SM: thread blocks that end after
- *           one or two runs of targets instead of staying to the end, so that kernels
- *           of a stream of higher priority find room on the SMs (the far
- *           field of the same FMM: 1.24 -> 1.16 ms for the whole potential at
- *           2^22 points).  The result is the same, bit for bit.
+ *   flags   FMM_ACCUMULATE; FMM_P2P_SHARE_SM: every thread block ends after
+ *           a few runs of targets, so that kernels of a stream of higher
+ *           priority find room on the SMs (the far field of the same FMM: 1.24 ->
+ *           1.16 ms for the whole potential at 2^22 points); without it only those
+ *           of calls with many sparse boxes stay to the end.  The result is
+ *           the same, bit for bit.
  *   FP32 arithmetic on positions taken relative to the target box's centre;
  *   1e-30 is added to every squared distance, so a source at exactly a
  *   target's position (e.g. the points themselves) contributes nothing

@@ -27,7 +27,7 @@
 // FP32 carries the difference of two nearby points to ~2^-24 of a box side.
 // A source at the target's position (the point itself, when targets are the
 // sources) contributes nothing: r^2 carries a 1e-30 offset and dx = dy = 0.
-#include <mutex>
+#include <algorithm>
 
 #include "fgt_hermite.cuh"
 
@@ -38,18 +38,24 @@ constexpr int kP2pWarps = kP2pThreads / 32;     // each takes a quarter of the s
 constexpr int kP2pR = 3;                        // targets per lane (rows of 32 targets per claim)
 constexpr int kP2pRun = 32 * kP2pR;             // targets per claim
 constexpr int kP2pBatch = 1024;                 // sources per shared-memory batch
-// With FMM_P2P_SHARE_SM a CTA (a warp of it in the warp kernel) ends after its share of the claims, one
-// or two, and kernels of
-// a stream of higher priority take its place; a persistent CTA would hold its registers to the end.  The
-// potential of 2^22 points with the far field beside it: 1,240 us with persistent CTAs (8 per SM), 1,167 /
-// 1,157 / 1,163 / 1,169 with 1 / 2 / 3 / 4 claims; the near field alone 923 us persistent, 925 with 2.  A warp a claim
-// loses more alone (2^22 points at level 9 689 -> 731), so that without the flag CTAs persist; but a few claims
-// go to a CTA each in any case: where some are heavy, one waits behind another in a persistent CTA,
-// and where two went to a CTA the SMs stood idle (us, persistent / two / one a CTA: 2^17 clustered points at level 6
-// 218 / 243 / 186, 2^15 at level 5 73 / 80 / 57, 2^15 uniform 24 / 24 / 22).
-constexpr int kP2pShareOne = 1 << 14;           // a CTA (warp) each for fewer claims
+// The CTA kernel's CTAs, and with FMM_P2P_SHARE_SM the warp kernel's, take one claim or a few each and
+// end: kernels of a stream of higher priority take their places, and no claim waits behind a heavy one
+// that a persistent CTA holds.  The potential of 2^22 points with the far field beside it: 1,240 us with
+// persistent CTAs (8 per SM), 1,167 / 1,157 / 1,163 / 1,169 with 1 / 2 / 3 / 4 claims; the near field alone, persistent
+// and so: 2^22 uniform points at level 8 939 and 915, 2^19 clustered at level 7 696 and 530, 2^17 at level 6 218 and
+// 181.  Where few, a CTA each: two a CTA left SMs idle (2^15 clustered points at level 5 80 us and 57).
+// A warp a claim loses alone (2^22 points at level 9 689 -> 731), so that without the flag the warp kernel
+// persists.
+constexpr int kP2pShareOne = 1 << 14;           // claims: a CTA (warp) each up to here, beyond it two
 constexpr int kP2pShareGrid = 1 << 16;          // more claims a CTA rather than more CTAs (most find none)
-constexpr int kP2pSplitGrid = 64;               // CTAs per SM of the CTA kernel beside the warp kernel
+// CTAs per SM of the CTA kernel beside the warp kernel: 16 / 32 / 64 for 2^20 clustered points at level 8 642 / 601 /
+// 566 us, for 2^18 uniform ones at level 7, which leave it nothing, 66 / 68 / 73 (64 before it).
+constexpr int kP2pSplitGrid = 32;
+// With the flag a call of few claims, or beside the warp kernel, leaves room on each SM: shared memory for 7
+// CTAs of the CTA kernel where registers allow 9, since among crowded boxes a claim lasts tens of
+// microseconds and the other stream's kernels wait for it (the whole potential of 2^17 clustered points at
+// level 6 263 -> 224 us, uniform 61 both; 2^22 uniform points lose, 1,106 -> 1,183).
+constexpr int kP2pRoomSmem = 12 << 10;
 // The warp kernel takes calls of fewer than kP2pDense targets a box on average, on kP2wBoxes boxes or
 // more (fewer claims than warps otherwise).  us, CTA / warp: 16 a box at level 5 26 / 35, level 6 31 / 35,
 // level 7 68 / 62, level 8 216 / 170, level 9 914 / 676; 32 a box at level 6 41 / 55, level 7 105 / 110,
@@ -89,8 +95,8 @@ struct P2pArgs {
     const int4* tab;    // claim table (p2p_claim_table_kernel), room for ntab entries
     int ntab;
     float2* phi;
-    int* cursor;  // [0] next claim index, [1] CTAs finished
-    int share;    // every CTA (warp) takes every gridDim-th place of the table and ends; no cursor
+    int* cursor;  // of the warp kernel: [0] next claim index, [1] warps finished; NULL: a warp takes every
+                  // (number of warps)-th place of the table and ends
     int go;       // the other kernel may start beside this one
     int* err;
 };
@@ -300,15 +306,8 @@ __global__ void __launch_bounds__(kP2pThreads) fmm_p2p_kernel(P2pArgs a)
     if (a.go) after_go();
     const int total = min(__ldg(a.nclaim), a.ntab);
     if (total <= 0) return;  // the same for every CTA
-    // thread 0 fetches the index of the CTA's next claim one claim ahead
-    int knext = a.share ? (int)blockIdx.x : tid == 0 ? atomicAdd(a.cursor, 1) : 0;
-
-    for (;;) {
-        if (tid == 0) {
-            const int k = knext;
-            s_claim = k < total ? __ldg(a.tab + k) : make_int4(-1, -1, 0, 0);
-            if (k < total) knext = a.share ? k + (int)gridDim.x : atomicAdd(a.cursor, 1);
-        }
+    for (int k = blockIdx.x;; k += gridDim.x) {
+        if (tid == 0) s_claim = k < total ? __ldg(a.tab + k) : make_int4(-1, -1, 0, 0);
         __syncthreads();
         const int4 cl = s_claim;
         const int first = cl.x, end = cl.y, box = cl.z;
@@ -419,14 +418,6 @@ __global__ void __launch_bounds__(kP2pThreads) fmm_p2p_kernel(P2pArgs a)
                 o.y += old.y;
             }
             a.phi[tj[r]] = o;
-        }
-    }
-    // the last CTA to finish returns the cursor slot to zero for its next use
-    if (tid == 0 && !a.share) {
-        __threadfence();
-        if (atomicAdd(a.cursor + 1, 1) == (int)gridDim.x - 1) {
-            atomicExch(a.cursor, 0);
-            atomicExch(a.cursor + 1, 0);
         }
     }
 }
@@ -557,11 +548,11 @@ __global__ void __launch_bounds__(kP2pThreads, kP2wCtas) fmm_p2p_warp_kernel(P2p
     const int total = min(*a.nclaim, a.ntab);
     // lane 0 fetches the index of the warp's next claim one claim ahead
     const int warp = (int)blockIdx.x * (kP2pThreads / 32) + (threadIdx.x >> 5), nwarp = (int)gridDim.x * (kP2pThreads / 32);
-    int knext = a.share ? warp : lane == 0 ? atomicAdd(a.cursor, 1) : 0;
+    int knext = !a.cursor ? warp : lane == 0 ? atomicAdd(a.cursor, 1) : 0;
     for (;;) {
         const int k = __shfl_sync(0xffffffffu, knext, 0);
         if (k >= total) break;
-        if (lane == 0) knext = a.share ? k + nwarp : atomicAdd(a.cursor, 1);
+        if (lane == 0) knext = !a.cursor ? k + nwarp : atomicAdd(a.cursor, 1);
         const int4 cl = a.tab[k];
         const int first = cl.x, m = cl.y - cl.x, box = cl.z;
         const int tx = box & (side - 1), ty = box >> a.level;
@@ -586,7 +577,7 @@ __global__ void __launch_bounds__(kP2pThreads, kP2wCtas) fmm_p2p_warp_kernel(P2p
         }
     }
     // the last warp to finish returns the cursor slot to zero for its next use
-    if (lane == 0 && !a.share) {
+    if (lane == 0 && a.cursor) {
         __threadfence();
         if (atomicAdd(a.cursor + 1, 1) == (int)gridDim.x * (kP2pThreads / 32) - 1) {
             atomicExch(a.cursor, 0);
@@ -599,8 +590,7 @@ __global__ void __launch_bounds__(kP2pThreads, kP2wCtas) fmm_p2p_warp_kernel(P2p
 // The sources in box order and the claim table of a call.
 static KeptBuffer g_p2p_buffer;
 
-// The claims of a table, at most `ctas` CTAs of them at one a CTA (warp); warp: by the warp kernel, else by
-// the CTA kernel, alone or (split) before the warp kernel.
+// The claims of table t, by the warp kernel or by the CTA kernel, alone or (split) before the warp kernel.
 static int p2p_launch(bool warp, bool split, P2pArgs& a, const P2pTable& t, bool share, cudaStream_t st)
 {
     auto kern = warp ? fmm_p2p_warp_kernel : fmm_p2p_kernel;
@@ -608,36 +598,29 @@ static int p2p_launch(bool warp, bool split, P2pArgs& a, const P2pTable& t, bool
     int sms = 0;
     if (int rc = device_sm_count(&sms)) return rc;
     a.go = split;
-    if (!warp && !split && ctas <= kP2pShareOne) share = true;
     a.nclaim = t.nclaim;
     a.tab = t.tab;
     a.ntab = t.cap;
-    a.share = share;
     a.cursor = nullptr;
     int64_t grid = 0;
-    if (share) {
-        grid = split ? std::min<int64_t>(ctas, kP2pSplitGrid * sms)
-                     : (ctas <= kP2pShareOne ? ctas : std::min<int64_t>((ctas + 1) / 2, kP2pShareGrid));
-    } else {
+    if (warp && !share) {
         if (int rc = tile_counter(&a.cursor, st)) return rc;
-        static int occ_cache[2];
-        static std::mutex mu;
-        int occ = 0;
-        {
-            std::lock_guard<std::mutex> lk(mu);
-            int& o = occ_cache[warp];
-            if (!o) {
-                FMM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, kern, kP2pThreads, 0));
-                if (o < 1) o = 1;
-            }
-            occ = o;
+        static int occ_cache;
+        int occ = __atomic_load_n(&occ_cache, __ATOMIC_ACQUIRE);
+        if (!occ) {
+            FMM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kP2pThreads, 0));
+            occ = std::max(occ, 1);
+            __atomic_store_n(&occ_cache, occ, __ATOMIC_RELEASE);
         }
         grid = std::min<int64_t>((int64_t)occ * sms, ctas);
+    } else {
+        grid = split ? std::min<int64_t>(ctas, kP2pSplitGrid * sms)
+                     : (ctas <= kP2pShareOne ? ctas : std::min<int64_t>((ctas + 1) / 2, kP2pShareGrid));
     }
     if (warp) {
         FMM_CUDA_TRY(launch_after(kern, (unsigned)grid, kP2pThreads, 0, st, a));
     } else {
-        kern<<<(unsigned)grid, kP2pThreads, 0, st>>>(a);
+        kern<<<(unsigned)grid, kP2pThreads, share && (split || ctas <= kP2pShareOne) ? kP2pRoomSmem : 0, st>>>(a);
         FMM_CUDA_TRY(cudaGetLastError());
     }
     return FMM_OK;
