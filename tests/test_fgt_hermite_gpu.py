@@ -2,6 +2,11 @@
 the device binning of points by box (fgt_bin_points) and the binned P2H
 (fgt_p2h_binned), against the FP64 oracle.
 
+fgt_h2p has three forms: through Chebyshev coefficients of each target box (from 2 targets a box on
+average, box sides of up to sqrt2 sigma / 2), and the direct sums on the CUDA cores and on the tensor
+cores.  The grid of a sigma (workloads.fgt_grid_log2) has box sides of 0.25 to 0.5 sqrt2 sigma; the
+tests of the direct kernels take the next coarser one, which the first form leaves to them.
+
 Bars: binning is exact (the same box for every point, every point once);
 G relative L2 over all targets <= 1e-5 (FP32) against the oracle evaluating
 the same FP32 coefficients in FP64, and every target's error <= 1e-5 of
@@ -156,13 +161,14 @@ def test_p2h_binned_matches_oracle(fmm, orc, gmm_sources, p):
         assert np.linalg.norm(got2 - 2 * ref) / np.linalg.norm(2 * ref) <= 1e-5
 
 
+@pytest.mark.parametrize("coarser", [0, 1])
 @pytest.mark.parametrize("p", [4, 8, 12, 16])
 @pytest.mark.parametrize("sigma,ncut", [(0.2, 10), (0.1, 3), (0.05, 1), (0.1, 0)])
-def test_h2p_matches_oracle(fmm, orc, gmm_sources, p, sigma, ncut):
+def test_h2p_matches_oracle(fmm, orc, gmm_sources, p, sigma, ncut, coarser):
     """Targets: uniform (many in boxes with no sources) plus a cluster of 700 in one
-    box (several claims of one box, a ragged last one)."""
+    box (coarser: several claims of one box by the direct kernel, a ragged last one)."""
     x, q = gmm_sources
-    g = workloads.fgt_grid_log2(sigma)
+    g = workloads.fgt_grid_log2(sigma) - coarser
     rng = np.random.default_rng(p * 100 + ncut)
     y = np.concatenate([rng.random((2500, 2)), 0.52 + 0.001 * rng.random((700, 2))])
     A32 = orc.fgt_p2h_grid(g, p, sigma, x, q).astype(np.float32)
@@ -199,7 +205,7 @@ def test_h2p_claim_order_grids(fmm, orc, g):
     rng = np.random.default_rng(300 + g)
     p, ncut = 8, 3
     n = 1 << g
-    sigma = 2.0 ** -g / (math.sqrt(2.0) * 0.442)
+    sigma = 2.0 ** -g / (math.sqrt(2.0) * 0.6)  # boxes that the direct kernel takes
     fact = np.array([math.factorial(a) for a in range(p)], float)
     A = rng.standard_normal((n * n, p, p)) * (0.3 ** (np.arange(p)[:, None] + np.arange(p)[None, :])) / np.outer(fact, fact)
     empty = rng.random(n * n) < 0.33
@@ -259,17 +265,18 @@ def test_hermite_transform_on_device_matches_direct_sum(fmm, orc, sigma, p):
     assert np.linalg.norm(got - direct) / np.linalg.norm(direct) <= 1e-5
 
 
-@pytest.mark.parametrize("sigma,p", [(0.05, 16), (0.2, 8)])
-def test_h2p_full_size_workload_sampled(fmm, orc, sigma, p):
+@pytest.mark.parametrize("sigma,p,coarser", [(0.05, 16, 0), (0.2, 8, 0), (0.05, 16, 1), (0.2, 8, 1)])
+def test_h2p_full_size_workload_sampled(fmm, orc, sigma, p, coarser):
     """2^20 Gaussian-mixture sources and 2^20 targets from the same mixture (n_cut = 10),
-    the launch the benchmark times; 1,500 sampled targets against the oracle."""
+    the launch the benchmark times, and (coarser) one of the direct kernel; 1,500 sampled targets
+    against the oracle."""
     import torch
 
     n = 1 << 20
     rng = np.random.default_rng(2024)
     x, q = workloads.gmm_particles(n, rng)
     y, _ = workloads.gmm_particles(n, np.random.default_rng(2025))
-    g = workloads.fgt_grid_log2(sigma)
+    g = workloads.fgt_grid_log2(sigma) - coarser
     xd, yd = torch.from_numpy(x).cuda(), torch.from_numpy(y).cuda()
     perm, _ = _bin(fmm, g, xd)
     A = torch.empty((4 ** g, p, p), dtype=torch.float32, device="cuda")
@@ -312,11 +319,14 @@ def _rel(got, ref):
     return np.linalg.norm(got - ref) / np.linalg.norm(ref)
 
 
+@pytest.mark.parametrize("coarser", [0, 1])
 @pytest.mark.parametrize("name", ["bf16x3", "bf16"])
 @pytest.mark.parametrize("sigma,ncut", [(0.2, 10), (0.1, 10), (0.05, 10), (0.1, 3), (0.05, 1), (0.1, 0), (0.05, 15)])
-def test_h2p_tc_matches_oracle(fmm, orc, gmm_sources, name, sigma, ncut):
+def test_h2p_tc_matches_oracle(fmm, orc, gmm_sources, name, sigma, ncut, coarser):
+    """A tensor-core precision: served in FP32 through the coefficients, and (coarser) by the tensor-core
+    kernel, the cluster in several claims of 128 targets; there it differs from the FP32 sums."""
     x, q = gmm_sources
-    g = workloads.fgt_grid_log2(sigma)
+    g = workloads.fgt_grid_log2(sigma) - coarser
     rng = np.random.default_rng(ncut + int(sigma * 100))
     y = np.concatenate([rng.random((2500, 2)), 0.52 + 0.001 * rng.random((700, 2))])
     A32 = orc.fgt_p2h_grid(g, 16, sigma, x, q).astype(np.float32)
@@ -327,6 +337,10 @@ def test_h2p_tc_matches_oracle(fmm, orc, gmm_sources, name, sigma, ncut):
     err = _rel(got, ref)
     assert err <= trunc + TC_BAR[name], f"relative L2 {err:.3e}"
     assert np.abs(got - ref).max() <= 10 * TC_BAR[name] * np.abs(ref).max()
+    fp32 = _h2p_tc(fmm, g, ncut, sigma, A32, y, fmm.FMM_FP32)
+    assert np.array_equal(got, fp32) == (not coarser)
+    if coarser and name == "bf16":  # one product of operands rounded to 8 bits: not the split form either
+        assert err >= 1e-4
 
 
 def test_h2p_tc_ragged_counts_and_accumulate(fmm, orc, gmm_sources):
@@ -346,15 +360,16 @@ def test_h2p_tc_ragged_counts_and_accumulate(fmm, orc, gmm_sources):
 
 
 def test_h2p_tc_agrees_with_fp32_path_at_full_size(fmm, orc):
-    """2^20 mixture targets, sigma 0.05, n_cut 10 (the benchmark's launch): the tensor-core
-    result against the FP32 path everywhere and the oracle on 1,500 sampled targets."""
+    """2^20 mixture targets, sigma 0.05, n_cut 10, on 16 x 16 boxes (wide ones, which the direct kernels
+    take): the tensor-core result against the FP32 kernel's everywhere and the oracle on 1,500 sampled
+    targets, accumulated too."""
     import torch
 
     n = 1 << 20
     x, q = workloads.gmm_particles(n, np.random.default_rng(2024))
     y, _ = workloads.gmm_particles(n, np.random.default_rng(2025))
     sigma, ncut = 0.05, workloads.FGT_NCUT
-    g = workloads.fgt_grid_log2(sigma)
+    g = workloads.fgt_grid_log2(sigma) - 1
     xd, yd = torch.from_numpy(x).cuda(), torch.from_numpy(y).cuda()
     perm, _ = _bin(fmm, g, xd)
     A = torch.empty((4 ** g, 16, 16), dtype=torch.float32, device="cuda")
@@ -366,10 +381,13 @@ def test_h2p_tc_agrees_with_fp32_path_at_full_size(fmm, orc):
     fmm.fgt_h2p(g, ncut, 16, sigma, A, yd, tperm, tstart, Gtc, prec=fmm.FMM_TC_BF16X3)
     fmm.fmm_sync_status()
     g32, gtc = G32.cpu().numpy().astype(np.float64), Gtc.cpu().numpy().astype(np.float64)
-    assert _rel(gtc, g32) <= 1e-4
+    assert 0.0 < _rel(gtc, g32) <= 1e-4
     pick = np.random.default_rng(6).choice(n, 1500, replace=False)
     ref = orc.fgt_hermite_eval_grid(g, ncut, 16, sigma, A.cpu().numpy().astype(np.float64), y[pick])
     assert _rel(gtc[pick], ref) <= 1e-4
+    fmm.fgt_h2p(g, ncut, 16, sigma, A, yd, tperm, tstart, Gtc, prec=fmm.FMM_TC_BF16X3, accumulate=True)
+    fmm.fmm_sync_status()
+    assert _rel(Gtc.cpu().numpy().astype(np.float64), 2 * gtc) <= 1e-6
 
 
 # ---------------------------------------------------------------------------

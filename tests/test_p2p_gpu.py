@@ -293,8 +293,8 @@ def test_p2p_short_lived_blocks_equal_persistent_ones(fmm, level, per_box):
 @pytest.mark.parametrize("level", [0, 3, 7])
 @pytest.mark.parametrize("n", [1, 257, 32767, 32768, 4097 * 304, 1_300_001])
 def test_binning_at_the_edges_of_its_blocks(fmm, level, n):
-    """Both block widths, chunks of every length up to four points a thread and more blocks than
-    that: the boxes' counts, and every point once in its own box."""
+    """The three block shapes (256 threads x 4 points, 512 x 8, 1024 x 4), chunks shorter than a block's
+    points and longer: the boxes' counts, and every point once in its own box."""
     import torch
 
     g = torch.Generator(device="cuda").manual_seed(n)
