@@ -574,15 +574,18 @@ int fgt_t2p_binned(int32_t grid_log2, int32_t p, double sigma, const float* C, c
  *   y, n, ...) of these targets; G: device float32 [n], indexed like y.
  *   n_cut 0..16, p 4, 8, 12 or 16, flags FMM_ACCUMULATE or 0.
  *   With two targets per box or more on average, grid_log2 <= 8 and a box side d =
- *   2^-g / (sqrt2 sigma) of up to 1/2, every prec is served in FP32 on
- *   the CUDA cores through Chebyshev coefficients of each target box (12 per dimension,
- *   interpolation error below 4e-10 of a Hermite function's largest value): the sums over
- *   source boxes are taken once per target box.  Targets outside the unit square, and
- *   boxes over which the field falls by more than e^5 (sources far away only), are summed
- *   directly in the same call, so that each value keeps its own FP32 accuracy.  The workspace, 1.4 KiB per box, is allocated
- *   per grid size and device on the first such call, in a stream capture or not, and kept
- *   (where there is no room for it the call takes the direct sums below, as every other call does).  Calls that
- *   overlap on the GPU share the workspace and must be serialised by the caller.
+ *   2^-g / (sqrt2 sigma) of up to 1/2, every prec is served in FP32 on the CUDA cores
+ *   through Chebyshev coefficients of each target box (12 per dimension): the sums over
+ *   source boxes are taken once per target box.  So FMM_TC_BF16 has an error of about
+ *   2e-7 or of about 1e-3 according to the number of targets, FMM_TC_BF16X3 2e-7 or
+ *   4e-6.  The interpolation adds at most 4e-10 of a Hermite function's largest value;
+ *   targets outside the unit square, and boxes over which the field falls by more
+ *   than e^5 (sources far away only), are summed directly in the same call, so that
+ *   each target's error stays relative to the terms of its own sum, as in the direct
+ *   forms.  The workspace, 1.4 KiB per box, is allocated per grid size and device on
+ *   the first such call, in a stream capture or not, and kept (where there is no room
+ *   for it the call takes the direct sums below, as every other call does).  Calls
+ *   that overlap on the GPU share the workspace and must be serialised by the caller.
  *   prec FMM_FP32: CUDA cores.  Source boxes whose coefficients are all zero
  *   are skipped: a first kernel writes one flag per box.  The targets are
  *   taken in runs of up to 256 of one box, the boxes with the most non-empty

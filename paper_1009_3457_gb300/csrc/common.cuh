@@ -101,7 +101,7 @@ __device__ __forceinline__ float pow2_neg(int k) { return __int_as_float((127 - 
 // that one ends, with it as soon as all of that one's CTAs have started: only the short kernels of the
 // FGT and of the binning call it, since CTAs that wait hold their registers (in the whole FMM, where
 // the far field runs beside the near field, calling it in the M2L and shift kernels cost 2 %).
-// Measured: M2L levels 2-8 at p = 16, back to back, 29.8 -> 27.4 us; the Taylor transform of 2^20 points
+// Measured: M2L levels 2-8 at p = 16, back to back, 29.8 -> 27.2 us; the Taylor transform of 2^20 points
 // (13 launches) 160 -> 151 us; the Hermite one of 3e5 92 -> 84 us.
 __device__ __forceinline__ void after_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void after_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

@@ -215,8 +215,11 @@ constexpr int kBinSmemMaxLog2 = 7;
 // turn left a thread waiting for each point's load).  fgt_bin_points takes
 //   - 1024 x 4 on grids of 4^6 boxes or more and 2^15 points or more: a histogram of 16 to 64 KB
 //     leaves room for few blocks, which then need their threads (2^20 points on 4^7 boxes 49 -> 33 us, 37
-//     with 512 threads; 2^18 on 4^6 20.5 -> 16.4);
-//   - 512 x 8 on smaller grids and 2^19 points or more (2^20 on 4^5 27 -> 22.5 us; 1024 threads 21, but
+//     with 512 threads; 2^18 on 4^6 20.5 -> 16.4).  A block scatters 4,096 points at most and walks its counters
+//     for them; two passes over the block's whole share of the points are still slower (2^22 / 2^24 / 2^26 points on
+//     4^7 boxes 93 -> 73, 490 -> 248, 3,258 -> 909 us, on 4^6 66 -> 57, 464 -> 198, 2,668 -> 737);
+//   - 512 x 8 on smaller grids and 2^19 points or more (on 4^5 boxes 2^18.5 / 2^19 / 2^19.5 points 20.9 / 23.0 / 26.8
+//     -> 19.4 / 19.0 / 20.5 us, the first by 256 x 4; 2^20 27 -> 22.5; 1024 threads 21, but
 //     they fill the SMs, and the next kernel's early part, the table of the Hermite evaluation, then waits:
 //     163 against 153 us for that transform);
 //   - 256 x 4 else: few blocks start and meet sooner (2^12 points 8.4 us against 9.6 with 1024

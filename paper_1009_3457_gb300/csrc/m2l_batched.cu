@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(kBatchThreads, kBatchMinCtas)
     }
 }
 
-// the kernel of variant v (kBatchVariants order)
+// the kernel of variant v (kBatchLoads order)
 static const void* batch_kernel(int v)
 {
     return v == 1 ? (const void*)m2l_batched_kernel<2> : (const void*)m2l_batched_kernel<3>;

@@ -37,7 +37,7 @@
 // 54 p^2 packed multiply-adds: 3.6x fewer cycles of the FP32 pipe at p = 16 (3.0x
 // at p = 8, 4.0x at p = 24).  Levels 2-8 of a 2^22-point tree (87,376 boxes):
 // p = 16 79.9 -> 27.2 us back to back, where the pipe's own time for this count is
-// 16.6 us (61 % of it; 68 % at level 10, 391 us, where the launch, the first tile and
+// 16.6 us (61 % of it; 68 % for levels 2-10, 391 us, where the launch, the first tile and
 // the last wave weigh less).  The rest is latency: 16 warps an SM, with the short
 // addition chains of the combinations between the multiply-adds.  The error
 // against 64 bits falls as well (2.9e-7 -> 1.6e-7): fewer terms are summed.
@@ -89,8 +89,8 @@ struct M2LCfg {
     static constexpr bool SOLO = THREADS == 64;
     static constexpr int PART2 = SOLO ? HALO : PART;  // where the second partial sum lies
     static constexpr int BUF = SOLO ? HALO + PART : (HALO > 2 * PART ? HALO : 2 * PART);  // the sums reuse the halo's room
-    // resident CTAs (registers): levels 2-8 at p = 16 take 31.7 / 31.1 / 33.5 us with 3 / 4 / 5 CTAs
-    // of 128, p = 24 60.7 / 74.8 (spills) with 3 / 4, p = 12 24.4 / 23.8 / 23.2 with 3 / 4 / 5
+    // resident CTAs (registers): levels 2-8 at p = 16 take 31.7 / 31.1 / 33.5 us as ordinary launches (4: 27.2
+    // as a dependent one) with 3 / 4 / 5 CTAs of 128, p = 24 60.7 / 74.8 (spills) with 3 / 4, p = 12 24.4 / 23.8 / 23.2 with 3 / 4 / 5
     static constexpr int MIN_CTAS = (P <= 12 ? 5 : (P <= 16 ? 4 : 3)) * 128 / NT;
     // halo loads a thread keeps in flight while staging a tile
     static constexpr int LOADS = P <= 6 ? 2 : (P <= 8 ? 3 : 4);
@@ -538,11 +538,10 @@ __device__ __forceinline__ void m2l_tile(unsigned char* raw, const TileGeom& g, 
 // ---------------------------------------------------------------------------
 // stencil kernel: every requested level in one launch, tiles ordered heaviest
 // level first.  Persistent when `counter` is set: each resident CTA loads the
-// operator once, takes its first tile by blockIdx and claims the next from the
-// work counter (counter[0]; counter[1] counts the CTAs that finished, and the
-// last one resets both), so the operator table is staged once per CTA instead
-// of once per tile and no second round of CTAs leaves SMs half empty at the
-// end.  With counter == NULL the grid covers every tile, one CTA each.
+// diagonal scalings once (the operator lies in constant memory), takes its first
+// tile by blockIdx and claims the next from the work counter (counter[0];
+// counter[1] counts the CTAs that finished, and the last one resets both), so
+// no second round of CTAs leaves SMs half empty at the end.  With counter == NULL the grid covers every tile, one CTA each.
 // ---------------------------------------------------------------------------
 template <int P, bool ADAPTIVE>
 __global__ void __launch_bounds__(M2LCfg<P>::THREADS, M2LCfg<P>::MIN_CTAS)

@@ -83,14 +83,10 @@ constexpr float kP2pTiny = 1e-30f;
 
 struct P2pArgs {
     int level, n, nz, accumulate;
-    const double* xy;
-    const double* c;
     const float4* src;  // sources in box order: x, y relative to their own box's centre, c (p2p_sort_kernel)
-    const int* sperm;
     const int* sstart;
     const double* z;
     const int* tperm;
-    const int* tstart;
     const int* nclaim;  // claims in the table
     const int4* tab;    // claim table (p2p_claim_table_kernel), room for ntab entries
     int ntab;
@@ -652,13 +648,9 @@ extern "C" int fmm_p2p(int32_t level, const double* xy, const double* c, int64_t
     args.n = (int)n;
     args.nz = (int)nz;
     args.accumulate = (flags & FMM_ACCUMULATE) ? 1 : 0;
-    args.xy = xy;
-    args.c = c;
-    args.sperm = src_perm;
     args.sstart = src_start;
     args.z = z;
     args.tperm = tgt_perm;
-    args.tstart = tgt_start;
     args.phi = reinterpret_cast<float2*>(phi);
     if (int rc = device_error_word(&args.err)) return rc;
     const int nbox = 1 << (2 * level);
