@@ -48,9 +48,9 @@ constexpr int kP2pBatch = 1024;                 // sources per shared-memory bat
 // persists.
 constexpr int kP2pShareOne = 1 << 14;           // claims: a CTA (warp) each up to here, beyond it two
 constexpr int kP2pShareGrid = 1 << 16;          // more claims a CTA rather than more CTAs (most find none)
-// CTAs per SM of the CTA kernel beside the warp kernel: 16 / 32 / 64 for 2^20 clustered points at level 8 642 / 601 /
+// CTAs per SM of the CTA kernel beside the warp kernel (four times the resident ones): 16 / 32 / 64 for 2^20 clustered points at level 8 642 / 601 /
 // 566 us, for 2^18 uniform ones at level 7, which leave it nothing, 66 / 68 / 73 (64 before it).
-constexpr int kP2pSplitGrid = 32;
+constexpr int kP2pSplitGrid = 36;
 // With the flag a call of few claims, or beside the warp kernel, leaves room on each SM: shared memory for 7
 // CTAs of the CTA kernel where registers allow 9, since among crowded boxes a claim lasts tens of
 // microseconds and the other stream's kernels wait for it (the whole potential of 2^17 clustered points at
@@ -223,13 +223,15 @@ __device__ __forceinline__ void p2p_batch(const float4* __restrict__ s_src, int 
 }
 
 // Claim table: one entry (first, end, box) per run of targets of one box, a box's targets cut
-// into equal runs of at most `most`.  The runs of a warp's 32 boxes take consecutive places
+// into runs of at most `most`, alike in whole rows of `row` targets (runs alike in targets leave every
+// run's last row half empty: 320 targets in 12 rows of 32 instead of 10; 2^22 points in a band of 1/20 of the square at
+// level 9 3,834 -> 3,437 us).  The runs of a warp's 32 boxes take consecutive places
 // from one addition to *nclaim (zero before); the order of the table only sets the order in
 // which claims are taken.  Places past `cap`, or a box_start that does not bin [0, nz), set the
 // error word (and those runs are skipped).  (A scan of the boxes' counts by one block, to give every
 // run a place of its own, took 73 us at 256 x 256 boxes and 290 us at 512 x 512.)
 struct P2pTable {
-    int most, cap;
+    int row, most, cap;
     int* nclaim;
     int4* tab;
 };
@@ -248,13 +250,13 @@ __device__ __forceinline__ void p2p_append(const P2pTable& t, int n, int f, int 
     if (lane == 31 && x > 0) at = atomicAdd(t.nclaim, x);
     at = __shfl_sync(0xffffffffu, at, 31) + x - n;
     if (n <= 0) return;
-    const int run = (e - f + n - 1) / n;
+    const int64_t rows = (e - f + t.row - 1) / t.row;
     for (int k = 0; k < n; ++k) {
         if ((unsigned)(at + k) >= (unsigned)t.cap) {
             atomicOr(err, DEV_ERR_CHECK);
             return;
         }
-        t.tab[at + k] = make_int4(f + k * run, min(f + (k + 1) * run, e), b, 0);
+        t.tab[at + k] = make_int4(f + t.row * (int)(k * rows / n), min(f + t.row * (int)((k + 1) * rows / n), e), b, 0);
     }
 }
 
@@ -536,7 +538,7 @@ __device__ __forceinline__ void p2p_claim(const P2pArgs& a, int first, int m, in
 
 // Runs beside the CTA kernel of the same call, in the room that one leaves (nothing it reads is
 // written by that kernel).
-__global__ void __launch_bounds__(kP2pThreads, kP2wCtas) fmm_p2p_warp_kernel(P2pArgs a)
+__global__ void __launch_bounds__(kP2pThreads, kP2wCtas) fmm_p2p_warp_kernel(const __grid_constant__ P2pArgs a)
 {
     __shared__ float4 s_src[kP2pThreads / 32][2 * kP2wChunk];  // two staging buffers a warp
     const int lane = threadIdx.x & 31;
@@ -659,7 +661,8 @@ extern "C" int fmm_p2p(int32_t level, const double* xy, const double* c, int64_t
     const bool dense = nz >= (int64_t)kP2pDense * nbox || nbox < kP2wBoxes;
     // one buffer: the sources in box order, the claim tables, the numbers of claims
     const int64_t boxes = std::min<int64_t>(nbox, nz);
-    P2pTable cta{kP2pRun, (int)(nz / kP2pRun + boxes)}, warp{kP2wRun, dense ? 0 : (int)(nz / kP2wRun + boxes)};  // claims can be no more
+    // claims can be no more than the rooms of the tables
+    P2pTable cta{32, kP2pRun, (int)(nz / kP2pRun + boxes)}, warp{2 * kP2wLanes, kP2wRun, dense ? 0 : (int)(nz / kP2wRun + boxes)};
     float4* src = nullptr;
     if (int rc = kept_buffer(g_p2p_buffer, (size_t)(n + cta.cap + warp.cap + 1) * sizeof(float4), (void**)&src)) return rc;
     cta.tab = reinterpret_cast<int4*>(src + n);

@@ -310,7 +310,7 @@ def test_binning_at_the_edges_of_its_blocks(fmm, level, n):
 @pytest.mark.parametrize("level", [7, 8])
 def test_p2p_crowded_boxes_among_sparse_ones(fmm, orc, level):
     """A call whose sparse boxes go to the warp kernel and whose dense or crowded ones to the CTA kernel:
-    boxes of 1, 31, 32, 33, 97 and 500 targets, and few targets beside 1,023, 1,024 and 3,000 sources
+    boxes of 1, 31, 32, 33, 97, 320 and 500 targets (one run, and runs of several row counts), and few targets beside 1,023, 1,024 and 3,000 sources
     (in the box, and in its neighbours), at corners and inside, every such target against the oracle;
     the same bits with short-lived blocks."""
     import torch
@@ -319,7 +319,7 @@ def test_p2p_crowded_boxes_among_sparse_ones(fmm, orc, level):
     side = 2 ** level
     at = lambda bx, by, k: (np.array([bx, by]) + 0.02 + 0.96 * rng.random((k, 2))) / side
     z, xy = [rng.random((side * side // 8, 2))], [rng.random((2000, 2))]
-    for i, m in enumerate((1, 31, 32, 33, 97, 500)):
+    for i, m in enumerate((1, 31, 32, 33, 97, 320, 500)):
         z.append(at(4 * i, 0 if i % 2 else side - 1, m))
         xy.append(at(4 * i, 0 if i % 2 else side - 1, 7))
     for i, k in enumerate((1023, 1024, 3000)):
