@@ -567,7 +567,8 @@ static int cheb_launch(const H2pSums& e, float* ws, cudaStream_t st)
     int sms = 0;
     if (int rc = device_sm_count(&sms)) return rc;
     const bool wide = a.n >= kEvalWide;
-    // with few targets, CTAs enough for the listed boxes (a list of 800 boxes of 16 targets: 150 -> 70 us)
+    // with few targets, CTAs enough for the listed boxes (2^14 uniform targets
+    // on 32 x 32 boxes, all sources in a spot of 2 % of the side, d = 0.44: 150 -> 63 us)
     const unsigned blocks = std::max(bin_blocks(a.n, kEvalThreads * (wide ? 4 : 1), (int64_t)nbox, kEvalThreads),
                                      (unsigned)std::min<size_t>(nbox, 2 * (size_t)sms));
     auto eval = wide ? cheb_eval_kernel<P, Q, 4> : cheb_eval_kernel<P, Q, 1>;

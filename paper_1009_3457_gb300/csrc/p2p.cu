@@ -63,8 +63,8 @@ constexpr int kP2pRoomSmem = 12 << 10;
 constexpr int kP2pDense = 32, kP2wBoxes = 1 << 14;
 // And of such a call only the boxes with fewer than kP2wBoxTargets targets and kP2wSources sources around
 // them; the others go to the CTA kernel, beside it.  (All boxes to the warp kernel left its warps waiting
-// for the crowded ones; us, before the warp kernel / that / so, Gaussian mixtures: 2^18 points at level 7 250 / 450 / 243,
-// at level 8 153 / 213 / 97, 2^20 at level 8 709 / 1,004 / 670, at level 9 501 / 430 / 260.  32 / 48 / 64 targets
+// for the crowded ones; us, before the warp kernel / that / so, Gaussian mixtures: 2^18 points at level 7 250 / 450 / 200,
+// at level 8 153 / 213 / 87, 2^20 at level 8 709 / 1,004 / 550, at level 9 501 / 430 / 255.  32 / 48 / 64 targets
 // with ordinary launches: 264 / 275 / 302, 133 / 143 / 172, 682 / 706 / 743, 319 / 341 / 418; 512 to 2,048 sources
 // measured alike.)
 constexpr int kP2wBoxTargets = 32, kP2wSources = 1024;
