@@ -61,9 +61,11 @@ static int t2p_p(int g, double sigma, const float* C, int64_t n, const double* y
 // scattered results.
 // Fewer than kT2pWide targets leave the SMs warps to spare: one target a lane, since four rows
 // one after the other are four times the latency (p = 16, 32 x 32 boxes, us, one / four: 300 targets 7.0 / 16.7,
-// 10^4 4.7 / 12.3, 2*10^5 9.5 / 11.3, 3*10^5 14.1 / 12.0, 2^20 38 / 26).
+// 10^4 4.7 / 12.3, 2*10^5 9.5 / 11.3, 3*10^5 14.1 / 12.0, 2^20 38 / 26).  Fewer than kT2pSplit: four lanes a
+// target, a quarter of its coefficients' rows each (1 to 4^10 boxes, all p, four lanes against one: 0.8 of the time for 30 to
+// 3,000 targets, 0.90 for 10^4, 0.97 for 2*10^4, 1.06 for 3*10^4).
 constexpr int kT2pThreads = 128;
-constexpr int64_t kT2pWide = 1 << 18;
+constexpr int64_t kT2pWide = 1 << 18, kT2pSplit = 1 << 14;
 
 template <bool VEC>
 __device__ __forceinline__ float4 t2p_load4(const float* c)
@@ -72,14 +74,14 @@ __device__ __forceinline__ float4 t2p_load4(const float* c)
     return make_float4(c[0], c[1], c[2], c[3]);
 }
 
-// sum_{b1,b2} c[b1][b2] t1^b1 t2^b2 by Horner's rule, NR targets of one box (NR = 1: a box per lane)
-template <int P, int NR, bool VEC>
+// sum_{b1 < B, b2 < P} c[b1][b2] t1^b1 t2^b2 by Horner's rule, NR targets of one box (NR = 1: a box per lane)
+template <int P, int B, int NR, bool VEC>
 __device__ __forceinline__ void t2p_sum(const float* c, const float* t1, const float* t2, float* out)
 {
 #pragma unroll
     for (int r = 0; r < NR; ++r) out[r] = 0.f;
-#pragma unroll (NR == 1 ? P : 4)
-    for (int b1 = P - 1; b1 >= 0; --b1) {
+#pragma unroll (NR == 1 ? B : 4)
+    for (int b1 = B - 1; b1 >= 0; --b1) {
         float inner[NR];
 #pragma unroll
         for (int r = 0; r < NR; ++r) inner[r] = 0.f;
@@ -99,22 +101,22 @@ __device__ __forceinline__ void t2p_sum(const float* c, const float* t1, const f
     }
 }
 
-template <int P, bool VEC, int ROWS>
+template <int P, bool VEC, int ROWS, int SPLIT>
 __global__ void __launch_bounds__(kT2pThreads) fgt_t2p_binned_kernel(int g, double inv_scale, float dcell,
                                                                      const float* C, int n, const double* y,
                                                                      const int* perm, const int* box_start,
                                                                      float* __restrict__ G, int accumulate, int* err)
 {
-    const int lane = threadIdx.x & 31, side = 1 << g, nbox = side * side;
+    const int lane = threadIdx.x & 31, side = 1 << g, nbox = side * side, part = lane % SPLIT;
     after_wait();
-    const int64_t base = ((int64_t)blockIdx.x * (kT2pThreads / 32) + (threadIdx.x >> 5)) * (32 * ROWS);
+    const int64_t base = ((int64_t)blockIdx.x * (kT2pThreads / 32) + (threadIdx.x >> 5)) * (32 * ROWS / SPLIT);
     bin_check(box_start, nbox, n, err);
     if (base >= n) return;
     int tj[ROWS], tb[ROWS];
     float t1[ROWS], t2[ROWS], out[ROWS];
 #pragma unroll
     for (int r = 0; r < ROWS; ++r) {
-        const int64_t pos = base + 32 * r + lane;
+        const int64_t pos = base + 32 * r + lane / SPLIT;
         tj[r] = tb[r] = -1;
         t1[r] = t2[r] = out[r] = 0.f;
         if (pos >= n) continue;
@@ -146,16 +148,27 @@ __global__ void __launch_bounds__(kT2pThreads) fgt_t2p_binned_kernel(int g, doub
             }
         }
     }
+    if constexpr (SPLIT > 1) {
+        constexpr int B = P / SPLIT;
+        if (tb[0] >= 0) {
+            t2p_sum<P, B, 1, VEC>(C + (size_t)tb[0] * P * P + part * B * P, t1, t2, out);
+            for (int k = 0; k < part * B; ++k) out[0] *= t1[0];
+        }
+#pragma unroll
+        for (int o = 1; o < SPLIT; o <<= 1) out[0] += __shfl_xor_sync(0xffffffffu, out[0], o);
+        if (tj[0] >= 0 && part == 0) G[tj[0]] = accumulate ? G[tj[0]] + out[0] : out[0];
+        return;
+    }
     const int b0 = __shfl_sync(0xffffffffu, tb[0], 0);
     bool same = b0 >= 0;
 #pragma unroll
     for (int r = 0; r < ROWS; ++r) same &= tb[r] == b0 || base + 32 * r + lane >= n;
     if (__all_sync(0xffffffffu, same)) {
-        t2p_sum<P, ROWS, VEC>(C + (size_t)b0 * P * P, t1, t2, out);
+        t2p_sum<P, P, ROWS, VEC>(C + (size_t)b0 * P * P, t1, t2, out);
     } else {
 #pragma unroll
         for (int r = 0; r < ROWS; ++r)
-            if (tb[r] >= 0) t2p_sum<P, 1, VEC>(C + (size_t)tb[r] * P * P, t1 + r, t2 + r, out + r);
+            if (tb[r] >= 0) t2p_sum<P, P, 1, VEC>(C + (size_t)tb[r] * P * P, t1 + r, t2 + r, out + r);
     }
 #pragma unroll
     for (int r = 0; r < ROWS; ++r)
@@ -168,10 +181,12 @@ static int t2p_binned_p(int g, double sigma, const float* C, int n, const double
 {
     const double inv_scale = 1.0 / (sqrt(2.0) * sigma);
     const float dcell = (float)(ldexp(1.0, -g) * inv_scale);
-    const bool wide = n >= kT2pWide, vec = ((uintptr_t)C & 15) == 0;
-    const unsigned grid = bin_blocks(n, kT2pThreads * (wide ? 4 : 1), (int64_t)1 << (2 * g), kT2pThreads);
-    auto kern = wide ? (vec ? fgt_t2p_binned_kernel<P, true, 4> : fgt_t2p_binned_kernel<P, false, 4>)
-                     : (vec ? fgt_t2p_binned_kernel<P, true, 1> : fgt_t2p_binned_kernel<P, false, 1>);
+    const bool vec = ((uintptr_t)C & 15) == 0;
+    const int per = n >= kT2pWide ? 4 * kT2pThreads : n >= kT2pSplit ? kT2pThreads : kT2pThreads / 4;  // targets a block
+    const unsigned grid = bin_blocks(n, per, (int64_t)1 << (2 * g), kT2pThreads);
+    auto kern = n >= kT2pWide    ? (vec ? fgt_t2p_binned_kernel<P, true, 4, 1> : fgt_t2p_binned_kernel<P, false, 4, 1>)
+                : n >= kT2pSplit ? (vec ? fgt_t2p_binned_kernel<P, true, 1, 1> : fgt_t2p_binned_kernel<P, false, 1, 1>)
+                                 : (vec ? fgt_t2p_binned_kernel<P, true, 1, 4> : fgt_t2p_binned_kernel<P, false, 1, 4>);
     FMM_CUDA_TRY(launch_after(kern, grid, kT2pThreads, 0, st, g, inv_scale, dcell, C, n, y, perm, box_start, G, acc ? 1 : 0,
                               err));
     return FMM_OK;

@@ -661,9 +661,10 @@ def test_p2h_and_t2p_binned_runs_and_alignments(fmm, orc, p):
 
 
 @pytest.mark.parametrize("p", [4, 8, 12, 16])
-@pytest.mark.parametrize("g,n", [(0, 1), (0, 33), (2, 31), (2, 129), (5, 1000), (5, 2 ** 18 - 1), (5, 2 ** 18), (8, 3000)])
+@pytest.mark.parametrize("g,n", [(0, 1), (0, 33), (2, 31), (2, 129), (5, 1000), (4, 2 ** 14 - 1), (4, 2 ** 14),
+                                 (5, 2 ** 18 - 1), (5, 2 ** 18), (8, 3000)])
 def test_t2p_binned_one_and_four_targets_a_lane(fmm, orc, p, g, n):
-    """T2P on both sides of the line between one and four targets a lane, from coefficients 16-byte aligned and
+    """T2P on both sides of the lines between four lanes a target, one, and four targets a lane, from coefficients 16-byte aligned and
     not, added and written: boxes of one target and of many, the last warp ragged."""
     import torch
 
